@@ -448,7 +448,6 @@ void batched_to_float(tlr_ctx* ctx, std::vector<ConvJob>& jobs);
 void col_sqnorms(tlr_ctx* ctx, const double* X, int rows, int64_t ncols, double* out);
 void scale_cols(tlr_ctx* ctx, int m, int n, const double* dvec, const double* X, int ldx, double* Y,
                 int ldy);
-void tril_mask(tlr_ctx* ctx, int n, double* A, int lda, int unit);
 void set_diag(tlr_ctx* ctx, int n, double* A, int lda, const double* d);
 void axpy_matrix(tlr_ctx* ctx, int m, int n, double alpha, const double* X, int ldx, double* Y, int ldy);
 

@@ -142,6 +142,8 @@ bool trim_fits(int b);
 void trim_tiles(tlr_ctx* ctx, int b, const std::vector<TrimTile>& tiles, double eps, std::vector<int>& rank,
                 std::vector<double*>& Zs, Buf& work);
 void trim_matrix(tlr_ctx* ctx, tlr_mat* M, double eps);
+// Y = op(M) X for a TLR matrix (TLR_OP_A) or factor (TLR_OP_L, _LT, _LLT), original point order (k_apply.cu)
+void tlr_apply(tlr_ctx* ctx, const tlr_mat* M, int op, int nrhs, const double* X, int64_t ldx, double* Y, int64_t ldy);
 // The rules of the factorization options (bs already defaulted), shared by tlr_potrf / tlr_ldlt /
 // tlr_factor_batch, tlr_session_add and tlr_submit.
 bool factor_opts_ok(const tlr_opts& o, int ldl, int64_t N, int b);

@@ -1171,22 +1171,6 @@ void scale_cols(tlr_ctx* ctx, int m, int n, const double* dvec, const double* X,
   TLR_LAUNCH_CHECK(ctx);
 }
 
-// Zero the strict upper triangle (and set a unit diagonal if `unit`).
-__global__ void k_tril_mask(int n, double* A, int lda, int unit) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)n * n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(e % n), c = (int)(e / n);
-    if (r < c) A[r + (size_t)c * lda] = 0.0;
-    else if (r == c && unit) A[r + (size_t)c * lda] = 1.0;
-  }
-}
-void tril_mask(tlr_ctx* ctx, int n, double* A, int lda, int unit) {
-  if (n <= 0) return;
-  TLR_SITE_PRE(ctx);
-  k_tril_mask<<<std::min<unsigned>(cdiv((int64_t)n * n, 256), 4096u), 256, 0, ctx->stream>>>(n, A, lda, unit);
-  TLR_LAUNCH_CHECK(ctx);
-}
-
 __global__ void k_set_diag(int n, double* A, int lda, const double* d) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) A[i + (size_t)i * lda] = d[i];

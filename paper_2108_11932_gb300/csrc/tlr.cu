@@ -1011,87 +1011,6 @@ static SolvePlan* plan_for(tlr_ctx* ctx, tlr_mat* F, int nrhs) {
 
 }  // namespace tlr
 
-// Y = L X or Y = L^T X (KD order, padded); Y must not alias X.
-static void tri_mul(tlr_ctx* ctx, const tlr_mat* F, int trans, int nrhs, const double* X, int64_t ldx, double* Y,
-                    int64_t ldy, Buf& tmp) {
-  const int nb = F->nb, b = F->b;
-  const int unit = F->state == 2;
-  // diagonal blocks: Y_k = L_kk X_k (or L_kk^T X_k) via the triangular tile as a dense GEMM on its lower part
-  double* Lt = tmp.need<double>((size_t)b * b);
-  for (int k = 0; k < nb; ++k) {
-    // build a clean lower-triangular copy (unit diagonal for LDL^T)
-    copy_matrix(ctx, b, b, F->diag + (size_t)k * b * b, b, Lt, b);
-    std::vector<GemmJob<double>> jj;
-    tril_mask(ctx, b, Lt, b, unit);
-    jj.push_back(job<double>(trans ? TN : NN, b, nrhs, Lt, b, X + (size_t)k * b, (int)ldx, b, Y + (size_t)k * b,
-                             (int)ldy, 1.0, 0.0));
-    gemm<double>(ctx, trans ? TN : NN, jj);
-  }
-  Buf t2(ctx);
-  for (int k = 0; k < nb; ++k) {
-    const int64_t Rk = F->vlen[k];
-    if (Rk == 0) continue;
-    double* T = t2.need<double>((size_t)Rk * nrhs);
-    if (!trans) {  // Y_i += U_ik (V_ik^T X_k)
-      std::vector<GemmJob<double>> j1{job<double>(TN, (int)Rk, nrhs, F->Vcol[k], b, X + (size_t)k * b, (int)ldx, b, T,
-                                                  (int)Rk, 1.0, 0.0)};
-      gemm<double>(ctx, TN, j1);
-      std::vector<GemmJob<double>> j2;
-      for (int i = k + 1; i < nb; ++i) {
-        const int r = F->rank[ix(F, i, k)];
-        if (r) j2.push_back(job<double>(NN, b, nrhs, Uptr(F, i, k), b, T + F->voff[ix(F, i, k)], (int)Rk, r,
-                                        Y + (size_t)i * b, (int)ldy, 1.0, 1.0));
-      }
-      gemm<double>(ctx, NN, j2);
-    } else {  // Y_k += V_ik (U_ik^T X_i)
-      std::vector<GemmJob<double>> j1;
-      for (int i = k + 1; i < nb; ++i) {
-        const int r = F->rank[ix(F, i, k)];
-        if (r) j1.push_back(job<double>(TN, r, nrhs, Uptr(F, i, k), b, X + (size_t)i * b, (int)ldx, b,
-                                        T + F->voff[ix(F, i, k)], (int)Rk, 1.0, 0.0));
-      }
-      gemm<double>(ctx, TN, j1);
-      std::vector<GemmJob<double>> j2{job<double>(NN, b, nrhs, F->Vcol[k], b, T, (int)Rk, (int)Rk,
-                                                  Y + (size_t)k * b, (int)ldy, 1.0, 1.0)};
-      gemm<double>(ctx, NN, j2);
-    }
-  }
-}
-
-// Y = A X for the symmetric TLR matrix A (state 0), KD order, padded.
-static void sym_mul(tlr_ctx* ctx, const tlr_mat* M, int nrhs, const double* X, int64_t ldx, double* Y, int64_t ldy) {
-  const int nb = M->nb, b = M->b;
-  std::vector<GemmJob<double>> jd;
-  for (int k = 0; k < nb; ++k)
-    jd.push_back(job<double>(NN, b, nrhs, M->diag + (size_t)k * b * b, b, X + (size_t)k * b, (int)ldx, b,
-                             Y + (size_t)k * b, (int)ldy, 1.0, 0.0));
-  gemm<double>(ctx, NN, jd);
-  Buf t(ctx), t2(ctx);
-  for (int k = 0; k < nb; ++k) {
-    const int64_t Rk = M->vlen[k];
-    if (Rk == 0) continue;
-    double* T = t.need<double>((size_t)Rk * nrhs);
-    double* S = t2.need<double>((size_t)Rk * nrhs);
-    std::vector<GemmJob<double>> j1{job<double>(TN, (int)Rk, nrhs, M->Vcol[k], b, X + (size_t)k * b, (int)ldx, b, T,
-                                                (int)Rk, 1.0, 0.0)};
-    gemm<double>(ctx, TN, j1);
-    std::vector<GemmJob<double>> j2, j3;
-    for (int i = k + 1; i < nb; ++i) {
-      const int r = M->rank[ix(M, i, k)];
-      if (!r) continue;
-      j2.push_back(job<double>(NN, b, nrhs, Uptr(M, i, k), b, T + M->voff[ix(M, i, k)], (int)Rk, r, Y + (size_t)i * b,
-                               (int)ldy, 1.0, 1.0));
-      j3.push_back(job<double>(TN, r, nrhs, Uptr(M, i, k), b, X + (size_t)i * b, (int)ldx, b, S + M->voff[ix(M, i, k)],
-                               (int)Rk, 1.0, 0.0));
-    }
-    gemm<double>(ctx, NN, j2);
-    gemm<double>(ctx, TN, j3);
-    std::vector<GemmJob<double>> j4{job<double>(NN, b, nrhs, M->Vcol[k], b, S, (int)Rk, (int)Rk, Y + (size_t)k * b,
-                                                (int)ldy, 1.0, 1.0)};
-    gemm<double>(ctx, NN, j4);
-  }
-}
-
 // ======================================================================== C ABI
 #define ABI_BEGIN try {
 #define ABI_END                                     \
@@ -1461,22 +1380,7 @@ tlr_status tlr_matvec(tlr_ctx* ctx, const tlr_mat* F, int op, int nrhs, const do
   if (op < 0 || op > 3) return TLR_ERR_ARG;
   if (nrhs == 0) return TLR_OK;
   ABI_BEGIN
-  const int64_t np = (int64_t)F->nb * F->b;
-  Buf bX(ctx), bY(ctx), bT(ctx), bZ(ctx);
-  double* Xp = bX.need<double>((size_t)np * nrhs);
-  double* Yp = bY.need<double>((size_t)np * nrhs);
-  const int64_t* perm = F->dperm;
-  permute_rows(ctx, F->N, nrhs, perm, 1, X, ldx, Xp, np, np);
-  if (op == TLR_OP_A) sym_mul(ctx, F, nrhs, Xp, np, Yp, np);
-  else if (op == TLR_OP_L) tri_mul(ctx, F, 0, nrhs, Xp, np, Yp, np, bT);
-  else if (op == TLR_OP_LT) tri_mul(ctx, F, 1, nrhs, Xp, np, Yp, np, bT);
-  else {
-    double* Zp = bZ.need<double>((size_t)np * nrhs);
-    tri_mul(ctx, F, 1, nrhs, Xp, np, Zp, np, bT);
-    if (F->state == 2) scale_rows(ctx, (int)np, nrhs, F->dvec, 0, Zp, (int)np, Zp, (int)np);
-    tri_mul(ctx, F, 0, nrhs, Zp, np, Yp, np, bT);
-  }
-  permute_rows(ctx, F->N, nrhs, perm, 0, Yp, np, Y, ldy, np);
+  tlr_apply(ctx, F, op, nrhs, X, ldx, Y, ldy);
   TLR_CUDA(cudaStreamSynchronize(ctx->stream));
   return TLR_OK;
   ABI_END

@@ -1,0 +1,83 @@
+"""Products with a whole matrix or factor (tlr_matvec) against the dense matrix of its exported tiles.
+
+Tolerance: every output is a sum of products in some order, so its error is at most n u (|D| + |U| |V|^T) |X|
+with n the number of terms of the two contractions (Higham, Section 3.1); applied twice for L L^T.
+"""
+import numpy as np
+import pytest
+
+import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def T():
+    import paper_2108_11932_gb300 as T
+    T.build()
+    return T
+
+
+def _dense(M, tri):
+    """The matrix of M's tiles in KD order and the same of the absolute factors (tri: lower block triangle,
+    of the diagonal tiles the lower triangle)."""
+    inf, rk = M.info(), M.ranks()
+    b, nb = inf["b"], inf["nb"]
+    D, P = np.zeros((nb * b, nb * b)), np.zeros((nb * b, nb * b))
+    d = np.ones(nb * b)
+    for i in range(nb):
+        s = slice(i * b, (i + 1) * b)
+        A, dv = M.tile(i, i)
+        if dv is not None:
+            A = np.tril(A, -1) + np.eye(b)
+            d[s] = dv
+        D[s, s] = np.tril(A) if tri else A
+        P[s, s] = np.abs(D[s, s])
+        for j in range(i):
+            if not rk[i, j]:
+                continue
+            q = slice(j * b, (j + 1) * b)
+            U, V = M.tile(i, j)
+            D[s, q], P[s, q] = U @ V.T, np.abs(U) @ np.abs(V).T
+            if not tri:
+                D[q, s], P[q, s] = D[s, q].T, P[s, q].T
+    return D, P, d
+
+
+@pytest.mark.parametrize("N,d,b,eps,ldl", [
+    (100, 2, 128, 1e-6, False),    # one tile, ragged
+    (1024, 2, 128, 1e-6, False),   # row blocks shared by clusters
+    (1000, 3, 64, 1e-4, True),     # ragged last tile
+    (700, 2, 75, 1e-6, False),     # odd tile size: 8-byte loads
+    (600, 2, 50, 1e-3, True),      # row blocks of 64 cut short
+    (1500, 1, 48, 1e-2, False),    # 1D: rank-1 and rank-0 tiles
+])
+def test_products_match_the_exported_tiles(T, N, d, b, eps, ldl):
+    import torch
+    ctx = T.Context(0)
+    o = T.default_opts(bs=16, seed=N)
+    A = ctx.compress(inputs.points(N, d, N), b, eps, 0.1, 1e-2 if eps > 1e-5 else 1e-4, o)
+    F = A.copy()
+    (F.ldlt if ldl else F.potrf)(eps, o)
+    DA, PA, _ = _dense(A, False)
+    L, PL, dv = _dense(F, True)
+    npad = DA.shape[0]
+    perm = A.perm()
+    u = 2.0 ** -53
+    rng = np.random.default_rng(N)
+    for nrhs in (1, 2, 3, 5, 7, 8, 9, 17):
+        X = rng.standard_normal((N, nrhs))
+        Xp = np.zeros((npad, nrhs))
+        Xp[:N] = X[perm]
+        n = npad + int(max(A.ranks().sum(), F.ranks().sum()))
+        want = {
+            "A": (A, T.OP_A, DA @ Xp, PA @ np.abs(Xp), 1),
+            "L": (F, T.OP_L, L @ Xp, PL @ np.abs(Xp), 1),
+            "Lt": (F, T.OP_LT, L.T @ Xp, PL.T @ np.abs(Xp), 1),
+            "LLt": (F, T.OP_LLT, L @ (dv[:, None] * (L.T @ Xp)),
+                    PL @ (np.abs(dv)[:, None] * (PL.T @ np.abs(Xp))), 2),
+        }
+        for name, (M, op, Y, B, times) in want.items():
+            g = M.matvec(T.fortran(torch.tensor(X, device="cuda:0")), op).cpu().numpy()[perm]
+            assert np.all(np.abs(g - Y[:N]) <= 2 * times * n * u * B[:N]), (name, nrhs)
+    ctx.close()
