@@ -314,9 +314,9 @@ tlr_status tlr_kernel_matvec(tlr_ctx* ctx, const double* points_host, int64_t N,
  * (a memory manager owns the whole device heap, cudaMalloc's implicit
  * synchronization is not acceptable, or no tlr_ctx exists).  It computes the
  * same Y = A X; instead of library-allocated device memory it stages the
- * points in a fixed device array compiled into the library (3 MiB, held by
- * every GPU that loads the library until the process exits), so it needs no
- * context and calls no allocator.
+ * points and their grid in a fixed device array compiled into the library
+ * (6 MiB, held by every GPU that loads the library until the process exits),
+ * so it needs no context and calls no allocator.
  *   cuda_stream: cudaStream_t of the CURRENT device (NULL: legacy default
  *     stream); the call is enqueued on it and returns without synchronizing.
  *   points_host: host, row-major N x d, original order; copied during the call

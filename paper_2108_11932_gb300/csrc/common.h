@@ -230,10 +230,10 @@ void omega(tlr_ctx* ctx, uint64_t seed, uint32_t stream, uint32_t k, uint32_t t,
 // Points on a 64-bit grid for the kernel tiles: X (device, N x d) = round(x 2^q) - round(o 2^q).
 struct GridInfo {
   int q;
-  int pad;
+  int ok;  // the grid resolves exp(-|x - y| / ell) at least as well as FP64 coordinate differences
   double o[3];
 };
-void grid_points(tlr_ctx* ctx, const double* pts, int64_t N, int d, GridInfo* gi /*device*/, long long* X);
+void grid_points(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell, GridInfo* gi /*device*/, long long* X);
 void gen_tiles(tlr_ctx* ctx, const long long* X, const GridInfo* gi, int64_t N, int d, double ell, double nugget,
                int b, const int* tile_ij /*device, 2 per tile*/, int ntiles, double* out,
                unsigned long long* tmax = nullptr /*device, per tile, zeroed*/);
@@ -274,8 +274,9 @@ void add_diag(tlr_ctx* ctx, int n, double* A, int lda, double s);
 void add_rowsum_abs(tlr_ctx* ctx, int n, const double* E, int lde, double* A, int lda);
 void logdet_reduce(tlr_ctx* ctx, int n, const double* diag_tiles, int b, int nb, const double* dvec,
                    double* out2 /*device: [sum log|.|, count negative]*/);
+// gi, grid: device workspace (N d) for the points' grid
 void kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell, double nugget,
-                   int nrhs, const double* X, int64_t ldx, double* Y, int64_t ldy);
+                   int nrhs, const double* X, int64_t ldx, double* Y, int64_t ldy, GridInfo* gi, long long* grid);
 void permute_rows(tlr_ctx* ctx, int64_t n_out, int nrhs, const int64_t* idx, int gather,
                   const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t n_pad);
 void copy_matrix(tlr_ctx* ctx, int m, int n, const double* X, int ldx, double* Y, int ldy);

@@ -1,8 +1,12 @@
 // Small and medium kernels of the TLR factorization (everything except the batched GEMM).
 #include <math.h>
 
+#include <cooperative_groups.h>
+
 #include "common.h"
 #include "cholqr.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace tlr {
 
@@ -177,38 +181,55 @@ __device__ __forceinline__ unsigned long long ord_key(double x) {
 __device__ __forceinline__ double ord_val(unsigned long long k) {
   return __longlong_as_double((long long)((k >> 63) ? (k & ~(1ull << 63)) : ~k));
 }
-__global__ void __launch_bounds__(256) k_grid_range(const double* __restrict__ pts, int64_t N, int d,
-                                                    GridInfo* __restrict__ gi) {
-  __shared__ unsigned long long smin[3][256], smax[3][256];
-  unsigned long long mn[3] = {~0ull, ~0ull, ~0ull}, mx[3] = {0, 0, 0};
-  for (int64_t p = threadIdx.x; p < N; p += blockDim.x)
-    for (int k = 0; k < d; ++k) {
+// One block of 1024 threads (the points are read once, by strided loads that are all independent).
+// gi->ok: the grid resolves the kernel at least as well as FP64 differences of the coordinates do, for
+// callers whose points need not meet that (k_kernel_matvec): every coordinate is finite and the largest
+// extent is at most 64 ell.  The grid spacing is 2^-q <= range 2^-61, so a distance is off by at most
+// sqrt(d) 2^-60 range, z = distance / ell by 2^-54 sqrt(d), half a unit roundoff of the entry.
+constexpr int GR_T = 1024;
+__global__ void __launch_bounds__(GR_T) k_grid_range(const double* __restrict__ pts, int64_t N, int d, double inv_ell,
+                                                     GridInfo* __restrict__ gi) {
+  __shared__ unsigned long long smin[3][GR_T / 32], smax[3][GR_T / 32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int k = 0; k < d; ++k) {
+    unsigned long long mn = ~0ull, mx = 0;
+#pragma unroll 4
+    for (int64_t p = threadIdx.x; p < N; p += GR_T) {
       const unsigned long long key = ord_key(pts[p * d + k]);
-      mn[k] = key < mn[k] ? key : mn[k];
-      mx[k] = key > mx[k] ? key : mx[k];
+      mn = key < mn ? key : mn;
+      mx = key > mx ? key : mx;
     }
-  for (int k = 0; k < 3; ++k) { smin[k][threadIdx.x] = mn[k]; smax[k][threadIdx.x] = mx[k]; }
-  __syncthreads();
-  for (int w = 128; w; w >>= 1) {
-    if ((int)threadIdx.x < w)
-      for (int k = 0; k < 3; ++k) {
-        const unsigned long long a = smin[k][threadIdx.x + w], c = smax[k][threadIdx.x + w];
-        if (a < smin[k][threadIdx.x]) smin[k][threadIdx.x] = a;
-        if (c > smax[k][threadIdx.x]) smax[k][threadIdx.x] = c;
-      }
-    __syncthreads();
+    for (int o = 16; o; o >>= 1) {
+      const unsigned long long a = __shfl_xor_sync(0xffffffffu, mn, o), c = __shfl_xor_sync(0xffffffffu, mx, o);
+      mn = a < mn ? a : mn;
+      mx = c > mx ? c : mx;
+    }
+    if (lane == 0) {
+      smin[k][warp] = mn;
+      smax[k][warp] = mx;
+    }
   }
+  __syncthreads();
   if (threadIdx.x == 0) {
     double R = 0.0, A = 0.0;
+    bool ok = true;
     for (int k = 0; k < d; ++k) {
-      const double lo = ord_val(smin[0 + k][0]), hi = ord_val(smax[k][0]);
+      unsigned long long mn = ~0ull, mx = 0;
+      for (int w = 0; w < GR_T / 32; ++w) {
+        mn = smin[k][w] < mn ? smin[k][w] : mn;
+        mx = smax[k][w] > mx ? smax[k][w] : mx;
+      }
+      const double lo = ord_val(mn), hi = ord_val(mx);
       gi->o[k] = lo;
+      ok &= isfinite(lo) && isfinite(hi);
       R = fmax(R, hi - lo);
       A = fmax(A, fmax(fabs(lo), fabs(hi)));
     }
     int q = R > 0.0 ? 61 - ilogb(R) : 0;
     if (A > 0.0) q = min(q, 125 - ilogb(A));
     gi->q = q;
+    // (an offset of more than 2^62 ranges would coarsen the grid: A <= 2^60 R keeps q at 61 - ilogb(R))
+    gi->ok = ok && isfinite(inv_ell) && R * inv_ell <= 64.0 && A <= 0x1p60 * R;
   }
 }
 __global__ void k_grid_points(const double* __restrict__ pts, int64_t n, int d, const GridInfo* __restrict__ gi,
@@ -220,10 +241,10 @@ __global__ void k_grid_points(const double* __restrict__ pts, int64_t n, int d, 
   X[e] = (long long)(grid_round(pts[e], q) - grid_round(gi->o[k], q));
 }
 
-void grid_points(tlr_ctx* ctx, const double* pts, int64_t N, int d, GridInfo* gi, long long* X) {
+void grid_points(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell, GridInfo* gi, long long* X) {
   if (N <= 0) return;
   TLR_SITE_PRE(ctx);
-  k_grid_range<<<1, 256, 0, ctx->stream>>>(pts, N, d, gi);
+  k_grid_range<<<1, GR_T, 0, ctx->stream>>>(pts, N, d, 1.0 / ell, gi);
   TLR_LAUNCH_CHECK(ctx);
   TLR_SITE_PRE(ctx);
   k_grid_points<<<cdiv(N * d, 256), 256, 0, ctx->stream>>>(pts, N * d, d, gi, X);
@@ -291,14 +312,21 @@ __global__ void __launch_bounds__(GT_THREADS) k_gen_tiles(const long long* __res
   }
 }
 
+// 1/ell = Cm 2^(ec - 63), Cm in [2^63, 2^64)
+static void fx_scale(double ell, uint64_t& Cm, int& ec) {
+  ec = 0;
+  const double mc = frexp(1.0 / ell, &ec);  // mc in [1/2, 1)
+  Cm = (uint64_t)ldexp(mc, 64);
+  ec -= 1;
+}
+
 void gen_tiles(tlr_ctx* ctx, const long long* X, const GridInfo* gi, int64_t N, int d, double ell, double nugget,
                int b, const int* tile_ij, int ntiles, double* out, unsigned long long* tmax) {
   if (ntiles <= 0) return;
   TLR_REQUIRE(d >= 1 && d <= 3, TLR_ERR_ARG, "points of dimension 1 to 3");
-  int ec = 0;
-  const double mc = frexp(1.0 / ell, &ec);  // 1/ell = mc 2^ec, mc in [1/2, 1)
-  const uint64_t Cm = (uint64_t)ldexp(mc, 64);
-  ec -= 1;
+  int ec;
+  uint64_t Cm;
+  fx_scale(ell, Cm, ec);
   dim3 grid(cdiv(b, GT_COLS), (unsigned)ntiles);
   TLR_SITE_PRE(ctx);
   if (d == 1)
@@ -779,50 +807,159 @@ void logdet_reduce(tlr_ctx* ctx, int n, const double* diag_tiles, int b, int nb,
   TLR_LAUNCH_CHECK(ctx);
 }
 
-// Exact kernel product Y = A X, A_ij = exp(-|x_i - x_j| / ell) + nugget delta_ij,
-// one thread per row, points of the column block staged in shared memory.
-constexpr int KMV_T = 128, KMV_R = 8;
-__global__ void __launch_bounds__(KMV_T) k_kernel_matvec(const double* __restrict__ pts, int64_t N, int d,
-                                                        double inv_ell, double nugget, int nr,
+// Exact kernel product Y = A X, A_ij = exp(-|x_i - x_j| / ell) + nugget delta_ij.
+//
+// The entries are what costs: in FP64 about 45 instructions at 2 lanes per clock and SM, on the integer
+// pipe (fx::entry, the entries of the compressed tiles) about 400 at 128.  So the entries are formed on
+// the integer pipe from the points' 64-bit grid, and the FP64 unit only multiplies them into up to eight
+// right-hand sides.  Points that the grid does not resolve as well as FP64 differences (GridInfo::ok,
+// decided on the device, so that a captured call follows the points of its replay) take FP64 entries.
+// A lane owns a row and the CTA's eight warps share the columns (each stages 32 of them at a time for
+// itself, no CTA barrier in the loop), a cluster of S CTAs splits them further so that small N fills the
+// GPU; partial sums are added in warp and rank order.
+// Measured: N = 32768, 3D, 4 right-hand sides 81.3 -> 16.3 ms (the FP64 products of 4 columns are 6.9 ms of it).
+constexpr int KMV_W = 8, KMV_T = 32 * KMV_W, KMV_R = 8;
+template <int D, int NR>
+__global__ void __launch_bounds__(KMV_T) k_kernel_matvec(const double* __restrict__ pts,
+                                                        const long long* __restrict__ grid,
+                                                        const GridInfo* __restrict__ gi, int64_t N, uint64_t Cm, int ec,
+                                                        double inv_ell, double nugget, int nr, int S,
                                                         const double* __restrict__ X, int64_t ldx,
                                                         double* __restrict__ Y, int64_t ldy) {
-  __shared__ double P[KMV_T][3];
-  __shared__ double Xs[KMV_T][KMV_R];
-  const int64_t i = blockIdx.x * (int64_t)KMV_T + threadIdx.x;
-  double xi[3] = {0, 0, 0};
-  if (i < N)
-    for (int q = 0; q < d; ++q) xi[q] = pts[i * d + q];
-  double acc[KMV_R] = {0, 0, 0, 0};
-  for (int64_t j0 = 0; j0 < N; j0 += KMV_T) {
-    const int64_t j = j0 + threadIdx.x;
-    __syncthreads();
-    if (j < N) {
-      for (int q = 0; q < d; ++q) P[threadIdx.x][q] = pts[j * d + q];
-      for (int c = 0; c < nr; ++c) Xs[threadIdx.x][c] = X[j + c * ldx];
-    }
-    __syncthreads();
-    const int cnt = (N - j0 < KMV_T) ? (int)(N - j0) : KMV_T;
-    for (int jj = 0; jj < cnt; ++jj) {
-      double s = 0.0;
-      for (int q = 0; q < d; ++q) {
-        const double df = xi[q] - P[jj][q];
-        s = fma(df, df, s);
+  __shared__ uint64_t tab[64];
+  __shared__ long long sp[KMV_W][32][D];  // grid points, or the bits of the coordinates
+  __shared__ __align__(16) double sx[KMV_W][32][NR];
+  __shared__ double part[32 * NR];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = (int)blockIdx.x % S;
+  const int64_t row = (int64_t)((int)blockIdx.x / S) * 32 + lane, r = min(row, N - 1);
+  if (threadIdx.x < 64) tab[threadIdx.x] = fx::TAB[threadIdx.x];
+  __syncthreads();
+  const bool fixed = gi->ok;
+  const int ezb = ec + 63 - gi->q;
+  const long long* src = fixed ? grid : reinterpret_cast<const long long*>(pts);
+  long long xr[D];
+#pragma unroll
+  for (int k = 0; k < D; ++k) xr[k] = src[r * D + k];
+  double acc[NR];
+#pragma unroll
+  for (int n = 0; n < NR; ++n) acc[n] = 0.0;
+  const int64_t nblk = (N + 31) / 32, b0 = nblk * rank / S, b1 = nblk * (rank + 1) / S;
+  for (int64_t blk = b0 + warp; blk < b1; blk += KMV_W) {
+    const int64_t j = blk * 32 + lane;
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < D; ++k) sp[warp][lane][k] = j < N ? src[j * D + k] : 0;
+#pragma unroll
+    for (int n = 0; n < NR; ++n) sx[warp][lane][n] = j < N && n < nr ? X[j + n * ldx] : 0.0;
+    __syncwarp();
+    const int cnt = (int)min((int64_t)32, N - blk * 32);
+    if (fixed) {
+      for (int c = 0; c < cnt; ++c) {
+        uint64_t hi = 0, lo = 0;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+          const long long df = xr[k] - sp[warp][c][k];
+          const uint64_t a = (uint64_t)(df < 0 ? -df : df);
+          const uint64_t l = a * a;
+          lo += l;
+          hi += __umul64hi(a, a) + (lo < l ? 1ull : 0ull);
+        }
+        const double a = fx::entry(hi, lo, ezb, Cm, tab);
+#pragma unroll
+        for (int n = 0; n < NR; ++n) acc[n] = fma(a, sx[warp][c][n], acc[n]);
       }
-      const double a = exp(-sqrt(s) * inv_ell);
-      for (int c = 0; c < nr; ++c) acc[c] = fma(a, Xs[jj][c], acc[c]);
+    } else {
+      for (int c = 0; c < cnt; ++c) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+          const double df = __longlong_as_double(xr[k]) - __longlong_as_double(sp[warp][c][k]);
+          s = fma(df, df, s);
+        }
+        const double a = exp(-sqrt(s) * inv_ell);
+#pragma unroll
+        for (int n = 0; n < NR; ++n) acc[n] = fma(a, sx[warp][c][n], acc[n]);
+      }
     }
   }
-  if (i < N)
-    for (int c = 0; c < nr; ++c) Y[i + c * ldy] = acc[c] + nugget * X[i + c * ldx];
+  __syncwarp();
+#pragma unroll
+  for (int n = 0; n < NR; ++n) sx[warp][lane][n] = acc[n];
+  __syncthreads();
+  auto store = [&](int o, double v) {
+    const int64_t g = (int64_t)((int)blockIdx.x / S) * 32 + o / NR;
+    const int n = o % NR;
+    if (g < N && n < nr) Y[g + n * ldy] = v + nugget * X[g + n * ldx];
+  };
+  for (int o = threadIdx.x; o < 32 * NR; o += KMV_T) {
+    double v = 0.0;
+#pragma unroll
+    for (int w = 0; w < KMV_W; ++w) v += sx[w][o / NR][o % NR];
+    if (S == 1) store(o, v);
+    else part[o] = v;
+  }
+  if (S == 1) return;
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  for (int o = rank * KMV_T + threadIdx.x; o < 32 * NR; o += S * KMV_T) {
+    double v = 0.0;
+    for (int q = 0; q < S; ++q) v += cl.map_shared_rank(part, q)[o];
+    store(o, v);
+  }
+  cl.sync();  // no CTA leaves while its part is still read
 }
-void kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell, double nugget,
-                   int nrhs, const double* X, int64_t ldx, double* Y, int64_t ldy) {
-  for (int c0 = 0; c0 < nrhs; c0 += KMV_R) {
-    const int nr = std::min(KMV_R, nrhs - c0);
-    TLR_SITE_PRE(ctx);
-    k_kernel_matvec<<<cdiv(N, KMV_T), KMV_T, 0, ctx->stream>>>(pts, N, d, 1.0 / ell, nugget, nr,
-                                                              X + c0 * ldx, ldx, Y + c0 * ldy, ldy);
-    TLR_LAUNCH_CHECK(ctx);
+
+template <int D, int NR>
+static void kernel_matvec_launch(tlr_ctx* ctx, const double* pts, const long long* grid, const GridInfo* gi, int64_t N,
+                                 uint64_t Cm, int ec, double ell, double nugget, int nr, const double* X, int64_t ldx,
+                                 double* Y, int64_t ldy) {
+  const int64_t rbs = (N + 31) / 32;
+  // CTAs sharing 32 rows: about 32 per SM in all (a CTA's work is then small against the whole, so the
+  // last wave is short), while each keeps a 32-column block for every warp
+  int S = 1;
+  while (S < 8 && rbs * S < 32LL * 152 && rbs / (2 * S) >= KMV_W) S *= 2;
+  cudaLaunchConfig_t cf{};
+  cf.gridDim = dim3((unsigned)(rbs * S));
+  cf.blockDim = dim3(KMV_T);
+  cf.stream = ctx->stream;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)S;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cf.attrs = &at;
+  cf.numAttrs = 1;
+  TLR_SITE_PRE(ctx);
+  TLR_CUDA(cudaLaunchKernelEx(&cf, k_kernel_matvec<D, NR>, pts, grid, gi, N, Cm, ec, 1.0 / ell, nugget, nr, S, X, ldx, Y,
+                              ldy));
+  TLR_LAUNCH_CHECK(ctx);
+}
+
+template <int D>
+static void kernel_matvec_d(tlr_ctx* ctx, const double* pts, const long long* grid, const GridInfo* gi, int64_t N,
+                            uint64_t Cm, int ec, double ell, double nugget, int nr, const double* X, int64_t ldx,
+                            double* Y, int64_t ldy) {
+  if (nr == 1) kernel_matvec_launch<D, 1>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy);
+  else if (nr == 2) kernel_matvec_launch<D, 2>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy);
+  else if (nr <= 4) kernel_matvec_launch<D, 4>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy);
+  else kernel_matvec_launch<D, KMV_R>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy);
+}
+
+void kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell, double nugget, int nrhs,
+                   const double* X, int64_t ldx, double* Y, int64_t ldy, GridInfo* gi, long long* grid) {
+  if (nrhs <= 0) return;
+  grid_points(ctx, pts, N, d, ell, gi, grid);
+  int ec;
+  uint64_t Cm;
+  fx_scale(ell, Cm, ec);
+  const int ng = (nrhs + KMV_R - 1) / KMV_R;  // right-hand sides in equal groups
+  for (int g = 0; g < ng; ++g) {
+    const int c0 = (int)((int64_t)nrhs * g / ng), nr = (int)((int64_t)nrhs * (g + 1) / ng) - c0;
+    const double* Xg = X + c0 * ldx;
+    double* Yg = Y + c0 * ldy;
+    if (d == 1) kernel_matvec_d<1>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy);
+    else if (d == 2) kernel_matvec_d<2>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy);
+    else kernel_matvec_d<3>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy);
   }
 }
 

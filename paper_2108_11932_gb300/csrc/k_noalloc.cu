@@ -5,13 +5,15 @@
 // a library allocate device memory: code that runs under a memory manager
 // which owns the whole device heap, processes that must not trigger
 // cudaMalloc's implicit synchronization, or callers without a tlr_ctx.  This
-// variant stages the points in a fixed, file-scope device array instead, so a
-// call allocates nothing and needs no context; the caller still owns X and Y.
+// variant stages the points (and their 64-bit grid, which the kernel reads) in a
+// fixed, file-scope device array instead, so a call allocates nothing and needs no
+// context; the caller still owns X and Y.
 //
 // Cost of that choice: every GPU that loads the library keeps the array
-// (kMaxPointDoubles doubles, 3 MiB) until the process exits, calls share it
-// (the last call's points stay in it), and calls whose work overlaps on the
-// GPU (different streams, or several host threads) race on it.
+// (points and grid, kMaxPointDoubles 8-byte words each, 6 MiB in all) until the
+// process exits, calls share it (the last call's points stay in it), and calls whose
+// work overlaps on the GPU (different streams, or several host threads) race on it.
+#include <cstddef>
 #include <mutex>
 
 #include "common.h"
@@ -20,24 +22,29 @@ namespace {
 
 // N * d doubles at most: 131072 points in three dimensions.
 constexpr int64_t kMaxPointDoubles = 3 * 131072;
-static __device__ __align__(256) double g_points[kMaxPointDoubles];
+struct Stage {
+  double points[kMaxPointDoubles];
+  long long grid[kMaxPointDoubles];
+  tlr::GridInfo info;
+};
+static __device__ __align__(256) Stage g_stage;
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mutex;
-double* g_points_addr[kMaxDevices] = {nullptr};
+Stage* g_stage_addr[kMaxDevices] = {nullptr};
 
-// Device address of g_points on the current device.  In host code the name
-// g_points is only a host-side stand-in for the symbol, so the address must be
+// Device address of g_stage on the current device.  In host code the name
+// g_stage is only a host-side stand-in for the symbol, so the address must be
 // asked for once per device, with that device current.
-cudaError_t points_address(int dev, double** out) {
+cudaError_t stage_address(int dev, Stage** out) {
   std::lock_guard<std::mutex> lock(g_mutex);
-  if (!g_points_addr[dev]) {
+  if (!g_stage_addr[dev]) {
     void* p = nullptr;
-    const cudaError_t e = cudaGetSymbolAddress(&p, g_points);
+    const cudaError_t e = cudaGetSymbolAddress(&p, g_stage);
     if (e != cudaSuccess) return e;
-    g_points_addr[dev] = static_cast<double*>(p);
+    g_stage_addr[dev] = static_cast<Stage*>(p);
   }
-  *out = g_points_addr[dev];
+  *out = g_stage_addr[dev];
   return cudaSuccess;
 }
 
@@ -55,11 +62,14 @@ extern "C" tlr_status tlr_kernel_matvec_noalloc(void* cuda_stream, const double*
     return TLR_ERR_CUDA;
   }
   if (dev < 0 || dev >= kMaxDevices) return TLR_ERR_LIMIT;
-  double* pts = nullptr;
-  if (points_address(dev, &pts) != cudaSuccess) {
+  Stage* st = nullptr;
+  if (stage_address(dev, &st) != cudaSuccess) {
     cudaGetLastError();
     return TLR_ERR_CUDA;
   }
+  double* pts = reinterpret_cast<double*>(st);  // device addresses: st is not dereferenced here
+  long long* grid = reinterpret_cast<long long*>(reinterpret_cast<char*>(st) + offsetof(Stage, grid));
+  tlr::GridInfo* info = reinterpret_cast<tlr::GridInfo*>(reinterpret_cast<char*>(st) + offsetof(Stage, info));
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
   if (cudaMemcpyAsync(pts, points_host, sizeof(double) * N * d, cudaMemcpyHostToDevice, stream) != cudaSuccess) {
     cudaGetLastError();
@@ -70,7 +80,8 @@ extern "C" tlr_status tlr_kernel_matvec_noalloc(void* cuda_stream, const double*
   launch_ctx.device = dev;
   launch_ctx.stream = stream;
   try {
-    tlr::kernel_matvec(&launch_ctx, pts, N, d, kern->ell, kern->nugget, nrhs, X, ldx, Y, ldy);
+    tlr::kernel_matvec(&launch_ctx, pts, N, d, kern->ell, kern->nugget, nrhs, X, ldx, Y, ldy,
+                       info, grid);
   } catch (const tlr::Error& e) {
     cudaGetLastError();  // a failed launch leaves its error pending: do not hand it to the caller's next call
     return e.status;

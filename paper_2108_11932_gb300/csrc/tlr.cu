@@ -723,7 +723,7 @@ static void compress_ordered_impl(tlr_ctx* ctx, const double* pts_dev, const int
   Buf bGx(ctx), bGi(ctx);
   long long* gx = bGx.need<long long>((size_t)N * d);
   GridInfo* ginfo = reinterpret_cast<GridInfo*>(bGi.need<double>(sizeof(GridInfo) / sizeof(double) + 1));
-  grid_points(ctx, M->pts, N, d, ginfo, gx);
+  grid_points(ctx, M->pts, N, d, kern->ell, ginfo, gx);
   {
     std::vector<int> ij;
     for (int k = 0; k < nb; ++k) { ij.push_back(k); ij.push_back(k); }
@@ -1391,9 +1391,14 @@ tlr_status tlr_kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, 
   if (!ctx || !kernel_product_args_ok(pts, kern, X, Y, N, d, nrhs, ldx, ldy)) return TLR_ERR_ARG;
   ABI_BEGIN
   Buf bp(ctx);
-  double* dp = bp.need<double>((size_t)N * d);
+  // the points, their grid and its scale
+  constexpr size_t GI = sizeof(GridInfo) / sizeof(double);
+  static_assert(sizeof(GridInfo) % sizeof(double) == 0 && sizeof(long long) == sizeof(double), "workspace layout");
+  double* dp = bp.need<double>((size_t)2 * N * d + GI);
+  long long* grid = reinterpret_cast<long long*>(dp + (size_t)N * d);
+  GridInfo* gi = reinterpret_cast<GridInfo*>(dp + (size_t)2 * N * d);
   TLR_CUDA(cudaMemcpyAsync(dp, pts, sizeof(double) * N * d, cudaMemcpyHostToDevice, ctx->stream));
-  kernel_matvec(ctx, dp, N, d, kern->ell, kern->nugget, nrhs, X, ldx, Y, ldy);
+  kernel_matvec(ctx, dp, N, d, kern->ell, kern->nugget, nrhs, X, ldx, Y, ldy, gi, grid);
   TLR_CUDA(cudaStreamSynchronize(ctx->stream));
   return TLR_OK;
   ABI_END

@@ -81,3 +81,39 @@ def test_products_match_the_exported_tiles(T, N, d, b, eps, ldl):
             g = M.matvec(T.fortran(torch.tensor(X, device="cuda:0")), op).cpu().numpy()[perm]
             assert np.all(np.abs(g - Y[:N]) <= 2 * times * n * u * B[:N]), (name, nrhs)
     ctx.close()
+
+
+@pytest.mark.parametrize("N,d,ell,scale,nrhs", [
+    (1, 2, 0.1, 1.0, 1),
+    (31, 1, 0.1, 1.0, 2),         # less than a warp's columns
+    (33, 3, 0.2, 1.0, 3),
+    (513, 2, 0.1, 1.0, 9),        # two groups of right-hand sides, a cluster of two
+    (5000, 3, 0.2, 1.0, 8),       # a full cluster
+    (700, 2, 0.01, 1.0, 5),       # extent above 64 ell: FP64 entries
+    (700, 3, 30.0, 250.0, 4),     # off the unit box, on the grid
+])
+def test_kernel_product_matches_dense(T, N, d, ell, scale, nrhs):
+    """Entries within 4 2^-52 (1 + z) of exp(-z) on either side, sums of N terms: the two sides differ by at most
+    2 (N + 4 (1 + z) + 4) 2^-52 of the sum of |a_ij x_j|."""
+    import torch
+    ctx = T.Context(0)
+    x = inputs.points(N, d, N) * scale - 0.3 * scale
+    if N > 100:
+        x[7] = x[60]  # coincident points
+    X = np.random.default_rng(N).standard_normal((N, nrhs))
+    g = ctx.kernel_matvec(x, ell, 1e-3, T.fortran(torch.tensor(X, device="cuda:0"))).cpu().numpy()
+    z = np.sqrt(((x[:, None, :] - x[None, :, :]) ** 2).sum(-1)) / ell
+    A = np.exp(-z) + 1e-3 * np.eye(N)
+    B = (A * 2 * (N + 4 * (1 + z) + 4) * 2.0 ** -52) @ np.abs(X)
+    assert np.all(np.abs(g - A @ X) <= B)
+    ctx.close()
+
+
+def test_kernel_product_of_non_finite_points_is_nan(T):
+    import torch
+    ctx = T.Context(0)
+    x = inputs.points(100, 2, 3)
+    x[41, 1] = np.nan
+    g = ctx.kernel_matvec(x, 0.1, 1e-3, T.fortran(torch.ones((100, 2), dtype=torch.float64, device="cuda:0")))
+    assert bool(torch.isnan(g).all())  # every row sums the entry with point 41
+    ctx.close()
