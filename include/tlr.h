@@ -259,21 +259,20 @@ tlr_status tlr_poll(tlr_ctx* ctx, uint64_t ticket, tlr_result* res, double* x, i
 /* Solve (L L^T) X = B or (L D L^T) X = B with the TLR triangular solve of
  * Algorithm 7 (forward) and its transpose (backward).  B: device, N x nrhs,
  * leading dimension ldb >= N, original point order; overwritten with X.
- * The factor keeps a solve plan per group width (right-hand sides are taken in
- * groups of at most 32; up to 4 widths are kept): two N x width work arrays and
- * the job tables, allocated on the first solve of that width and freed with the
- * factor.  The first solve of a width runs the plan's launches directly; the
- * next captures them once as a CUDA graph, which later solves replay (same
- * kernels, bitwise the same results).  Solves with one factor must not run
- * concurrently (they share the plan's work arrays). */
+ * The whole solve is one persistent kernel (a cooperative launch of one CTA per
+ * SM) per group of at most 32 right-hand sides, enqueued on the context's stream.
+ * The factor keeps its step list and the work arrays of the widest solve so far
+ * (allocated on the first solve, freed with the factor).  Solves with one factor
+ * must not run concurrently (they share the work arrays).  Every device wait is
+ * bounded: should one run out, the result is NaN and the context's next solve
+ * returns TLR_ERR_TIMEOUT. */
 tlr_status tlr_solve(tlr_ctx* ctx, const tlr_mat* F, int nrhs, double* B, int64_t ldb);
 
 /* Preconditioned conjugate gradients (Section 6: a low-accuracy TLR factor of
  * A + eps I as the CG preconditioner, run until ||A x - b|| / ||b|| <= tol).
  * A: a compressed matrix (state "A", the operator, applied with tlr_matvec);
- * F: a factor of the same N (the preconditioner, applied with tlr_solve, so its
- * solves replay a captured graph after the first).  B: device, N x nrhs,
- * leading dimension ldb >= N, original point order (read only); X: device,
+ * F: a factor of the same N (the preconditioner, applied with tlr_solve).
+ * B: device, N x nrhs, leading dimension ldb >= N, original point order (read only); X: device,
  * N x nrhs, ldx >= N, receives the solutions (started from 0).  Each column
  * runs its own iteration (textbook PCG, Saad Algorithm 9.1) and stops when its
  * updated residual is at most tol ||b|| or after maxit iterations; iters[c]

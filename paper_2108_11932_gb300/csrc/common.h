@@ -91,7 +91,6 @@ struct tlr_ctx {
   cudaStream_t main = nullptr;    // caller's stream
   cudaStream_t side = nullptr;    // library stream for work overlapped with the main stream
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  cudaStream_t capture = nullptr;  // library stream on which solve graphs are captured
   tlr_alloc_fn alloc = nullptr;
   tlr_free_fn free_fn = nullptr;
   void* user = nullptr;
@@ -112,6 +111,8 @@ struct tlr_ctx {
   size_t split_ctr_cap[2] = {0, 0};
   // grid-barrier words of the fused orthogonalization kernel: {arrivals, generation} per stream
   unsigned* orth_bar = nullptr;
+  // host-visible word that a solve's grid barrier sets when its bounded wait runs out
+  int* wait_out = nullptr;
   // Small host-pinned status buffer for per-round device->host reads.
   void* hstatus = nullptr;
   size_t hstatus_cap = 0;
@@ -174,8 +175,7 @@ struct tlr_mat {
   double flops_exec = 0, flops_model = 0, ara_rounds = 0, seconds = 0;
   double tiles_fp32 = 0, tiles_fp64 = 0;  // tile-rounds sampled in each precision (mixed mode)
   double flops_fp32 = 0;                  // FP32 flops of the mixed-precision chains
-  // solve plans of a factor (buffers, job tables, captured graph), one per nrhs, most recent last
-  std::vector<tlr::SolvePlan*> plans;
+  tlr::SolvePlan* plan = nullptr;  // a factor's solve tables and work vectors (k_solve.cu)
 };
 
 namespace tlr {
@@ -268,8 +268,6 @@ void trsm_left_block(tlr_ctx* ctx, int nbk, const double* L, int lda, int unit, 
                      int ldx);
 void trsm_left_t_block(tlr_ctx* ctx, int nbk, const double* L, int lda, int unit, int nrhs,
                        double* X, int ldx);
-void scale_rows(tlr_ctx* ctx, int m, int n, const double* dvec, int inv, const double* X, int ldx,
-                double* Y, int ldy);
 void add_diag(tlr_ctx* ctx, int n, double* A, int lda, double s);
 void add_rowsum_abs(tlr_ctx* ctx, int n, const double* E, int lde, double* A, int lda);
 void logdet_reduce(tlr_ctx* ctx, int n, const double* diag_tiles, int b, int nb, const double* dvec,
@@ -277,8 +275,6 @@ void logdet_reduce(tlr_ctx* ctx, int n, const double* diag_tiles, int b, int nb,
 // gi, grid: device workspace (N d) for the points' grid
 void kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell, double nugget,
                    int nrhs, const double* X, int64_t ldx, double* Y, int64_t ldy, GridInfo* gi, long long* grid);
-void permute_rows(tlr_ctx* ctx, int64_t n_out, int nrhs, const int64_t* idx, int gather,
-                  const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t n_pad);
 void copy_matrix(tlr_ctx* ctx, int m, int n, const double* X, int ldx, double* Y, int ldy);
 void to_float(tlr_ctx* ctx, int64_t n, const double* x, float* y);
 void to_double(tlr_ctx* ctx, int64_t n, const float* x, double* y);
@@ -416,22 +412,6 @@ struct CopyJob {
   int64_t n;
 };
 void batched_copy(tlr_ctx* ctx, std::vector<CopyJob>& jobs);
-// Skinny products of the triangular solves (k_solve.cu): C = alpha op(A) B + beta C with nrhs
-// columns, op(A) = A (tn = 0, A M x K) or A^T (tn = 1, A K x M), all column-major; lower: A is a
-// lower-triangular block (its zero half is skipped).  Job tables are device-resident.
-struct SkJob {
-  const double* A;
-  const double* B;
-  double* C;
-  int lda, ldb, ldc, M, K, lower;
-  double alpha, beta;
-};
-// work items of a launch: one CTA each (job, first row, log2 of the k-slots of an NN product)
-struct SkItem {
-  int job, m0, cfg;
-};
-void sk_items(int tn, const std::vector<SkJob>& jobs, int job0, std::vector<SkItem>& items);
-void sk_gemm(tlr_ctx* ctx, int tn, const SkJob* jobs, const SkItem* items, int nitems, int nrhs);
 // Preconditioned CG vectors (k_solve.cu): per-column dot products (fixed-order sums) and the two
 // vector updates of an iteration, with per-column coefficients num/den read on the device.
 void coldot(tlr_ctx* ctx, int64_t n, int ncols, const double* X, int64_t ldx, const double* Y, int64_t ldy,

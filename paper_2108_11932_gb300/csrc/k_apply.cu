@@ -28,6 +28,7 @@
 #include <cstring>
 
 #include "internal.h"
+#include "warpsum.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -82,25 +83,6 @@ __device__ __forceinline__ void ap_ld_a(const double* p, double (&a)[VEC]) {
   } else {
     a[0] = __ldg(p);
   }
-}
-
-// Sums of P (a power of two) values over the warp by halving exchanges: afterwards lane l holds the sum
-// of value (l >> (5 - log2 P)).
-template <int P>
-__device__ __forceinline__ double ap_reduce(double (&v)[P], int lane) {
-  int o = 16;
-#pragma unroll
-  for (int n = P; n > 1; n /= 2, o /= 2) {
-    const bool up = lane & o;
-#pragma unroll
-    for (int i = 0; i < n / 2; ++i) {
-      const double keep = up ? v[i + n / 2] : v[i], send = up ? v[i] : v[i + n / 2];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-#pragma unroll
-  for (int q = 16 / P; q; q /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], q);
-  return v[0];
 }
 
 // X (original order) -> Xp (KD order, padded with zeros, row-major)
@@ -216,7 +198,7 @@ __global__ void __launch_bounds__(AP_T) k_apply_tn(ApTab T, const double* __rest
   double v[P];
 #pragma unroll
   for (int i = 0; i < P; ++i) v[i] = i % (P / AP_CW) < NR ? acc[i / (P / AP_CW)][(i % (P / AP_CW)) % NR] : 0.0;
-  const double s = ap_reduce<P>(v, lane);
+  const double s = warp_sums<P>(v, lane);
   if (out) *O = s;
 }
 

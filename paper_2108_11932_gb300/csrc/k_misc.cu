@@ -725,24 +725,6 @@ void trsm_left_t_block(tlr_ctx* ctx, int nbk, const double* L, int lda, int unit
 }
 
 // ------------------------------------------------------------------ elementwise helpers
-__global__ void k_scale_rows(int m, int n, const double* __restrict__ dv, int inv, const double* X,
-                             int ldx, double* Y, int ldy) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)m * n;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(e % m), c = (int)(e / m);
-    const double s = inv ? 1.0 / dv[r] : dv[r];
-    Y[r + (size_t)c * ldy] = X[r + (size_t)c * ldx] * s;
-  }
-}
-void scale_rows(tlr_ctx* ctx, int m, int n, const double* dvec, int inv, const double* X, int ldx,
-                double* Y, int ldy) {
-  if ((int64_t)m * n <= 0) return;
-  TLR_SITE_PRE(ctx);
-  k_scale_rows<<<std::min<unsigned>(cdiv((int64_t)m * n, 256), 4096u), 256, 0, ctx->stream>>>(
-      m, n, dvec, inv, X, ldx, Y, ldy);
-  TLR_LAUNCH_CHECK(ctx);
-}
-
 __global__ void k_add_diag(int n, double* A, int lda, double s) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) A[i + (size_t)i * lda] += s;
@@ -961,32 +943,6 @@ void kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell
     else if (d == 2) kernel_matvec_d<2>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy);
     else kernel_matvec_d<3>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy);
   }
-}
-
-// Row permutation between the original order and the KD (padded) order.
-// gather: Y[p] = X[idx[p]] for p < n_out (rows n_out..n_pad-1 of Y zeroed);
-// scatter: Y[idx[p]] = X[p] for p < n_out.
-__global__ void k_permute(int64_t n_out, int nrhs, const int64_t* __restrict__ idx, int gather,
-                          const double* __restrict__ X, int64_t ldx, double* __restrict__ Y, int64_t ldy,
-                          int64_t n_pad) {
-  const int64_t tot = (gather ? n_pad : n_out) * nrhs;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t rows = gather ? n_pad : n_out;
-    const int64_t p = e % rows;
-    const int c = (int)(e / rows);
-    if (gather) Y[p + c * ldy] = (p < n_out) ? X[idx[p] + c * ldx] : 0.0;
-    else Y[idx[p] + c * ldy] = X[p + c * ldx];
-  }
-}
-void permute_rows(tlr_ctx* ctx, int64_t n_out, int nrhs, const int64_t* idx, int gather,
-                  const double* X, int64_t ldx, double* Y, int64_t ldy, int64_t n_pad) {
-  const int64_t tot = (gather ? n_pad : n_out) * nrhs;
-  if (tot <= 0) return;
-  TLR_SITE_PRE(ctx);
-  k_permute<<<std::min<unsigned>(cdiv(tot, 256), 8192u), 256, 0, ctx->stream>>>(n_out, nrhs, idx, gather,
-                                                                               X, ldx, Y, ldy, n_pad);
-  TLR_LAUNCH_CHECK(ctx);
 }
 
 __global__ void k_copy_matrix(int m, int n, const double* __restrict__ X, int ldx, double* __restrict__ Y,

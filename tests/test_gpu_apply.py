@@ -83,6 +83,40 @@ def test_products_match_the_exported_tiles(T, N, d, b, eps, ldl):
     ctx.close()
 
 
+@pytest.mark.parametrize("N,d,b,eps,ldl", [
+    (100, 2, 128, 1e-6, False),     # one tile, ragged
+    (1000, 3, 64, 1e-4, True),      # L D L^T, ragged last tile
+    (700, 2, 75, 1e-6, False),      # odd tile size: columns on 8-byte boundaries
+    (600, 2, 50, 1e-3, True),
+    (1500, 1, 48, 1e-2, False),     # rank-1 and rank-0 tiles
+    (1500, 2, 1100, 1e-4, False),   # columns longer than a thread's loads in flight
+    (2600, 2, 2100, 1e-4, True),    # with 8 columns: longer than the staged vector
+])
+def test_solves_match_the_exported_factor(T, N, d, b, eps, ldl):
+    """The solve applies explicit inverses of the diagonal tiles and sums of n terms, so its forward error is
+    within n u cond(L D L^T) (Higham, Sections 8.1, 14.2); every column of every width on its own."""
+    import torch
+    ctx = T.Context(0)
+    o = T.default_opts(bs=16, seed=N)
+    F = ctx.compress(inputs.points(N, d, N), b, eps, 0.1, 1e-2 if eps > 1e-5 else 1e-4, o)
+    (F.ldlt if ldl else F.potrf)(eps, o)
+    L, _, dv = _dense(F, True)
+    A = L @ (dv[:, None] * L.T)
+    perm = F.perm()
+    tol = A.shape[0] * 2.0 ** -52 * np.linalg.cond(A)
+    rng = np.random.default_rng(N)
+    Y = rng.standard_normal((N, 33))
+    Yp = np.zeros((A.shape[0], 33))
+    Yp[:N] = Y[perm]
+    X = np.linalg.solve(A, Yp)[:N]
+    for nrhs in (1, 2, 3, 5, 7, 8, 9, 33):
+        B = T.fortran(torch.tensor(Y[:, :nrhs], device="cuda:0"))
+        g = F.solve(B).cpu().numpy()[perm]
+        err = np.linalg.norm(g - X[:, :nrhs], axis=0) / np.linalg.norm(X[:, :nrhs], axis=0)
+        assert np.all(err <= tol), (nrhs, err.max(), tol)
+    ctx.close()
+
+
 @pytest.mark.parametrize("N,d,ell,scale,nrhs", [
     (1, 2, 0.1, 1.0, 1),
     (31, 1, 0.1, 1.0, 2),         # less than a warp's columns
