@@ -150,18 +150,21 @@ struct BatchSampler : Sampler {
   // compressed rank / bs + 2), a later one half as many.  One Gaussian launch, one slicing and one
   // product of width bs (t1 - t0) replace that many per-round launches; each product keeps the
   // split-K of its one-round shape (rule_n = bs), so every element equals the one-round result.
+  int range_rounds(const Mat& M, int t) const {
+    int r0max = 0;
+    for (int i = M.k + 1; i < M.nb; ++i) r0max = std::max(r0max, M.A->rank[ix(M.A, i, M.k)]);
+    int n = (r0max + bs - 1) / bs + 2;
+    if (t > 0) n = std::max(2, n / 2);
+    const int64_t per = (int64_t)(std::max(M.Kk, 1) + std::max<int64_t>(M.R0k, 1)) * bs * (int64_t)sizeof(T);
+    return (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)n, 32, (int64_t)(32 << 20) / per}));
+  }
   void form_ranges(const std::vector<int>& ms, int t) {
     std::vector<int> nr(ms.size());
     std::vector<int64_t> omo(ms.size());
     int64_t omt = 0;
     for (size_t u = 0; u < ms.size(); ++u) {
       const Mat& M = *(*L)[ms[u]];
-      int r0max = 0;
-      for (int i = M.k + 1; i < M.nb; ++i) r0max = std::max(r0max, M.A->rank[ix(M.A, i, M.k)]);
-      int n = (r0max + bs - 1) / bs + 2;
-      if (t > 0) n = std::max(2, n / 2);
-      const int64_t per = (int64_t)(std::max(M.Kk, 1) + std::max<int64_t>(M.R0k, 1)) * bs * (int64_t)sizeof(T);
-      n = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)n, 32, (int64_t)(32 << 20) / per}));
+      const int n = range_rounds(M, t);
       nr[u] = n;
       omo[u] = omt;
       omt += (int64_t)M.b * bs * n;
@@ -295,36 +298,67 @@ struct BatchSampler : Sampler {
     oz_split_cols(ctx, cj);
   }
 
-  void sample(const std::vector<int>& ops, int t, const double*, const std::vector<double*>& Ydst) override {
+  // Rounds of an operand sampled in one product (Y = [U0 | Urow_i][W_t | W_(t+1) | ..]).  Every column sums as
+  // it would alone (the split of K is pinned to the one-round shape), so this changes no result; it spares
+  // the launches and host work of a round, which are most of its cost when few operands are active, and
+  // loads the panel once for all its rounds.  As many rounds as the tile's compressed rank says it will
+  // need (the updated tile's rank is a little lower: 14.9 against 16.2 on average for cov2d N = 131072 at 1e-6), at
+  // most AHEAD; past the prediction two at a time while at most AHEAD_TAIL operands are active (an unused
+  // sample costs less there than another round).  Within the rounds whose X blocks exist.
+  // Likelihood 2D N = 131072 1.585 -> 1.531 s, batch of 8 matrices up to 8192 points 99.5 -> 94.6 ms.
+  static constexpr int AHEAD = 8, AHEAD_TAIL = 4;
+  int ahead(int op, int t, int ns) override {
+    if (F32 || !mine(op)) return 1;
+    const int m = (*op_m)[op];
+    const Mat& M = *(*L)[m];
+    const int r0 = M.A->rank[ix(M.A, (*op_i)[op], M.k)];
+    int n = (int)std::ceil(0.9 * r0 / bs) + 1 - t;
+    if (n < 2) n = ns <= AHEAD_TAIL && t > 0 ? 2 : 1;
+    n = std::min(n, AHEAD);
+    if (M.mixed16 && bs % 16) return 1;  // a 16-column block of the truncated product would span two rounds
+    int end = t == 0 ? range_rounds(M, 0) : t + 1;  // the range this call forms: one round unless it is the first
+    if (xr.size() > (size_t)m)
+      for (const auto& r : xr[m])
+        if (t >= r.t0 && t < r.t1) end = r.t1;
+    return std::max(1, std::min(n, end - t));
+  }
+  void unused(int op, int n) override {
+    if (F32 || !mine(op)) return;
+    (*L)[(*op_m)[op]]->t64 -= n;
+  }
+
+  void sample(const std::vector<int>& ops, const std::vector<int>& ts, const std::vector<int>& ms, const double*,
+              const std::vector<double*>& Ydst) override {
     if (!u0_ready) prepare_u0();
-    // matrices present in this call
-    std::vector<int> mp;
-    std::vector<int> slot_of_m(L->size(), -1);
-    for (int op : ops) {
-      const int m = (*op_m)[op];
-      if (slot_of_m[m] < 0) { slot_of_m[m] = (int)mp.size(); mp.push_back(m); }
-    }
     // the shared products X = Urow_k^T Omega_t and X0 = V0col_k^T Omega_t of each matrix, formed for a
     // range of rounds at once
     if (xr.size() < L->size()) xr.resize(L->size());
-    std::vector<const XRange*> rng(mp.size(), nullptr);
-    std::vector<int> need;
-    for (size_t u = 0; u < mp.size(); ++u) {
-      for (const auto& r : xr[mp[u]])
-        if (t >= r.t0 && t < r.t1) rng[u] = &r;
-      if (!rng[u]) need.push_back(mp[u]);
-    }
-    if (!need.empty()) {
-      form_ranges(need, t);
-      for (size_t u = 0; u < mp.size(); ++u)
-        if (!rng[u]) rng[u] = &xr[mp[u]].back();
+    auto range_of = [&](int m, int t) -> const XRange* {
+      for (const auto& r : xr[m])
+        if (t >= r.t0 && t < r.t1) return &r;
+      return nullptr;
+    };
+    std::vector<int> order(ops.size());
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return ts[a] < ts[c]; });
+    for (size_t u = 0; u < order.size();) {  // round by round, the matrices without the round's blocks
+      const int t = ts[order[u]];
+      std::vector<int> need;
+      for (; u < order.size() && ts[order[u]] == t; ++u) {
+        const int m = (*op_m)[ops[order[u]]];
+        if (!range_of(m, t) && std::find(need.begin(), need.end(), m) == need.end()) need.push_back(m);
+      }
+      if (!need.empty()) form_ranges(need, t);
     }
     // W blocks of every operand (block-diagonal Gram products), then Y = [U0 | Urow] W
     std::vector<SlotDescT<T>> sd(ops.size());
     int64_t wtot = 0, ytot = 0;
     for (size_t s = 0; s < ops.size(); ++s) {
-      const int op = ops[s], u = slot_of_m[(*op_m)[op]], i = (*op_i)[op];
+      const int op = ops[s], t = ts[s], i = (*op_i)[op];
+      const int bsm = bs * ms[s];  // columns of the operand's sample
       const Mat& M = *(*L)[(*op_m)[op]];
+      const XRange* rg = range_of((*op_m)[op], t);
+      TLR_REQUIRE(rg && t + ms[s] <= rg->t1, TLR_ERR_STATE, "sampling: rounds outside the formed range");
       SlotDescT<T>& d = sd[s];
       d.rank = M.dtab;
       d.uoff = M.dtab + (size_t)M.nb * M.nb;
@@ -334,8 +368,8 @@ struct BatchSampler : Sampler {
       d.G = Panels<T>::G(M);
       d.ldx = std::max(M.Kk, 1);
       d.ldx0 = (int)std::max<int64_t>(M.R0k, 1);
-      d.X = rng[u]->X + (size_t)d.ldx * bs * (t - rng[u]->t0);
-      d.X0 = rng[u]->X0 + (size_t)d.ldx0 * bs * (t - rng[u]->t0);
+      d.X = rg->X + (size_t)d.ldx * bs * (t - rg->t0);
+      d.X0 = rg->X0 + (size_t)d.ldx0 * bs * (t - rg->t0);
       d.nb = M.nb;
       d.k = M.k;
       d.i = i;
@@ -343,14 +377,14 @@ struct BatchSampler : Sampler {
       d.x0off = (int)M.A->voff[ix(M.A, i, M.k)];
       d.Ki = (int)M.F->ulen[i];
       d.Kk = M.Kk;
-      d.q = bs;
-      d.bs = bs;
+      d.q = bsm;
+      d.bs = bsm;
       d.r0w = u0off[op] >= 0 ? round32(d.r0) : d.r0;
       d.W = reinterpret_cast<T*>(wtot);  // offset, fixed below
       d.P = nullptr;
       d.Z = nullptr;
-      wtot += (int64_t)(d.r0w + d.Ki) * bs;
-      ytot += (int64_t)M.b * bs;
+      wtot += (int64_t)(d.r0w + d.Ki) * bsm;
+      ytot += (int64_t)M.b * bsm;
     }
     T* W = bw->need<T>((size_t)std::max<int64_t>(wtot, 1));
     for (auto& d : sd) d.W = W + reinterpret_cast<size_t>(d.W);
@@ -362,7 +396,7 @@ struct BatchSampler : Sampler {
       for (int j = 0; j <= M.k; ++j) {
         const int R = j < M.k ? M.F->rank[ix(M.F, i, j)] : sd[s].r0w;
         for (int rc = 0; 16 * rc < R; ++rc)
-          for (int cc = 0; 16 * cc < bs; ++cc)
+          for (int cc = 0; 16 * cc < sd[s].bs; ++cc)
             items.push_back(BlkItem{(uint32_t)s, (uint16_t)j, (uint8_t)rc, (uint8_t)cc});
       }
     }
@@ -385,27 +419,29 @@ struct BatchSampler : Sampler {
     int64_t wsl = 0, wex = 0;  // slices of the W_i rows of the split products
     for (size_t s = 0; s < ops.size(); ++s) {
       const int ks = split_k(s);
-      if (ks > 0) { wsl += (int64_t)8 * oz_ld(ks) * bs; wex += bs; }
+      if (ks > 0) { wsl += (int64_t)8 * oz_ld(ks) * sd[s].bs; wex += sd[s].bs; }
     }
     int8_t* ws_ = wsl ? bws->need<int8_t>((size_t)wsl) : nullptr;
     int* we_ = wex ? bwe->need<int>((size_t)wex) : nullptr;
     for (size_t s = 0; s < ops.size(); ++s) {
       const int op = ops[s], i = (*op_i)[op];
       Mat& M = *(*L)[(*op_m)[op]];
-      const int r0 = sd[s].r0, r0w = sd[s].r0w, Ki = sd[s].Ki, ldw = std::max(r0w + Ki, 1);
+      const int bsm = sd[s].bs, r0 = sd[s].r0, r0w = sd[s].r0w, Ki = sd[s].Ki, ldw = std::max(r0w + Ki, 1);
       T* Yo = F32 ? Y32 + yo : reinterpret_cast<T*>(Ydst[s]);
       const T* U0 = r0 ? Panels<T>::AU(M, i) + (size_t)M.b * M.A->uoff[ix(M.A, i, M.k)] : nullptr;
-      GemmJob<T> g = job<T>(NN, M.b, bs, U0, M.b, sd[s].W, ldw, r0, Yo, M.b, 1.0, 0.0);
+      GemmJob<T> g = job<T>(NN, M.b, bsm, U0, M.b, sd[s].W, ldw, r0, Yo, M.b, 1.0, 0.0);
+      g.rule_n = bs;
       const int ks = split_k(s);  // exact integer totals need K <= 16384
       if (ks > 0) {
         const int ldo = oz_ld(ks);
         const int w0 = folded(s) ? 0 : r0;  // first W row of the product
-        OzColJob c{reinterpret_cast<const double*>(sd[s].W + w0), ws_, we_, ldw, bs, 0, ks};
+        OzColJob c{reinterpret_cast<const double*>(sd[s].W + w0), ws_, we_, ldw, bsm, 0, ks};
         c.ldo = ldo;
         wcj.push_back(c);
         OzJob y{M.FUt[i], ws_, d_one, we_, reinterpret_cast<double*>(Yo), (size_t)M.b * M.futcap[i],
-                (size_t)ldo * bs, (int)M.futcap[i], M.b, M.b, bs, ks};
+                (size_t)ldo * bsm, (int)M.futcap[i], M.b, M.b, bsm, ks};
         y.ldb = ldo;
+        y.rule_n = bs;
         if (folded(s)) {  // Y = [U0 | Urow_i] W on the tensor cores alone
           const int8_t* u0 = static_cast<const int8_t*>(bu0->p) + u0off[ops[s]];
           if (Ki > 0) {
@@ -425,8 +461,8 @@ struct BatchSampler : Sampler {
         }
         if (M.mixed16) y.tol = M.thr / (8.0 * std::sqrt((double)M.b));  // column norm of Y within thr / 8
         wyj.push_back(y);
-        ws_ += (size_t)8 * ldo * bs;
-        we_ += bs;
+        ws_ += (size_t)8 * ldo * bsm;
+        we_ += bsm;
       } else {
         g.A[1] = Panels<T>::U(M, i);
         g.lda[1] = M.b;
@@ -435,13 +471,13 @@ struct BatchSampler : Sampler {
         g.K[1] = Ki;
         jy.push_back(g);
       }
-      if (F32) cb.push_back(ConvBackJob{reinterpret_cast<const float*>(Yo), Ydst[s], (int64_t)M.b * bs});
-      yo += (int64_t)M.b * bs;
-      (F32 ? M.fl32 : M.fl_exec) += 2.0 * M.b * bs * (r0 + Ki);
+      if (F32) cb.push_back(ConvBackJob{reinterpret_cast<const float*>(Yo), Ydst[s], (int64_t)M.b * bsm});
+      yo += (int64_t)M.b * bsm;
+      (F32 ? M.fl32 : M.fl_exec) += 2.0 * M.b * bsm * (r0 + Ki);
       double R = r0;  // paper model: 4 products per (i, j) pair, Equation 2
       for (int j = 0; j < M.k; ++j) R += M.F->rank[ix(M.F, i, j)] + M.F->rank[ix(M.F, M.k, j)];
-      M.fl_model += 4.0 * M.b * bs * R;
-      (F32 ? M.t32 : M.t64) += 1;
+      M.fl_model += 4.0 * M.b * bsm * R;
+      (F32 ? M.t32 : M.t64) += ms[s];
     }
     gemm<T>(ctx, NN, jy);
     oz_split_cols(ctx, wcj);
@@ -625,15 +661,23 @@ struct SplitSampler : Sampler {
   BatchSampler<float>* f32;
   const std::vector<char>* is32;
   bool owns_omega() const override { return true; }
-  void sample(const std::vector<int>& ops, int t, const double* Om, const std::vector<double*>& Y) override {
-    std::vector<int> o32, o64;
-    std::vector<double*> y32, y64;
+  void sample(const std::vector<int>& ops, const std::vector<int>& ts, const std::vector<int>& ms, const double* Om,
+              const std::vector<double*>& Y) override {
+    std::vector<int> o[2], t[2], m[2];  // FP64, FP32
+    std::vector<double*> y[2];
     for (size_t s = 0; s < ops.size(); ++s) {
-      if ((*is32)[ops[s]]) { o32.push_back(ops[s]); y32.push_back(Y[s]); }
-      else { o64.push_back(ops[s]); y64.push_back(Y[s]); }
+      const int w = (*is32)[ops[s]] ? 1 : 0;
+      o[w].push_back(ops[s]);
+      t[w].push_back(ts[s]);
+      m[w].push_back(ms[s]);
+      y[w].push_back(Y[s]);
     }
-    if (!o32.empty()) f32->sample(o32, t, Om, y32);
-    if (!o64.empty()) f64->sample(o64, t, Om, y64);
+    if (!o[1].empty()) f32->sample(o[1], t[1], m[1], Om, y[1]);
+    if (!o[0].empty()) f64->sample(o[0], t[0], m[0], Om, y[0]);
+  }
+  int ahead(int op, int t, int ns) override { return (*is32)[op] ? 1 : f64->ahead(op, t, ns); }
+  void unused(int op, int n) override {
+    if (!(*is32)[op]) f64->unused(op, n);
   }
   void project(const std::vector<int>& q) override {
     f32->project(q);
@@ -1577,9 +1621,12 @@ struct Session {
       struct Deferred : Sampler {
         Sampler* f;
         bool owns_omega() const override { return true; }
-        void sample(const std::vector<int>& ops, int t, const double* Om, const std::vector<double*>& Y) override {
-          f->sample(ops, t, Om, Y);
+        void sample(const std::vector<int>& ops, const std::vector<int>& ts, const std::vector<int>& ms, const double* Om,
+                    const std::vector<double*>& Y) override {
+          f->sample(ops, ts, ms, Om, Y);
         }
+        int ahead(int op, int t, int ns) override { return f->ahead(op, t, ns); }
+        void unused(int op, int n) override { f->unused(op, n); }
         void project(const std::vector<int>&) override {}
       } dsmp;
       dsmp.f = smp;

@@ -64,8 +64,15 @@ struct Sampler {
   virtual ~Sampler() {}
   // true: the sampler draws its own Gaussian blocks (one per matrix of the batch)
   virtual bool owns_omega() const { return false; }
-  // Y[s] = T_{ops[s]} Omega_t, written to Ydst[s] (n_op x bs, leading dimension n_op).
-  virtual void sample(const std::vector<int>& ops, int t, const double* Om, const std::vector<double*>& Ydst) = 0;
+  // Y[s] = T_{ops[s]} [Omega_t .. Omega_(t + m[s] - 1)], t = ts[s], written to Ydst[s] (n_op x bs m[s], leading
+  // dimension n_op).  A sampler that takes its Gaussian blocks from the engine gets m = 1 and one t per call.
+  virtual void sample(const std::vector<int>& ops, const std::vector<int>& ts, const std::vector<int>& m,
+                      const double* Om, const std::vector<double*>& Ydst) = 0;
+  // rounds worth sampling at once for an operand about to sample round t while ns operands are active; a sample
+  // does not depend on the rounds before it, so it may be formed ahead of them
+  virtual int ahead(int, int /*t*/, int /*ns*/) { return 1; }
+  // the operand converged with n of its rounds sampled ahead but not used
+  virtual void unused(int, int /*n*/) {}
   // B_op = T_op^T Q_op for every operand, given the final widths q.
   virtual void project(const std::vector<int>& q) = 0;
 };

@@ -9,6 +9,8 @@
 #include <chrono>
 #include <cstring>
 #include <cstdio>
+#include <map>
+#include <memory>
 #include <numeric>
 
 #include "internal.h"
@@ -422,9 +424,8 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
   int nmax = 0;
   for (int v : nrow) nmax = std::max(nmax, v);
   const int slots = std::max(1, std::min(cf.max_slots > 0 ? cf.max_slots : nops, nops));
-  Buf bOm(ctx), bY(ctx), bW(ctx), bS(ctx), bG(ctx), bM(ctx), bSt(ctx), bE(ctx), bT(ctx), bOr(ctx);
+  Buf bOm(ctx), bW(ctx), bS(ctx), bG(ctx), bM(ctx), bSt(ctx), bE(ctx), bT(ctx), bOr(ctx);
   double* Om = S.owns_omega() ? nullptr : bOm.need<double>((size_t)nmax * bs);
-  double* Y = bY.need<double>((size_t)slots * nmax * bs);
   double* W = bW.need<double>((size_t)slots * nmax * bs);
   double* Sb = bS.need<double>((size_t)slots * (nmax + bs) * bs);
   double* G = bG.need<double>((size_t)slots * bs * bs);
@@ -433,6 +434,29 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
   double* en = bE.need<double>((size_t)slots);
   double* thr_d = bT.need<double>((size_t)slots);
   std::vector<double> thr_h(slots);
+
+  // Samples of m rounds of an operand, formed in one product; rounds next .. m - 1 are still to be used.
+  // Their blocks are kept by size and handed on (everything runs on one stream).
+  struct Ahead {
+    double* Y = nullptr;
+    int m = 0, next = 0;
+  };
+  std::vector<Ahead> have(nops);
+  std::vector<std::unique_ptr<Buf>> pool;
+  std::map<int, std::vector<double*>> spare;
+  auto take = [&](int m) -> double* {
+    std::vector<double*>& f = spare[m];
+    if (f.empty()) {
+      const int64_t one = (int64_t)m * nmax * bs * (int64_t)sizeof(double);
+      const int n = (int)std::max<int64_t>(1, std::min<int64_t>(slots, ((int64_t)64 << 20) / one));  // allocated together
+      pool.emplace_back(new Buf(ctx));
+      double* p = pool.back()->need<double>((size_t)n * m * nmax * bs);
+      for (int i = 0; i < n; ++i) f.push_back(p + (size_t)i * m * nmax * bs);
+    }
+    double* p = f.back();
+    f.pop_back();
+    return p;
+  };
 
   std::vector<int> active;
   std::vector<int> round(nops, 0);
@@ -445,21 +469,44 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
   while (!active.empty()) {
     const int ns = (int)active.size();
     prof_mark(ctx, PH_SAMPLE);
-    // Omega depends on the operand's own round: group the slots by round
-    std::vector<int> rounds_present;
-    for (int op : active) rounds_present.push_back(round[op]);
-    std::sort(rounds_present.begin(), rounds_present.end());
-    rounds_present.erase(std::unique(rounds_present.begin(), rounds_present.end()), rounds_present.end());
-    for (int t : rounds_present) {
-      std::vector<int> ops_t;
+    // sample the operands whose current round has not been sampled ahead
+    {
+      std::vector<int> ops, ts, ms;
       std::vector<double*> ydst;
-      for (int s = 0; s < ns; ++s)
-        if (round[active[s]] == t) {
-          ops_t.push_back(active[s]);
-          ydst.push_back(Y + (size_t)s * nmax * bs);
+      for (int op : active) {
+        Ahead& h = have[op];
+        if (h.next < h.m) continue;
+        h.next = 0;
+        h.m = std::max(1, Om ? 1 : S.ahead(op, round[op], ns));
+        h.Y = take(h.m);
+        ops.push_back(op);
+        ts.push_back(round[op]);
+        ms.push_back(h.m);
+        ydst.push_back(h.Y);
+      }
+      if (!Om) {
+        if (!ops.empty()) S.sample(ops, ts, ms, nullptr, ydst);
+      } else {  // Omega depends on the operand's own round: group the slots by round
+        std::vector<int> rounds_present(ts);
+        std::sort(rounds_present.begin(), rounds_present.end());
+        rounds_present.erase(std::unique(rounds_present.begin(), rounds_present.end()), rounds_present.end());
+        for (int t : rounds_present) {
+          std::vector<int> ops_t;
+          std::vector<double*> y_t;
+          for (size_t s = 0; s < ops.size(); ++s)
+            if (ts[s] == t) {
+              ops_t.push_back(ops[s]);
+              y_t.push_back(ydst[s]);
+            }
+          omega(ctx, cf.seed, cf.stream, cf.k, (uint32_t)t, nrow[ops_t[0]], bs, Om);
+          S.sample(ops_t, std::vector<int>(ops_t.size(), t), std::vector<int>(ops_t.size(), 1), Om, y_t);
         }
-      if (Om) omega(ctx, cf.seed, cf.stream, cf.k, (uint32_t)t, nrow[ops_t[0]], bs, Om);
-      S.sample(ops_t, t, Om, ydst);
+      }
+    }
+    std::vector<double*> Y(ns);  // each slot's sample of its round
+    for (int s = 0; s < ns; ++s) {
+      Ahead& h = have[active[s]];
+      Y[s] = h.Y + (size_t)nrow[active[s]] * bs * h.next++;
     }
     prof_mark(ctx, PH_ORTH);
     bool fused = orth_fused_ok(bs);
@@ -473,7 +520,7 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
       std::vector<OrthSlot> os(ns);
       for (int s = 0; s < ns; ++s) {
         const int op = active[s], n = nrow[op];
-        os[s] = OrthSlot{Q + qoff[op], Y + (size_t)s * nmax * bs, W + (size_t)s * nmax * bs, n, q[op], thr[op]};
+        os[s] = OrthSlot{Q + qoff[op], Y[s], W + (size_t)s * nmax * bs, n, q[op], thr[op]};
         st.flops += 8.0 * n * q[op] * bs + 6.0 * n * bs * bs;
       }
       orth_round(ctx, bs, os, status, en, TAU_DROP, bOr);
@@ -487,7 +534,7 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
       for (int s = 0; s < ns; ++s) {
         const int op = active[s], n = nrow[op];
         const double* Qo = Q + qoff[op];
-        double* Ys = Y + (size_t)s * nmax * bs;
+        double* Ys = Y[s];
         double* Ss = Sb + (size_t)s * (nmax + bs) * bs;
         if (q[op] > 0) {
           j1.push_back(job<double>(TN, q[op], bs, Qo, n, Ys, n, n, Ss, q[op], 1.0, 0.0));
@@ -503,7 +550,7 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
       std::vector<GemmJob<double>> j4;
       for (int s = 0; s < ns; ++s) {
         const int n = nrow[active[s]];
-        j4.push_back(job<double>(NN, n, bs, Y + (size_t)s * nmax * bs, n, M + (size_t)s * bs * bs, bs, bs,
+        j4.push_back(job<double>(NN, n, bs, Y[s], n, M + (size_t)s * bs * bs, bs, bs,
                                  W + (size_t)s * nmax * bs, n, 1.0, 0.0));
       }
       gemm<double>(ctx, NN, j4);
@@ -552,6 +599,12 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
       }
       if (!done && round[op] > 2 * n + 4) done = true;  // hard bound (each round adds >= 1 column)
       if (!done) still.push_back(op);
+      Ahead& h = have[op];
+      if (done || h.next == h.m) {
+        if (h.next < h.m) S.unused(op, h.m - h.next);
+        spare[h.m].push_back(h.Y);
+        h = Ahead();
+      }
     }
     active.swap(still);
     refill();
@@ -574,7 +627,8 @@ struct DenseSampler : Sampler {
   double* B;        // nops x n x n (first q columns used)
   const OzTiles* oz = nullptr;
   double flops = 0;
-  void sample(const std::vector<int>& ops, int, const double* Om, const std::vector<double*>& Ydst) override {
+  void sample(const std::vector<int>& ops, const std::vector<int>&, const std::vector<int>&, const double* Om,
+              const std::vector<double*>& Ydst) override {
     flops += 2.0 * n * n * bs * ops.size();
     if (oz) {
       int8_t* Xs = oz->bx->need<int8_t>((size_t)8 * n * bs);
