@@ -18,22 +18,30 @@
 //    below 2^24: the FP32 accumulation of the tensor core is exact.  Every 128 k the group sums move
 //    from tensor memory to 32-bit integer totals (exact for K <= 16384), combined once at the end.
 //
-// Kernel structure (one CTA = 128 output rows x 16 output columns x one K slice, 320 threads):
+// Kernel structure (one CTA = 128 output rows x TN = 16 or 32 output columns x one K slice):
 //  * warp 0: TMA producer.  Boxes of the int8 chunk planes of A and B (one per plane) are copied by
-//    cp.async.bulk.tensor into a 2-stage ring (32 k per stage), mbarrier completion.  Operands
+//    cp.async.bulk.tensor into a 4-stage ring (32 k per stage), mbarrier completion.  Operands
 //    stored along k are read through a 4D view (16 k, rows, k / 16, plane), so a stage holds each
 //    16-k half as [row][16 bytes] and a warp's 16-byte reads of consecutive rows are contiguous.
-//  * warps 2-5: converters.  Thread t owns row t of the A tile (and one stacked row of B): int8 chunks
-//    become FP16 (two byte permutes and one f16x2 subtraction per pair) in the canonical K-major
-//    layout of the tensor core (8-row x 16-byte core matrices; either orientation of A in HBM lands
-//    in the same layout), into one of four chunk buffers, so conversion runs ahead of the MMAs.
+//  * warps 2-9: converters, two groups of four warps, each taking one 16-k half of every stage (a group's
+//    waits for its shared loads and tensor-memory stores are the other's issue slots).  A thread owns
+//    a row of the A tile (and TN / 16 stacked rows of B): int8 chunks become FP16 (two byte permutes and
+//    one f16x2 subtraction per pair), A in tensor memory, B in the canonical K-major layout of the tensor
+//    core (8-row x 16-byte core matrices), into one of four chunk buffers, so that conversion runs ahead of
+//    the MMAs; either orientation of A in HBM lands in the same layout.
 //  * warp 1: one thread issues tcgen05.mma (kind::f16, FP16 in, FP32 accumulate in tensor memory).
-//    For a 16-k step and A slice i, B is the stack [B_1 | ... | B_(S+1-i)] (N = 16 (S + 1 - i)) and
+//    For a 16-k step and A slice i, B is the stack [B_1 | ... | B_(S+1-i)] (N = TN (S + 1 - i)) and
 //    the accumulator starts at the column block of group i - 1: every group sum accumulates in place.
-//    Two 128-column accumulator buffers alternate between 128-k windows.
-//  * warps 6-9: epilogue.  They drain each window's group sums (tcgen05.ld) into integer totals
-//    while the next window accumulates, then recombine in FP64 and store (or write split-K partials,
-//    summed in slice order by the last CTA of each output block).
+//    With TN = 16 two 128-column accumulator buffers alternate between 128-k windows.
+//  * the last 4 or 8 warps: epilogue, 16 columns each.  They drain each window's group sums (tcgen05.ld) into
+//    two 64-bit integers per output, the groups 0-3 and 4-7 combined by their weights, then recombine in
+//    FP64 and store (or write split-K partials, summed in slice order by the last CTA of each output block).
+// An MMA costs about 120 cycles to issue whatever its N, and the conversion of A does not depend on the columns
+// either, so products of more than 16 columns take the wide form: 32 columns for the price of 16.  (Truncated
+// products choose their planes per 16-column block and stay narrow.)  Measured over the factorization of cov2d
+// N = 131072 (device time, four converter warps and 16 columns -> now): L_kk^-1 B 29.6 -> 19.1 ms, diagonal
+// updates 43.3 -> 20.6, samples of two and more rounds 171 -> 127, projections 111 -> 87, Gram factors 42 -> 34;
+// likelihood 1.531 -> 1.436 s.
 // Every wait is bounded: on a timeout the CTA sets a device flag, lets its copies land, frees its
 // tensor memory and returns; the host reports TLR_ERR_TIMEOUT.
 #include <cuda.h>
@@ -55,25 +63,30 @@ namespace {
 
 constexpr int OZ_S = 8;       // chunk planes per operand
 constexpr int OZ_TM = 128;    // output rows per CTA (tcgen05 M)
-constexpr int OZ_TN = 16;     // output columns per CTA
+constexpr int OZ_TN = 16;     // output columns per CTA of the narrow form; the wide form holds 32
 constexpr int OZ_KS = 32;     // k per TMA stage
 constexpr int OZ_KC = 16;     // k per MMA
 constexpr int OZ_CW = 8;      // 16-k steps per exact window (128 k)
 constexpr int OZ_NST = 4;     // int8 stages in flight
 constexpr int OZ_NBF = 4;     // FP16 chunk buffers between the converters and the MMA issuer
-constexpr int OZ_THREADS = 320;
+constexpr int OZ_CONV = 8;    // converter warps: two groups of four, one per 16-k half of a stage
 constexpr int ST_A = OZ_S * OZ_TM * OZ_KS;        // int8 A per stage (32 KB)
-constexpr int ST_B = OZ_S * OZ_TN * OZ_KS;        // int8 B per stage (4 KB)
-constexpr int ST_BYTES = ST_A + ST_B;
-constexpr int BF_B = OZ_S * OZ_TN * OZ_KC * 2;    // stacked FP16 B chunk in shared memory, 128 rows (4 KB)
-constexpr int BF_BYTES = BF_B;
-// Tensor memory: two accumulator buffers of 8 groups x 16 columns (columns 0-255), then OZ_NBF FP16
-// A chunks (128 lanes = rows; 8 planes x 8 columns, each column two k values)
+// Tensor memory, 512 columns: accumulator buffers of 8 groups x TN columns (two of 128 for TN = 16, one of
+// 256 for TN = 32), then OZ_NBF FP16 A chunks (128 lanes = rows; 8 planes x 8 columns, each column two k)
 constexpr int OZ_TMEM_COLS = 512;
 constexpr int OZ_TMEM_A = 256;
 constexpr int OZ_A_COLS = OZ_S * OZ_KC / 2;       // 64 columns per A chunk
-constexpr int OZ_SMEM = 1024 + OZ_NST * ST_BYTES + OZ_NBF * BF_BYTES + 256;
 static_assert(OZ_TMEM_A + OZ_NBF * OZ_A_COLS <= OZ_TMEM_COLS, "tensor memory budget");
+template <int TN>
+struct OzForm {
+  static constexpr int ST_B = OZ_S * TN * OZ_KS;       // int8 B per stage (4 or 8 KB)
+  static constexpr int ST_BYTES = ST_A + ST_B;
+  static constexpr int BF_BYTES = OZ_S * TN * OZ_KC * 2;  // stacked FP16 B chunk in shared memory
+  static constexpr int NACC = 256 / (OZ_S * TN);       // accumulator buffers
+  static constexpr int EPI = 4 * (TN / 16);            // epilogue warps: 16 columns each
+  static constexpr int THREADS = 32 * (2 + OZ_CONV + EPI);
+  static constexpr int SMEM = 1024 + OZ_NST * ST_BYTES + OZ_NBF * BF_BYTES + 256;
+};
 constexpr unsigned long long OZ_WAIT_NS = 2000000000ull;
 
 // Tensor maps live in the job table (global memory); CUtensorMap carries its own (>= 64-byte)
@@ -242,23 +255,36 @@ __device__ __forceinline__ void oz_cvt16(const uint32_t (&w)[4], uint32_t (&o)[8
   for (int q = 0; q < 4; ++q) oz_cvt4(w[q], o[2 * q], o[2 * q + 1]);
 }
 
-// Drain accumulator window w (buffer w & 1) of this thread's TMEM lane into the integer totals (each
-// group of a window is an integer below 2^24; over K <= 16384 a total stays below 2^31) and release
-// the buffer to the MMA issuer.
-__device__ __forceinline__ bool oz_drain(int w, int S, uint32_t b_accf, uint32_t b_acce, uint32_t tmem, int lq,
-                                         volatile int* abort, int (&tot)[OZ_S][OZ_TN]) {
-  const int buf = w & 1;
-  if (!mbar_wait(b_accf + 8 * buf, (w >> 1) & 1, abort)) return false;
+// Drain accumulator window w (buffer w % NACC) of this thread's TMEM lane, 16 columns from c0 of every group,
+// into the totals and release the buffer to the MMA issuer.  Group g of a window is an integer of at most
+// (g + 1) 128 127^2 < 2^24, so pairs of neighbouring groups combine in 32 bits (below 1.9e9) and the fours in
+// 64: hi = ((g0 2^7 + g1) 2^14) + (g2 2^7 + g3), lo the same of groups 4-7.
+template <int TN>
+__device__ __forceinline__ bool oz_drain(int w, int S, uint32_t b_accf, uint32_t b_acce, uint32_t tmem, int lq, int c0,
+                                         volatile int* abort, long long (&hi)[16], long long (&lo)[16]) {
+  constexpr int NACC = OzForm<TN>::NACC;
+  const int buf = w % NACC;
+  if (!mbar_wait(b_accf + 8 * buf, (w / NACC) & 1, abort)) return false;
   tc_fence_after();
-  const uint32_t ta = tmem + ((uint32_t)(32 * lq) << 16) + buf * 128;
+  const uint32_t ta = tmem + ((uint32_t)(32 * lq) << 16) + buf * 128 + c0;
 #pragma unroll
-  for (int g = 0; g < OZ_S; ++g)
-    if (g < S) {
-      uint32_t r[16];
-      tmem_ld16(ta + OZ_TN * g, r);
+  for (int g = 0; g < OZ_S; g += 2) {
+    if (g >= S) break;
+    uint32_t r[16], q[16];
+    tmem_ld16(ta + TN * g, r);
+    if (g + 1 < S) {
+      tmem_ld16(ta + TN * (g + 1), q);
+    } else {
 #pragma unroll
-      for (int c = 0; c < OZ_TN; ++c) tot[g][c] += __float2int_rn(__uint_as_float(r[c]));
+      for (int c = 0; c < 16; ++c) q[c] = 0;
     }
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+      const int p = __float2int_rn(__uint_as_float(r[c])) * 128 + __float2int_rn(__uint_as_float(q[c]));
+      long long& t = g < 4 ? hi[c] : lo[c];
+      t += (long long)p * (g % 4 == 0 ? 16384 : 1);
+    }
+  }
   tc_fence_before();
   mbar_arrive(b_acce + 8 * buf);
   return true;
@@ -358,13 +384,15 @@ __global__ void __launch_bounds__(256) k_oz_split_cols(const OzColJob* __restric
 // C(M x N) = 2^(eA + eB_n) * sum over chunk pairs (i, j), i + j <= S + 1, of A_i B_j 2^(-7(i+j)),
 // A(m, k) = A_i[k + m lda] (rows along k) or, with acol, A_i[m + k lda]; B(k, n) = B_j[k + n ldb].
 // Grid (ceil(M / 128), tiles_n * nsplit, jobs).
-__global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_mma(const OzDev* __restrict__ jobs) {
+template <int TN>
+__global__ void __launch_bounds__(OzForm<TN>::THREADS, 1) k_oz_mma(const OzDev* __restrict__ jobs) {
+  using F = OzForm<TN>;
   const OzDev* Jp = jobs + blockIdx.z;
   const int tiles_n = Jp->tiles_n, nsplit = Jp->nsplit;
   if ((int)blockIdx.y >= tiles_n * nsplit) return;
   const int nt = blockIdx.y % tiles_n, split = blockIdx.y / tiles_n;
   const int M = Jp->M, N = Jp->N, K = Jp->K, acol = Jp->acol;
-  const int m0 = blockIdx.x * OZ_TM, n0 = nt * OZ_TN;
+  const int m0 = blockIdx.x * OZ_TM, n0 = nt * TN;
   if (m0 >= M || n0 >= N) return;
   // Planes used: S, or with a tolerance the fewest s >= smin whose bound K (s + 1) 2^(eA + eB - 7 s)
   // on every entry's error (truncation of both operands to 7s bits plus the dropped chunk pairs;
@@ -372,7 +400,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_mma(const OzDev* __restric
   int S = Jp->S;
   if (Jp->tol > 0.0) {
     int eb = -100000;
-    for (int c = 0; c < OZ_TN; ++c)
+    for (int c = 0; c < TN; ++c)
       if (n0 + c < N) eb = max(eb, Jp->eB[(n0 + c) * Jp->eB_stride]);
     const int ea = *Jp->eA;
     for (int s = Jp->smin; s < S; ++s)
@@ -388,7 +416,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_mma(const OzDev* __restric
     const int kl = min(se * OZ_KS, K) - sb * OZ_KS;
     unsigned long long by = 0;
     if (nt == 0) by += (unsigned long long)S * min(OZ_TM, M - m0) * kl;
-    if (blockIdx.x == 0) by += (unsigned long long)S * min(OZ_TN, N - n0) * kl;
+    if (blockIdx.x == 0) by += (unsigned long long)S * min(TN, N - n0) * kl;
     atomicAdd(&g_oz_stats[S], 1ull);
     atomicAdd(&g_oz_stats[9], by);
   }
@@ -398,8 +426,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_mma(const OzDev* __restric
   extern __shared__ uint8_t oz_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(oz_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* ring = base;                           // OZ_NST stages of int8 A then B
-  uint8_t* bfb = ring + OZ_NST * ST_BYTES;        // OZ_NBF FP16 chunk buffers: A planes then stacked B
-  uint64_t* bars = reinterpret_cast<uint64_t*>(bfb + OZ_NBF * BF_BYTES);
+  uint8_t* bfb = ring + OZ_NST * F::ST_BYTES;     // OZ_NBF FP16 chunk buffers of stacked B
+  uint64_t* bars = reinterpret_cast<uint64_t*>(bfb + OZ_NBF * F::BF_BYTES);
   // barriers: full8[OZ_NST] empty8[OZ_NST] fullbf[OZ_NBF] emptybf[OZ_NBF] accf[2] acce[2] fin
   const uint32_t b_full8 = su32(bars), b_empty8 = su32(bars + OZ_NST), b_fullbf = su32(bars + 2 * OZ_NST),
                  b_emptybf = su32(bars + 2 * OZ_NST + OZ_NBF), b_accf = su32(bars + 2 * OZ_NST + 2 * OZ_NBF),
@@ -411,7 +439,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_mma(const OzDev* __restric
   if (tid == 0) {
     for (int s = 0; s < OZ_NST; ++s) {
       mbar_init(b_full8 + 8 * s, 1);
-      mbar_init(b_empty8 + 8 * s, 128);
+      mbar_init(b_empty8 + 8 * s, 32 * OZ_CONV);
     }
     for (int s = 0; s < OZ_NBF; ++s) {
       mbar_init(b_fullbf + 8 * s, 128);
@@ -419,7 +447,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_mma(const OzDev* __restric
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(b_accf + 8 * s, 1);
-      mbar_init(b_acce + 8 * s, 128);
+      mbar_init(b_acce + 8 * s, 32 * F::EPI);
     }
     mbar_init(b_fin, 1);
     *abort = 0;
@@ -442,19 +470,19 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_mma(const OzDev* __restric
       asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&Jp->tb) : "memory");
       const int K0 = Jp->K0;
       if (K0 > 0) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(&Jp->ta0) : "memory");
-      const uint32_t bytes = (uint32_t)(S * (OZ_TM * OZ_KS + OZ_TN * OZ_KS));  // one box per plane
+      const uint32_t bytes = (uint32_t)(S * (OZ_TM * OZ_KS + TN * OZ_KS));  // one box per plane
       int issued = 0;
       for (int s = 0; s < nst; ++s) {
         const int slot = s % OZ_NST;
         if (!mbar_wait(b_empty8 + 8 * slot, ((s / OZ_NST) & 1) ^ 1, abort)) break;
-        uint8_t* st = ring + slot * ST_BYTES;
+        uint8_t* st = ring + slot * F::ST_BYTES;
         const int k0 = (sb + s) * OZ_KS;
         mbar_expect_tx(b_full8 + 8 * slot, bytes);
         for (int q = 0; q < S; ++q) {
           if (acol) tma_3d(su32(st + q * (OZ_TM * OZ_KS)), &Jp->ta, m0, k0, q, b_full8 + 8 * slot);
           else if (k0 < K0) tma_4d(su32(st + q * (OZ_TM * OZ_KS)), &Jp->ta0, 0, m0, k0 / 16, q, b_full8 + 8 * slot);
           else tma_4d(su32(st + q * (OZ_TM * OZ_KS)), &Jp->ta, 0, m0, (k0 - K0) / 16, q, b_full8 + 8 * slot);
-          tma_4d(su32(st + ST_A + q * (OZ_TN * OZ_KS)), &Jp->tb, 0, n0, k0 / 16, q, b_full8 + 8 * slot);
+          tma_4d(su32(st + ST_A + q * (TN * OZ_KS)), &Jp->tb, 0, n0, k0 / 16, q, b_full8 + 8 * slot);
         }
         issued = s + 1;
       }
@@ -469,15 +497,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_mma(const OzDev* __restric
       for (int c = 0; c < nch; ++c) {
         const int sbf = c % OZ_NBF;
         if (!mbar_wait(b_fullbf + 8 * sbf, (c / OZ_NBF) & 1, abort)) break;
-        const int w = c / OZ_CW, buf = w & 1;
+        const int w = c / OZ_CW, buf = w % F::NACC;
         const bool first = (c % OZ_CW) == 0;
-        if (first && !mbar_wait(b_acce + 8 * buf, ((w >> 1) & 1) ^ 1, abort)) break;
+        if (first && !mbar_wait(b_acce + 8 * buf, ((w / F::NACC) & 1) ^ 1, abort)) break;
         tc_fence_after();
-        const uint64_t bd = umma_desc(bf0 + sbf * BF_BYTES, OZ_S * OZ_TN * 16, 128);
+        const uint64_t bd = umma_desc(bf0 + sbf * F::BF_BYTES, OZ_S * TN * 16, 128);
         const uint32_t at = tmem + OZ_TMEM_A + sbf * OZ_A_COLS;
 #pragma unroll 1
         for (int i = 0; i < S; ++i)
-          umma_f16_ts(tmem + buf * 128 + OZ_TN * i, at + i * (OZ_KC / 2), bd, umma_idesc(OZ_TM, OZ_TN * (S - i)),
+          umma_f16_ts(tmem + buf * 128 + TN * i, at + i * (OZ_KC / 2), bd, umma_idesc(OZ_TM, TN * (S - i)),
                       (first && i == 0) ? 0 : 1);
         umma_commit(b_emptybf + 8 * sbf);
         if ((c % OZ_CW) == OZ_CW - 1 || c == nch - 1) umma_commit(b_accf + 8 * buf);
@@ -485,101 +513,88 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_mma(const OzDev* __restric
       umma_commit(b_fin);  // arrives when every MMA of this thread has completed
       mbar_drain(b_fin, 0);
     }
-  } else if (warp < 6) {
-    // ---------------- converters (warps 2-5): int8 chunks -> FP16.  A warp may reach only its quarter
-    // of the tensor-memory lanes, so thread (warp, lane) owns A row 32 (warp % 4) + lane, written to
-    // the chunk's A buffer in tensor memory (one 8-column store per plane); thread t = tid - 64 owns
-    // stacked B row t when t < 16 S, written to shared memory in the canonical K-major layout.
-    const int t = tid - 64;
+  } else if (warp < 2 + OZ_CONV) {
+    // ---------------- converters: int8 chunks -> FP16.  A warp may reach only its quarter of the
+    // tensor-memory lanes, so thread (warp, lane) owns A row 32 (warp % 4) + lane, written to the chunk's A
+    // buffer in tensor memory (one 8-column store per plane); thread t of the group's 128 owns stacked B
+    // rows t, t + 128 below TN S, written to shared memory in the canonical K-major layout.
+    const int h = (warp - 2) >> 2, t = tid - 64 - 128 * h;  // the group's half of every stage
     const int row = 32 * (warp & 3) + lane;
     const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + OZ_TMEM_A;
-    bool ok = true;
-    for (int s = 0; s < nst && ok; ++s) {
+    for (int s = 0; s < nst; ++s) {
       const int slot = s % OZ_NST;
       if (!mbar_wait(b_full8 + 8 * slot, (s / OZ_NST) & 1, abort)) break;
-      const uint8_t* a8 = ring + slot * ST_BYTES;
+      const uint8_t* a8 = ring + slot * F::ST_BYTES;
       const uint8_t* b8 = a8 + ST_A;
-      for (int h = 0; h < 2; ++h) {
-        const int c = 2 * s + h, sbf = c % OZ_NBF;
-        if (!mbar_wait(b_emptybf + 8 * sbf, ((c / OZ_NBF) & 1) ^ 1, abort)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        uint8_t* bbf = bfb + sbf * BF_BYTES;
-        uint32_t w[OZ_S][4];
-        if (acol) {  // stage image [q][k 32][m 128]: 16 byte loads per plane
-#pragma unroll
-          for (int q = 0; q < OZ_S; ++q)
-            if (q < S) {
-              const uint8_t* p = a8 + q * (OZ_TM * OZ_KS) + (16 * h) * OZ_TM + row;
-#pragma unroll
-              for (int u = 0; u < 4; ++u)
-                w[q][u] = __byte_perm(
-                    __byte_perm((uint32_t)p[(4 * u) * OZ_TM], (uint32_t)p[(4 * u + 1) * OZ_TM], 0x0040u),
-                    __byte_perm((uint32_t)p[(4 * u + 2) * OZ_TM], (uint32_t)p[(4 * u + 3) * OZ_TM], 0x0040u), 0x5410u);
-            }
-        } else {  // stage image [q][half 2][m 128][16 k]: one contiguous 16-byte load per plane
-#pragma unroll
-          for (int q = 0; q < OZ_S; ++q)
-            if (q < S) {
-              const uint4 v = *reinterpret_cast<const uint4*>(a8 + q * (OZ_TM * OZ_KS) + h * (OZ_TM * 16) + row * 16);
-              w[q][0] = v.x;
-              w[q][1] = v.y;
-              w[q][2] = v.z;
-              w[q][3] = v.w;
-            }
-        }
-        const uint32_t ta = trow + sbf * OZ_A_COLS;
+      const int c = 2 * s + h, sbf = c % OZ_NBF;
+      if (!mbar_wait(b_emptybf + 8 * sbf, ((c / OZ_NBF) & 1) ^ 1, abort)) break;
+      tc_fence_after();
+      uint8_t* bbf = bfb + sbf * F::BF_BYTES;
+      uint32_t w[OZ_S][4];
+      if (acol) {  // stage image [q][k 32][m 128]: 16 byte loads per plane
 #pragma unroll
         for (int q = 0; q < OZ_S; ++q)
           if (q < S) {
-            uint32_t o[8];
-            oz_cvt16(w[q], o);
-            tmem_st8(ta + q * (OZ_KC / 2), o);
+            const uint8_t* p = a8 + q * (OZ_TM * OZ_KS) + (16 * h) * OZ_TM + row;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              w[q][u] = __byte_perm(
+                  __byte_perm((uint32_t)p[(4 * u) * OZ_TM], (uint32_t)p[(4 * u + 1) * OZ_TM], 0x0040u),
+                  __byte_perm((uint32_t)p[(4 * u + 2) * OZ_TM], (uint32_t)p[(4 * u + 3) * OZ_TM], 0x0040u), 0x5410u);
           }
-        if (t < OZ_TN * S) {  // B image [q][half 2][n 16][16 k] -> stacked row t
-          const uint4 v = *reinterpret_cast<const uint4*>(b8 + (t / OZ_TN) * (OZ_TN * OZ_KS) + h * (OZ_TN * 16) +
-                                                          (t % OZ_TN) * 16);
+      } else {  // stage image [q][half 2][m 128][16 k]: one contiguous 16-byte load per plane
+#pragma unroll
+        for (int q = 0; q < OZ_S; ++q)
+          if (q < S) {
+            const uint4 v = *reinterpret_cast<const uint4*>(a8 + q * (OZ_TM * OZ_KS) + h * (OZ_TM * 16) + row * 16);
+            w[q][0] = v.x;
+            w[q][1] = v.y;
+            w[q][2] = v.z;
+            w[q][3] = v.w;
+          }
+      }
+      const uint32_t ta = trow + sbf * OZ_A_COLS;
+#pragma unroll
+      for (int q = 0; q < OZ_S; ++q)
+        if (q < S) {
+          uint32_t o[8];
+          oz_cvt16(w[q], o);
+          tmem_st8(ta + q * (OZ_KC / 2), o);
+        }
+#pragma unroll
+      for (int r = t; r < TN * OZ_S; r += 128)
+        if (r < TN * S) {  // B image [q][half 2][n TN][16 k] -> stacked row r
+          const uint4 v = *reinterpret_cast<const uint4*>(b8 + (r / TN) * (TN * OZ_KS) + h * (TN * 16) + (r % TN) * 16);
           const uint32_t wb[4] = {v.x, v.y, v.z, v.w};
           uint32_t o[8];
           oz_cvt16(wb, o);
-          uint8_t* d = bbf + t * 16;
+          uint8_t* d = bbf + r * 16;
           *reinterpret_cast<uint4*>(d) = make_uint4(o[0], o[1], o[2], o[3]);
-          *reinterpret_cast<uint4*>(d + OZ_S * OZ_TN * 16) = make_uint4(o[4], o[5], o[6], o[7]);
+          *reinterpret_cast<uint4*>(d + OZ_S * TN * 16) = make_uint4(o[4], o[5], o[6], o[7]);
         }
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_fence_before();
-        mbar_arrive(b_fullbf + 8 * sbf);
-      }
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      tc_fence_before();
+      mbar_arrive(b_fullbf + 8 * sbf);
       mbar_arrive(b_empty8 + 8 * slot);
     }
   } else {
-    // ---------------- epilogue (warps 6-9): window drains, FP64 recombination, store
+    // ---------------- epilogue: window drains, FP64 recombination, store
     const int lq = warp & 3, row = 32 * lq + lane, m = m0 + row;
-    int tot[OZ_S][OZ_TN];
+    const int cb = 16 * ((warp - 2 - OZ_CONV) >> 2);  // this warp's first column of the tile
+    long long hi[16], lo[16];
 #pragma unroll
-    for (int g = 0; g < OZ_S; ++g)
-#pragma unroll
-      for (int c = 0; c < OZ_TN; ++c) tot[g][c] = 0;
+    for (int c = 0; c < 16; ++c) hi[c] = lo[c] = 0;
     bool ok = true;
-    for (int w = 0; w < nwin && ok; ++w) ok = oz_drain(w, S, b_accf, b_acce, tmem, lq, abort, tot);
-    // group g has weight 2^-7(g+2): hi = groups 0-3 and lo = groups 4-7, both below 2^53 (exact in
-    // 64-bit integers and in FP64); value = (hi 2^28 + lo) 2^-63 (one rounding)
-    long long hi[OZ_TN], lo[OZ_TN];
-#pragma unroll
-    for (int c = 0; c < OZ_TN; ++c) {
-      hi[c] = ((long long)tot[0][c] << 21) + ((long long)tot[1][c] << 14) + ((long long)tot[2][c] << 7) + tot[3][c];
-      lo[c] = ((long long)tot[4][c] << 21) + ((long long)tot[5][c] << 14) + ((long long)tot[6][c] << 7) + tot[7][c];
-    }
+    for (int w = 0; w < nwin && ok; ++w) ok = oz_drain<TN>(w, S, b_accf, b_acce, tmem, lq, cb, abort, hi, lo);
+    // group g has weight 2^-7(g+2); hi and lo are below 2^53 (exact in FP64): (hi 2^28 + lo) 2^-63, one rounding
     const int eA = *Jp->eA;
     double* Cp = Jp->C;
     const int ldc = Jp->ldc;
     const size_t MN = (size_t)M * N;
 #pragma unroll
-    for (int c = 0; c < OZ_TN; ++c) {
-      const int n = n0 + c;
+    for (int c = 0; c < 16; ++c) {
+      const int n = n0 + cb + c;
       if (m < M && n < N) {
         double v = fma((double)hi[c], 268435456.0, (double)lo[c]);
         v = ldexp(v, eA + Jp->eB[n * Jp->eB_stride] - 63);
@@ -594,16 +609,16 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_mma(const OzDev* __restric
     if (nsplit > 1) {
       // the last slice to finish this output block sums the partials in slice order
       __threadfence();
-      asm volatile("bar.sync 1, 128;" ::: "memory");
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * F::EPI) : "memory");
       __shared__ int last;
       int* ctr = Jp->ctr + (m0 / OZ_TM) * tiles_n + nt;
-      if (row == 0) last = (atomicAdd(ctr, 1) == nsplit - 1);
-      asm volatile("bar.sync 1, 128;" ::: "memory");
+      if (row == 0 && cb == 0) last = (atomicAdd(ctr, 1) == nsplit - 1);
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * F::EPI) : "memory");
       if (last) {
         __threadfence();
         if (m < M)
-          for (int c = 0; c < OZ_TN; ++c) {
-            const int n = n0 + c;
+          for (int c = 0; c < 16; ++c) {
+            const int n = n0 + cb + c;
             if (n >= N) break;
             const size_t o = m + (size_t)n * M;
             double v = 0.0;
@@ -611,7 +626,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_mma(const OzDev* __restric
             double* cp = Cp + m + (size_t)n * ldc;
             *cp = Jp->accumulate ? *cp + v : v;
           }
-        if (row == 0) *ctr = 0;
+        if (row == 0 && cb == 0) *ctr = 0;
       }
     }
   }
@@ -735,15 +750,17 @@ int oz_timeout_flag(tlr_ctx* ctx) {
   return v;
 }
 
-void oz_gemm(tlr_ctx* ctx, std::vector<OzJob>& jobs) {
+template <int TN>
+static void oz_launch(tlr_ctx* ctx, std::vector<OzJob>& jobs) {
   if (jobs.empty()) return;
   static bool attr = false;
   if (!attr) {
-    TLR_CUDA(cudaFuncSetAttribute(k_oz_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
+    TLR_CUDA(cudaFuncSetAttribute(k_oz_mma<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, OzForm<TN>::SMEM));
     attr = true;
   }
   // Split K per job (its shape only, so a product sums in the same order alone or in a batch):
-  // enough slices of at least eight 32-deep stages for the job alone to give ~1 CTA per SM.
+  // enough slices of at least eight 32-deep stages for the job alone to give ~1 CTA per SM of 16 columns (also
+  // in the wide form, so that the form changes no sum).
   int mx = 0, ny = 0;
   double flops = 0, bytes = 0;
   size_t ws_elems = 0, nctr = 0;
@@ -751,9 +768,9 @@ void oz_gemm(tlr_ctx* ctx, std::vector<OzJob>& jobs) {
     TLR_REQUIRE(j.K > 0 && j.K <= 16384 && j.M > 0 && j.N > 0 && j.S >= 1 && j.S <= OZ_S, TLR_ERR_LIMIT,
                 "split product: unsupported shape");
     const int tm = (int)oz_cdiv(j.M, OZ_TM);
-    j.tiles_n = (int)oz_cdiv(j.N, OZ_TN);
+    j.tiles_n = (int)oz_cdiv(j.N, TN);
     const int nst = (int)oz_cdiv(j.K, OZ_KS);
-    const int tnr = j.rule_n > 0 ? (int)oz_cdiv(j.rule_n, OZ_TN) : j.tiles_n;
+    const int tnr = (int)oz_cdiv(j.rule_n > 0 ? j.rule_n : j.N, OZ_TN);
     const int64_t want = ((int64_t)std::max(ctx->sm_count, 1) + (int64_t)tm * tnr - 1) / ((int64_t)tm * tnr);
     if (j.nsplit <= 0) j.nsplit = (int)std::max<int64_t>(1, std::min<int64_t>({want, nst / 8, 64}));
     mx = std::max(mx, j.M);
@@ -785,7 +802,7 @@ void oz_gemm(tlr_ctx* ctx, std::vector<OzJob>& jobs) {
       map_kmajor(&d.ta, j.A, (uint64_t)j.K, (uint64_t)j.M, (uint64_t)j.lda, j.sA, OZ_TM);
     }
     d.K0 = j.K0;
-    map_kmajor(&d.tb, j.B, (uint64_t)j.K, (uint64_t)j.N, (uint64_t)ldb, j.sB, OZ_TN);
+    map_kmajor(&d.tb, j.B, (uint64_t)j.K, (uint64_t)j.N, (uint64_t)ldb, j.sB, TN);
     d.eA = j.eA;
     d.eB = j.eB;
     d.C = j.C;
@@ -815,10 +832,18 @@ void oz_gemm(tlr_ctx* ctx, std::vector<OzJob>& jobs) {
     dim3 grid((unsigned)oz_cdiv(mx, OZ_TM), (unsigned)ny, (unsigned)cnt);
     ctx->site_next_flops = flops * cnt / jobs.size();
     TLR_SITE_PRE(ctx);
-    k_oz_mma<<<grid, OZ_THREADS, OZ_SMEM, ctx->stream>>>(dj);
+    k_oz_mma<TN><<<grid, OzForm<TN>::THREADS, OzForm<TN>::SMEM, ctx->stream>>>(dj);
     TLR_LAUNCH_CHECK(ctx);
     if (ctx->kprof) kprof_end(ctx, 6, flops * cnt / jobs.size(), bytes * cnt / jobs.size());
   }
+}
+
+void oz_gemm(tlr_ctx* ctx, std::vector<OzJob>& jobs) {
+  // products of more than 16 columns in the wide form, a launch of its own
+  std::vector<OzJob> form[2];
+  for (auto& j : jobs) form[j.N > OZ_TN && j.tol <= 0.0 ? 1 : 0].push_back(j);
+  oz_launch<OZ_TN>(ctx, form[0]);
+  oz_launch<2 * OZ_TN>(ctx, form[1]);
 }
 
 }  // namespace tlr
