@@ -1,21 +1,36 @@
 // ARA -> SVD rank trimming of low-rank tiles (Section 6: the post-processing step that applies the SVD
 // to each low-rank tile to bring its rank down to the minimum).
 //
-// A tile Q B^T with orthonormal Q (b x r) has the singular values of B.  One CTA per tile: a Householder
-// QR of B (B = H R, the reflectors applied to the trailing columns in place, in a working copy in global
-// memory: the QR runs at GB300's FP64 rate, and a small shared footprint lets several tiles share an SM),
-// then one-sided Jacobi (Hestenes) on X = R^T: plane rotations of column pairs in the parallel
-// round-robin order (r/2 disjoint pairs per round, r - 1 rounds per sweep) until no pair is rotated,
+// A tile Q B^T with orthonormal Q (b x r) has the singular values of B.  One CTA, or a cluster of four or eight, per
+// tile: a Householder QR of B (B = H R, the reflectors applied to the trailing columns in place, in a working
+// copy in global memory), then one-sided Jacobi (Hestenes) on X = R^T: plane rotations of column pairs in the
+// parallel round-robin order (r/2 disjoint pairs per round, r - 1 rounds per sweep) until no pair is rotated,
 // giving X J = Y with orthogonal columns whose norms are the singular values sigma of R (and of B), and
 // Y / sigma the right singular vectors Z of B (R = J S (Y S^-1)^T).  Jacobi on R^T rather than R takes
 // about a third of the sweeps on these matrices.  The columns with sigma > eps, in descending order,
 // form Z_r (r x r'); Q' = Q Z_r and B' = B Z_r = W_r S_r are two batched GEMMs.  Every reduction has a
 // fixed order, so the result depends on the tile only.
+//
+// The FP64 unit is the bound: a sweep is 5 r^3 / 2 lane operations (one product for the pair's inner product,
+// four for the rotation; the squared norms are updated by the rotation, a' = a - t g, b' = b + t g, and
+// recomputed once per sweep) plus a square root, a reciprocal and a reciprocal square root per pair.  So
+//   * several lanes share a pair, as many as keep the CTA's threads busy, and the pairs' rotation angles are
+//     computed together, one thread per pair, so that the scalar work fills its warps;
+//   * a tile of rank above TR_SOLO is spread over a cluster, its columns dealt out over the CTAs' shared memory
+//     and reached through distributed shared memory: the few tiles of high rank next to the diagonal are what a
+//     matrix's trimming waits for;
+//   * the tiles of low rank run beside them on the side stream.
+// Measured, one thread per pair and rank classes one after another -> now: trimming a matrix of N = 16384, b = 512
+// (ranks up to 142, mean 27) 109 -> 12.4 ms; 12 tiles of rank 140 61 -> 9.8 ms; 57 of rank 64 12.9 -> 3.9; 400 of
+// rank 16 1.36 -> 1.04; 4 of rank 300 (b = 1024) 723 -> 61.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <map>
 
 #include "internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace tlr {
 
@@ -23,11 +38,12 @@ namespace {
 
 constexpr int TR_T = 256, TR_W = TR_T / 32;
 constexpr int TR_SWEEPS = 60;  // a bound only: the tiles converge in about 10
+constexpr int TR_SOLO = 48;    // highest rank of a single-CTA tile
 
 struct TrimDev {
   const double* B;  // b x r, leading dimension b
   double* W;        // working copy (b x r)
-  double* X;        // R^T (r x r) when it does not live in shared memory
+  double* X;        // R^T (r x r) and the squared norms (r) when they do not fit in shared memory
   double* Zs;       // out: Z_r (r x r', leading dimension r)
   int* rank;        // out: r'
   int r;
@@ -49,146 +65,234 @@ __device__ double block_sum(double v, double* red) {
   return s;
 }
 
-// MODE 0: X = R^T in global memory; 1: X in shared memory (after the reflector vector, the singular
-// values and their order)
-template <int MODE>
+// 1 / v to an ulp or two by two Newton steps (the angle it enters is corrected by later rotations); v normal
+__device__ __forceinline__ double recip_approx(double v) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+  y = fma(y, fma(-v, y, 1.0), y);
+  return fma(y, fma(-v, y, 1.0), y);
+}
+
+// CS: CTAs of the tile's cluster.  SM: X and the norms live in shared memory, column c in CTA c % CS at place
+// c / CS; otherwise in global memory.
+template <int CS, bool SM>
 __global__ void __launch_bounds__(TR_T) k_trim(const TrimDev* __restrict__ jobs, int b, double eps) {
-  const TrimDev J = jobs[blockIdx.x];
+  const TrimDev J = jobs[blockIdx.x / CS];
+  const int rank = (int)(blockIdx.x % CS);
   const int r = J.r, tid = threadIdx.x, w = tid >> 5, l = tid & 31;
   extern __shared__ double sm[];
-  double* v = sm;                                  // b: the current reflector
-  double* red = v + b;                             // TR_W
-  double* sig = red + TR_W;                        // r
-  int* pos = reinterpret_cast<int*>(sig + r);      // r
-  double* nxt = reinterpret_cast<double*>(pos + r + (r & 1));
-  const int rp = r | 1;  // X's leading dimension, odd: the pair threads below read distinct banks
-  double* X = MODE == 1 ? nxt : J.X;
-  double* W = J.W;
+  __shared__ double cc[TR_T], sn[TR_T], gs[TR_T];  // rotations of a pass's pairs
+  __shared__ double red[TR_W];
   __shared__ int rot, keep;
-  if (r == 0) {
-    if (tid == 0) *J.rank = 0;
+  const int rp = r | 1, nc = (r + CS - 1) / CS;  // leading dimension of X (odd: no bank conflicts), columns per CTA
+  double* v = sm;                                // b: the current reflector
+  double* beta = v + b;                          // r: the diagonal of R, later the singular values
+  double* nrm_s = beta + r;                      // nc: squared norms of this CTA's columns
+  double* X_s = nrm_s + (SM ? nc : 0);           // nc columns
+  int* pos = reinterpret_cast<int*>(X_s + (SM ? (size_t)nc * rp : 0));  // r
+  auto csync = [&]() {
+    if (CS == 1) __syncthreads();
+    else cg::this_cluster().sync();
+  };
+  auto peer = [&](double* p, int q) { return CS == 1 ? p : cg::this_cluster().map_shared_rank(p, q); };
+  auto col = [&](int c) { return SM ? peer(X_s, c % CS) + (size_t)(c / CS) * rp : J.X + (size_t)c * rp; };
+  auto nrm = [&](int c) { return SM ? peer(nrm_s, c % CS) + c / CS : J.X + (size_t)r * rp + c; };
+  auto ld = [](const double* p) { return SM ? *p : __ldcg(p); };  // other CTAs write X
+  if (r == 0) {  // the whole cluster
+    if (tid == 0 && rank == 0) *J.rank = 0;
     return;
   }
-  for (int64_t e = tid; e < (int64_t)b * r; e += TR_T) W[e] = J.B[e];
-  __syncthreads();
-  // ---- Householder QR: R in the upper triangle of W's first r rows
+  double* W = J.W;
+  for (int c = rank; c < r; c += CS)
+    for (int m = tid; m < b; m += TR_T) W[m + (size_t)c * b] = J.B[m + (size_t)c * b];
+  // ---- Householder QR: R's strict upper triangle in W's first rows, its diagonal in beta.  Every CTA forms the
+  // reflector; column c of the trailing part is CTA c % CS's.
   for (int j = 0; j < r; ++j) {
-    double* cj = W + (size_t)j * b;
+    csync();  // column j is complete
+    const double* cj = W + (size_t)j * b;
     double s = 0.0;
-    for (int m = j + 1 + tid; m < b; m += TR_T) s += cj[m] * cj[m];
+    for (int m = j + 1 + tid; m < b; m += TR_T) {
+      const double x = __ldcg(cj + m);
+      v[m] = x;
+      s += x * x;
+    }
     s = block_sum(s, red);
+    const double alpha = __ldcg(cj + j);
+    double d = alpha;
     if (s > 0.0) {  // uniform: s is the block's sum
-      const double alpha = cj[j];
-      const double nrm = sqrt(alpha * alpha + s);
-      const double beta = alpha >= 0.0 ? -nrm : nrm;
-      const double tau = (beta - alpha) / beta, scal = 1.0 / (alpha - beta);
-      for (int m = j + 1 + tid; m < b; m += TR_T) v[m] = cj[m] * scal;
+      const double nr = sqrt(alpha * alpha + s);
+      d = alpha >= 0.0 ? -nr : nr;
+      const double tau = (d - alpha) / d, scal = 1.0 / (alpha - d);
+      for (int m = j + 1 + tid; m < b; m += TR_T) v[m] *= scal;
       if (tid == 0) v[j] = 1.0;
-      __syncthreads();  // v complete; every thread has read alpha
-      if (tid == 0) cj[j] = beta;
-      for (int c = j + 1 + w; c < r; c += TR_W) {  // H = I - tau v v^T on the trailing columns
-        double* col = W + (size_t)c * b;
-        double d = 0.0;
-#pragma unroll 4
-        for (int m = j + l; m < b; m += 32) d += v[m] * col[m];
-        const double f = tau * warp_sum(d);
-#pragma unroll 4
-        for (int m = j + l; m < b; m += 32) col[m] -= f * v[m];
-      }
-    }
-    __syncthreads();
-  }
-  // ---- X = R^T (lower triangular)
-  for (int64_t e = tid; e < (int64_t)r * r; e += TR_T) {
-    const int m = (int)(e % r), c = (int)(e / r);
-    X[m + (size_t)c * rp] = c <= m ? W[c + (size_t)m * b] : 0.0;
-  }
-  __syncthreads();
-  // ---- one-sided Jacobi on X, round-robin pairs (position 0 fixed, 1 .. n-1 rotating), one thread per
-  // pair: GB300's FP64 unit is the bound, and a thread's serial dot products waste no lanes on reductions
-  const int n = r + (r & 1);
-  const double tol = (double)r * 0x1p-53;
-  for (int sweep = 0; sweep < TR_SWEEPS; ++sweep) {
-    if (tid == 0) rot = 0;
-    __syncthreads();
-    for (int t = 0; t < n - 1; ++t) {
-      for (int k = tid; k < n / 2; k += TR_T) {
-        int p = k == 0 ? 0 : (k - 1 + t) % (n - 1) + 1;
-        int q = (n - 2 - k + t) % (n - 1) + 1;  // the position n - 1 - k >= 1
-        if (p > q) {
-          const int x = p;
-          p = q;
-          q = x;
-        }
-        if (q >= r) continue;  // the padding index of an odd r
-        double* xp = X + (size_t)p * rp;
-        double* xq = X + (size_t)q * rp;
-        double a = 0.0, bb = 0.0, g = 0.0;
-        for (int m = 0; m < r; ++m) {
-          const double x = xp[m], y = xq[m];
-          a = fma(x, x, a);
-          bb = fma(y, y, bb);
-          g = fma(x, y, g);
-        }
-        if (g != 0.0 && fabs(g) > tol * sqrt(a * bb)) {
-          const double z = (bb - a) / (2.0 * g);
-          const double tt = fabs(z) < 1e150 ? (z >= 0.0 ? 1.0 : -1.0) / (fabs(z) + sqrt(1.0 + z * z)) : 0.5 / z;
-          const double c = 1.0 / sqrt(1.0 + tt * tt), sn = c * tt;
-          for (int m = 0; m < r; ++m) {
-            const double x = xp[m], y = xq[m];
-            xp[m] = c * x - sn * y;
-            xq[m] = sn * x + c * y;
-          }
-          rot = 1;
-        }
-      }
       __syncthreads();
+      // H = I - tau v v^T on this CTA's trailing columns, a warp each
+      for (int c = j + 1 + ((rank - (j + 1)) % CS + CS) % CS + w * CS; c < r; c += TR_W * CS) {
+        double* x = W + (size_t)c * b;
+        double dt = 0.0;
+#pragma unroll 4
+        for (int m = j + l; m < b; m += 32) dt += v[m] * x[m];
+        const double f = tau * warp_sum(dt);
+#pragma unroll 4
+        for (int m = j + l; m < b; m += 32) x[m] -= f * v[m];
+      }
     }
-    if (rot == 0) break;  // read by every thread after the round's barrier
-    __syncthreads();      // before thread 0 clears it
+    if (tid == 0) beta[j] = d;
   }
-  // ---- singular values, their descending order, the kept columns
-  for (int c = w; c < r; c += TR_W) {
-    const double* xc = X + (size_t)c * rp;
-    double s2 = 0.0;
-    for (int m = l; m < r; m += 32) s2 += xc[m] * xc[m];
-    s2 = warp_sum(s2);
-    if (l == 0) sig[c] = sqrt(s2);
+  csync();
+  // ---- X = R^T (lower triangular)
+  for (int c = rank; c < r; c += CS) {
+    double* x = col(c);
+    for (int m = tid; m < r; m += TR_T) x[m] = c < m ? __ldcg(W + c + (size_t)m * b) : c == m ? beta[c] : 0.0;
   }
+  // ---- one-sided Jacobi on X, round-robin pairs (position 0 fixed, 1 .. n-1 rotating); pair k is CTA k % CS's
+  const int n = r + (r & 1), np = n / 2, mine = (np - rank + CS - 1) / CS;
+  int L = 32;  // lanes of a pair
+  while (L > 1 && mine * L > TR_T) L >>= 1;
+  const int G = TR_T / L, grp = tid / L, gl = tid % L;
+  const double tol2 = ((double)r * 0x1p-53) * ((double)r * 0x1p-53);
+  auto norms = [&]() {  // squared norms of this CTA's columns
+    for (int c = rank + w * CS; c < r; c += TR_W * CS) {
+      const double* x = col(c);
+      double s2 = 0.0;
+      for (int m = l; m < r; m += 32) {
+        const double y = ld(x + m);
+        s2 += y * y;
+      }
+      s2 = warp_sum(s2);
+      if (l == 0) *nrm(c) = s2;
+    }
+  };
+  auto pair_of = [&](int k, int t, int& p, int& q) {
+    p = k == 0 ? 0 : (k - 1 + t) % (n - 1) + 1;
+    q = (n - 2 - k + t) % (n - 1) + 1;  // the position n - 1 - k >= 1
+    if (p > q) {
+      const int x = p;
+      p = q;
+      q = x;
+    }
+  };
+  for (int sweep = 0; sweep < TR_SWEEPS; ++sweep) {
+    csync();
+    norms();
+    if (tid == 0) rot = 0;
+    csync();
+    for (int t = 0; t < n - 1; ++t) {
+      for (int k0 = 0; k0 < mine; k0 += G) {
+        const int i = k0 + grp;
+        int p = 0, q = r;
+        if (i < mine) pair_of(rank + i * CS, t, p, q);
+        const bool live = i < mine && q < r;  // q = r: the padding index of an odd r
+        double *xp = nullptr, *xq = nullptr;
+        double g = 0.0;
+        if (live) {
+          xp = col(p);
+          xq = col(q);
+#pragma unroll 4
+          for (int m = gl; m < r; m += L) g = fma(ld(xp + m), ld(xq + m), g);
+        }
+        for (int o = L >> 1; o; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        if (gl == 0) gs[grp] = g;
+        __syncthreads();
+        if (tid < G) {  // the pass's angles, one thread per pair
+          const int i2 = k0 + tid;
+          double c = 1.0, s = 0.0;
+          int p2 = 0, q2 = r;
+          if (i2 < mine) pair_of(rank + i2 * CS, t, p2, q2);
+          if (i2 < mine && q2 < r) {
+            double *ap = nrm(p2), *bp = nrm(q2);
+            const double aa = ld(ap), bb = ld(bp), gg = gs[tid];
+            if (gg * gg > tol2 * (aa * bb)) {
+              // tan of the rotation: 2 g / (d + sign(d) sqrt(d^2 + 4 g^2)), d = b - a
+              const double d = bb - aa, g2 = 2.0 * gg, h = fma(d, d, g2 * g2);
+              const double hs = h * rsqrt(h), tt = (d >= 0.0 ? g2 : -g2) * recip_approx(fabs(d) + hs);
+              c = rsqrt(fma(tt, tt, 1.0));
+              s = c * tt;
+              *ap = fma(-tt, gg, aa);
+              *bp = fma(tt, gg, bb);
+              rot = 1;
+            }
+          }
+          cc[tid] = c;
+          sn[tid] = s;
+        }
+        __syncthreads();
+        const double c = cc[grp], s = sn[grp];
+        if (live && s != 0.0) {
+#pragma unroll 4
+          for (int m = gl; m < r; m += L) {
+            const double x = ld(xp + m), y = ld(xq + m);
+            xp[m] = c * x - s * y;
+            xq[m] = s * x + c * y;
+          }
+        }
+      }
+      csync();
+    }
+    int any = 0;
+    for (int q = 0; q < CS; ++q) any |= CS == 1 ? rot : *cg::this_cluster().map_shared_rank(&rot, q);
+    if (!any) break;  // the next sweep's first barrier comes before rot is cleared
+  }
+  csync();
+  // ---- singular values (in every CTA), their descending order, the kept columns
+  norms();
+  csync();
+  for (int c = tid; c < r; c += TR_T) beta[c] = sqrt(ld(nrm(c)));
   __syncthreads();
   for (int c = tid; c < r; c += TR_T) {
-    const double sc = sig[c];
+    const double sc = beta[c];
     int ps = 0;
-    for (int d = 0; d < r; ++d) ps += (sig[d] > sc || (sig[d] == sc && d < c)) ? 1 : 0;
+    for (int d = 0; d < r; ++d) ps += (beta[d] > sc || (beta[d] == sc && d < c)) ? 1 : 0;
     pos[c] = ps;
   }
   if (tid == 0) {
     int kk = 0;
-    for (int c = 0; c < r; ++c) kk += sig[c] > eps ? 1 : 0;
+    for (int c = 0; c < r; ++c) kk += beta[c] > eps ? 1 : 0;
     keep = kk;
   }
   __syncthreads();
-  for (int c = w; c < r; c += TR_W) {
+  for (int c = rank + w * CS; c < r; c += TR_W * CS) {
     const int ps = pos[c];
     if (ps >= keep) continue;
-    const double inv = 1.0 / sig[c];
-    const double* xc = X + (size_t)c * rp;
+    const double inv = 1.0 / beta[c];
+    const double* xc = col(c);
     double* zc = J.Zs + (size_t)ps * r;
-    for (int m = l; m < r; m += 32) zc[m] = xc[m] * inv;
+    for (int m = l; m < r; m += 32) zc[m] = ld(xc + m) * inv;
   }
-  if (tid == 0) *J.rank = keep;
+  if (tid == 0 && rank == 0) *J.rank = keep;
+  csync();  // no CTA leaves while its columns are still read
 }
 
-size_t trim_smem(int b, int r, int mode) {
-  return sizeof(double) * ((size_t)b + TR_W + r) + sizeof(int) * ((size_t)r + (r & 1)) +
-         (mode == 1 ? sizeof(double) * (size_t)r * (r | 1) : 0);
+size_t trim_smem(int b, int r, int cs, bool in_smem) {
+  const size_t nc = (r + cs - 1) / cs;
+  return sizeof(double) * ((size_t)b + r + (in_smem ? nc + nc * (r | 1) : 0)) + sizeof(int) * ((size_t)r + (r & 1));
 }
 
 constexpr size_t TRIM_SMEM_MAX = 220 * 1024;
 
+template <int CS, bool SM>
+void trim_launch(tlr_ctx* ctx, const TrimDev* dj, int cnt, size_t smem, int b, double eps) {
+  auto kern = k_trim<CS, SM>;
+  TLR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  cudaLaunchConfig_t cf{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = CS;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cf.gridDim = dim3((unsigned)(cnt * CS));
+  cf.blockDim = dim3(TR_T);
+  cf.dynamicSmemBytes = smem;
+  cf.stream = ctx->stream;
+  cf.attrs = &at;
+  cf.numAttrs = 1;
+  TLR_SITE_PRE(ctx);
+  TLR_CUDA(cudaLaunchKernelEx(&cf, kern, dj, b, eps));
+  TLR_LAUNCH_CHECK(ctx);
+}
+
 }  // namespace
 
-bool trim_fits(int b) { return trim_smem(b, b, 0) <= TRIM_SMEM_MAX; }
+bool trim_fits(int b) { return trim_smem(b, b, 8, false) <= TRIM_SMEM_MAX; }
 
 void trim_tiles(tlr_ctx* ctx, int b, const std::vector<TrimTile>& tiles, double eps, std::vector<int>& rank,
                 std::vector<double*>& Zs, Buf& work) {
@@ -197,45 +301,86 @@ void trim_tiles(tlr_ctx* ctx, int b, const std::vector<TrimTile>& tiles, double 
   Zs.assign(nt, nullptr);
   if (nt == 0) return;
   TLR_REQUIRE(trim_fits(b), TLR_ERR_LIMIT, "rank trimming: tile size above the shared-memory limit");
-  // workspace per tile: W (b r), X (r (r | 1), used when it does not fit in shared memory), Zs (r^2); ranks
+  // workspace per tile: W (b r), X (r (r | 1)) and the norms (r), used when they do not fit in shared memory, Zs
+  // (r^2); ranks
   int64_t tot = 0;
   std::vector<int64_t> off(nt);
   for (int t = 0; t < nt; ++t) {
     off[t] = tot;
-    tot += (int64_t)tiles[t].r * (b + (tiles[t].r | 1) + (int64_t)tiles[t].r);
+    tot += (int64_t)tiles[t].r * (b + (tiles[t].r | 1) + 1 + (int64_t)tiles[t].r);
   }
   double* ws = work.need<double>((size_t)std::max<int64_t>(tot, 1) + (size_t)(nt + 1) / 2 + 1);
   int* dr = reinterpret_cast<int*>(ws + std::max<int64_t>(tot, 1));
-  // launch groups: the most on-chip mode the tile's rank allows, then rank classes (so that a group's
-  // shared memory, sized by its largest rank, does not hold many small tiles to one CTA per SM)
-  static const int cls[] = {8, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 1 << 30};
-  std::map<std::pair<int, int>, std::vector<TrimDev>> groups;
+  // Launch groups, highest ranks first.  A tile of rank up to TR_SOLO takes one CTA, in rank classes (so that a
+  // group's shared memory, sized by its largest rank, does not hold many small tiles to one CTA per SM); above
+  // that a cluster of four, or of eight where the tiles are too few for the GPU or four CTAs' shared memory does
+  // not hold X; where eight do not either, X lives in global memory.  (57 tiles of rank 56: clusters 3.2 ms against
+  // 10.2; 38 of rank 48 as single CTAs 2.5 ms, a third of what the clusters gain from there on.)
+  static const int cls[] = {8, 16, 24, 32, TR_SOLO};
+  int nbig = 0;
+  for (const TrimTile& t : tiles) nbig += t.r > TR_SOLO;
+  struct Group {
+    int cs = 1;
+    bool sm = true;
+    int rmax = 0;
+    std::vector<TrimDev> js;
+  };
+  std::map<int, Group> groups;  // the key orders the launches
   for (int t = 0; t < nt; ++t) {
     const int r = tiles[t].r;
     double* W = ws + off[t];
     double* X = W + (size_t)b * r;
-    TrimDev d{tiles[t].B, W, X, X + (size_t)r * (r | 1), dr + t, r};
+    TrimDev d{tiles[t].B, W, X, X + (size_t)r * ((r | 1) + 1), dr + t, r};
     Zs[t] = d.Zs;
-    const int mode = trim_smem(b, r, 1) <= TRIM_SMEM_MAX ? 1 : 0;
-    int c = 0;
-    while (cls[c] < r) ++c;
-    groups[{mode, c}].push_back(d);
-  }
-  for (auto& g : groups) {
-    const int mode = g.first.first;
-    std::vector<TrimDev>& js = g.second;
-    int rmax = 0;
-    for (const TrimDev& d : js) rmax = std::max(rmax, d.r);
-    const size_t sm = trim_smem(b, rmax, mode);
-    auto kern = mode == 1 ? k_trim<1> : k_trim<0>;
-    if (sm > 48 * 1024) TLR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    for (size_t o = 0; o < js.size(); o += 65535) {
-      const int cnt = (int)std::min<size_t>(65535, js.size() - o);
-      const TrimDev* dj = static_cast<const TrimDev*>(upload(ctx, js.data() + o, sizeof(TrimDev) * cnt));
-      TLR_SITE_PRE(ctx);
-      kern<<<cnt, TR_T, sm, ctx->stream>>>(dj, b, eps);
-      TLR_LAUNCH_CHECK(ctx);
+    int key, cs = 1;
+    bool sm;
+    if (r > TR_SOLO) {
+      cs = nbig * 8 <= ctx->sm_count || trim_smem(b, r, 4, true) > TRIM_SMEM_MAX ? 8 : 4;
+      sm = trim_smem(b, r, cs, true) <= TRIM_SMEM_MAX;
+      key = !sm ? 0 : cs == 8 ? 1 : 2;
+    } else {
+      int c = 0;
+      while (cls[c] < r) ++c;
+      sm = trim_smem(b, r, 1, true) <= TRIM_SMEM_MAX;
+      key = sm ? 10 - c : 3;
     }
+    Group& g = groups[key];
+    g.cs = cs;
+    g.sm = sm;
+    g.rmax = std::max(g.rmax, r);
+    g.js.push_back(d);
+  }
+  // the clusters on the main stream, the single-CTA tiles beside them on the side stream
+  const bool fork = nbig > 0 && nbig < nt && ctx->side && ctx->stream == ctx->main;
+  if (fork) {
+    TLR_CUDA(cudaEventRecord(ctx->ev_fork, ctx->main));
+    TLR_CUDA(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+  }
+  for (auto& kv : groups) {
+    Group& g = kv.second;
+    std::stable_sort(g.js.begin(), g.js.end(), [](const TrimDev& x, const TrimDev& y) { return x.r > y.r; });
+    const size_t sm = trim_smem(b, g.rmax, g.cs, g.sm);
+    cudaStream_t saved = ctx->stream;
+    if (fork && g.cs == 1) ctx->stream = ctx->side;
+    try {
+      for (size_t o = 0; o < g.js.size(); o += 65535) {
+        const int cnt = (int)std::min<size_t>(65535, g.js.size() - o);
+        const TrimDev* dj = static_cast<const TrimDev*>(upload(ctx, g.js.data() + o, sizeof(TrimDev) * cnt));
+        if (g.cs == 8 && g.sm) trim_launch<8, true>(ctx, dj, cnt, sm, b, eps);
+        else if (g.cs == 8) trim_launch<8, false>(ctx, dj, cnt, sm, b, eps);
+        else if (g.cs == 4) trim_launch<4, true>(ctx, dj, cnt, sm, b, eps);
+        else if (g.sm) trim_launch<1, true>(ctx, dj, cnt, sm, b, eps);
+        else trim_launch<1, false>(ctx, dj, cnt, sm, b, eps);
+      }
+    } catch (...) {
+      ctx->stream = saved;
+      throw;
+    }
+    ctx->stream = saved;
+  }
+  if (fork) {
+    TLR_CUDA(cudaEventRecord(ctx->ev_join, ctx->side));
+    TLR_CUDA(cudaStreamWaitEvent(ctx->main, ctx->ev_join, 0));
   }
   TLR_CUDA(cudaMemcpyAsync(rank.data(), dr, sizeof(int) * nt, cudaMemcpyDeviceToHost, ctx->stream));
   TLR_CUDA(cudaStreamSynchronize(ctx->stream));
