@@ -51,6 +51,14 @@ __device__ __forceinline__ void cholqr_warp(const double* G, double* M, int* st,
   } else {
     n = nk_in;
     thr2 = 0.0;
+    if (n <= 0) {  // nothing kept by the first pass, or converged there
+      if (lane < BS) {
+#pragma unroll
+        for (int r = 0; r < BS; ++r) M[r + lane * BS] = 0.0;
+      }
+      if (lane == 0) st[1] = 0;
+      return;
+    }
   }
   double rt[BS];      // rt[j] = Rt(j, lane)
   double inv[BS];     // 1 / Rt(j, j), the same in every lane

@@ -64,6 +64,7 @@ struct GemmJob {
   int rule_n;    // columns the split-K rule assumes (0: N), so that a product formed for several
                  // right-hand blocks at once sums every element as the one-block product does
   double alpha, beta;
+  const int* skip;  // device: the job does nothing when *skip != 0 (null: always runs)
 };
 enum { GEMM_TRIL = 1, GEMM_ALOWER = 2 };
 enum GemmMode { NN = 0, TN = 1, NT = 2 };

@@ -65,7 +65,8 @@ struct Sampler {
   // true: the sampler draws its own Gaussian blocks (one per matrix of the batch)
   virtual bool owns_omega() const { return false; }
   // Y[s] = T_{ops[s]} [Omega_t .. Omega_(t + m[s] - 1)], t = ts[s], written to Ydst[s] (n_op x bs m[s], leading
-  // dimension n_op).  A sampler that takes its Gaussian blocks from the engine gets m = 1 and one t per call.
+  // dimension n_op).  A sampler that takes its Gaussian blocks from the engine gets one t per call and the blocks of
+  // all its rounds, one after another.
   virtual void sample(const std::vector<int>& ops, const std::vector<int>& ts, const std::vector<int>& m,
                       const double* Om, const std::vector<double*>& Ydst) = 0;
   // rounds worth sampling at once for an operand about to sample round t while ns operands are active; a sample

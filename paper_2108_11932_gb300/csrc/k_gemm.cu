@@ -52,6 +52,7 @@ __device__ __forceinline__ void gemm_body(const GemmJob<T>* __restrict__ jobs, i
     J = jobs[lo];
   }
   __syncthreads();
+  if (J.skip && __ldcg(J.skip) != 0) return;
   int local = blockIdx.x - J.tile0;
   const int split = local % J.nsplit;
   local /= J.nsplit;

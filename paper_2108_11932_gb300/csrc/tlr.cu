@@ -477,7 +477,7 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
         Ahead& h = have[op];
         if (h.next < h.m) continue;
         h.next = 0;
-        h.m = std::max(1, Om ? 1 : S.ahead(op, round[op], ns));
+        h.m = std::max(1, S.ahead(op, round[op], ns));
         h.Y = take(h.m);
         ops.push_back(op);
         ts.push_back(round[op]);
@@ -491,15 +491,21 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
         std::sort(rounds_present.begin(), rounds_present.end());
         rounds_present.erase(std::unique(rounds_present.begin(), rounds_present.end()), rounds_present.end());
         for (int t : rounds_present) {
-          std::vector<int> ops_t;
+          std::vector<int> ops_t, m_t;
           std::vector<double*> y_t;
+          int mt = 1;
           for (size_t s = 0; s < ops.size(); ++s)
             if (ts[s] == t) {
               ops_t.push_back(ops[s]);
+              m_t.push_back(ms[s]);
               y_t.push_back(ydst[s]);
+              mt = std::max(mt, ms[s]);
             }
-          omega(ctx, cf.seed, cf.stream, cf.k, (uint32_t)t, nrow[ops_t[0]], bs, Om);
-          S.sample(ops_t, std::vector<int>(ops_t.size(), t), std::vector<int>(ops_t.size(), 1), Om, y_t);
+          const int n = nrow[ops_t[0]];  // operands of one size
+          Om = bOm.need<double>((size_t)nmax * bs * mt);
+          for (int u = 0; u < mt; ++u)
+            omega(ctx, cf.seed, cf.stream, cf.k, (uint32_t)(t + u), n, bs, Om + (size_t)u * n * bs);
+          S.sample(ops_t, std::vector<int>(ops_t.size(), t), m_t, Om, y_t);
         }
       }
     }
@@ -552,6 +558,7 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
         const int n = nrow[active[s]];
         j4.push_back(job<double>(NN, n, bs, Y[s], n, M + (size_t)s * bs * bs, bs, bs,
                                  W + (size_t)s * nmax * bs, n, 1.0, 0.0));
+        j4.back().skip = status + 2 * s;  // a slot that has converged needs none of the rest of the round
       }
       gemm<double>(ctx, NN, j4);
     }
@@ -566,8 +573,10 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
         if (q[op] > 0) {
           j1.push_back(job<double>(TN, q[op], bs, Qo, n, Ws, n, n, Ss, q[op], 1.0, 0.0));
           j2.push_back(job<double>(NN, n, bs, Qo, n, Ss, q[op], q[op], Ws, n, -1.0, 1.0));
+          j1.back().skip = j2.back().skip = status + 2 * s;
         }
         j3.push_back(job<double>(TN, bs, bs, Ws, n, Ws, n, n, G + (size_t)s * bs * bs, bs, 1.0, 0.0));
+        j3.back().skip = status + 2 * s;
         st.flops += 4.0 * n * q[op] * bs + 2.0 * n * bs * bs * 2;
       }
       gemm<double>(ctx, TN, j1);
@@ -578,6 +587,7 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
         const int op = active[s], n = nrow[op];
         j4.push_back(job<double>(NN, n, bs, W + (size_t)s * nmax * bs, n, M + (size_t)s * bs * bs, bs, bs,
                                  Q + qoff[op] + (size_t)q[op] * n, n, 1.0, 0.0));
+        j4.back().skip = status + 2 * s;
       }
       gemm<double>(ctx, NN, j4);
     }
@@ -627,24 +637,34 @@ struct DenseSampler : Sampler {
   double* B;        // nops x n x n (first q columns used)
   const OzTiles* oz = nullptr;
   double flops = 0;
-  void sample(const std::vector<int>& ops, const std::vector<int>&, const std::vector<int>&, const double* Om,
+  // Rounds formed in one product of 32 columns, which costs what 16 do (k_oz_mma): every tile but those of rank 0
+  // needs a second round to see that its first sufficed.  Truncated products keep their 16-column blocks.
+  // (With the skipped slots of ara_run: likelihood 2D N = 131072 1.436 -> 1.377 s, 3D N = 30011 118.7 -> 109.0 ms.)
+  int ahead(int, int t, int) override {
+    if (!oz || oz->thr8 > 0.0) return 1;
+    return std::max(t == 0 ? 2 : 1, 32 / bs);
+  }
+  // Om: n x bs blocks of the rounds, one after another
+  void sample(const std::vector<int>& ops, const std::vector<int>&, const std::vector<int>& ms, const double* Om,
               const std::vector<double*>& Ydst) override {
-    flops += 2.0 * n * n * bs * ops.size();
     if (oz) {
-      int8_t* Xs = oz->bx->need<int8_t>((size_t)8 * n * bs);
-      int* ex = oz->be->need<int>((size_t)bs);
-      std::vector<OzColJob> cj{OzColJob{Om, Xs, ex, n, bs, 0, n}};
+      const int w = bs * *std::max_element(ms.begin(), ms.end());
+      int8_t* Xs = oz->bx->need<int8_t>((size_t)8 * n * w);
+      int* ex = oz->be->need<int>((size_t)w);
+      std::vector<OzColJob> cj{OzColJob{Om, Xs, ex, n, w, 0, n}};
       oz_split_cols(ctx, cj);
       std::vector<OzJob> jobs;
       for (size_t s = 0; s < ops.size(); ++s) {
+        flops += 2.0 * n * n * bs * ms[s];
         jobs.push_back(OzJob{oz->Sr + (size_t)ops[s] * 8 * n * n, Xs, oz->e + ops[s], ex, Ydst[s], (size_t)n * n,
-                             (size_t)n * bs, n, n, n, bs, n});
+                             (size_t)n * w, n, n, n, bs * ms[s], n});
         jobs.back().nsplit = 1;  // a batch of tiles fills the GPU without splitting K
         jobs.back().tol = oz->thr8 / std::sqrt((double)n);  // column norm of the sample within thr / 8
       }
       oz_gemm(ctx, jobs);
       return;
     }
+    flops += 2.0 * n * n * bs * ops.size();
     std::vector<GemmJob<double>> jobs;
     for (size_t s = 0; s < ops.size(); ++s)
       jobs.push_back(job<double>(NN, n, bs, T + (size_t)ops[s] * n * n, n, Om, n, n, Ydst[s], n, 1.0, 0.0));
