@@ -16,7 +16,7 @@
 // recomputed once per sweep) plus a square root, a reciprocal and a reciprocal square root per pair.  So
 //   * several lanes share a pair, as many as keep the CTA's threads busy, and the pairs' rotation angles are
 //     computed together, one thread per pair, so that the scalar work fills its warps;
-//   * a tile of rank above TR_SOLO is spread over a cluster, its columns dealt out over the CTAs' shared memory
+//   * the tiles of the highest ranks are each spread over a cluster, the columns dealt out over the CTAs' shared memory
 //     and reached through distributed shared memory: the few tiles of high rank next to the diagonal are what a
 //     matrix's trimming waits for;
 //   * the tiles of low rank run beside them on the side stream.
@@ -26,6 +26,7 @@
 #include <cooperative_groups.h>
 #include <math.h>
 
+#include <functional>
 #include <map>
 
 #include "internal.h"
@@ -38,7 +39,7 @@ namespace {
 
 constexpr int TR_T = 256, TR_W = TR_T / 32;
 constexpr int TR_SWEEPS = 60;  // a bound only: the tiles converge in about 10
-constexpr int TR_SOLO = 48;    // highest rank of a single-CTA tile
+constexpr int TR_SOLO = 48;    // tiles up to this rank always take one CTA
 
 struct TrimDev {
   const double* B;  // b x r, leading dimension b
@@ -311,14 +312,21 @@ void trim_tiles(tlr_ctx* ctx, int b, const std::vector<TrimTile>& tiles, double 
   }
   double* ws = work.need<double>((size_t)std::max<int64_t>(tot, 1) + (size_t)(nt + 1) / 2 + 1);
   int* dr = reinterpret_cast<int*>(ws + std::max<int64_t>(tot, 1));
-  // Launch groups, highest ranks first.  A tile of rank up to TR_SOLO takes one CTA, in rank classes (so that a
-  // group's shared memory, sized by its largest rank, does not hold many small tiles to one CTA per SM); above
-  // that a cluster of four, or of eight where the tiles are too few for the GPU or four CTAs' shared memory does
-  // not hold X; where eight do not either, X lives in global memory.  (57 tiles of rank 56: clusters 3.2 ms against
-  // 10.2; 38 of rank 48 as single CTAs 2.5 ms, a third of what the clusters gain from there on.)
-  static const int cls[] = {8, 16, 24, 32, TR_SOLO};
+  // Launch groups, highest ranks first.  The tiles of the highest ranks, as many as fill the GPU twice, take a cluster
+  // of four (57 tiles of rank 80: 5.5 ms against 7.2 as single CTAs; of rank 56: 3.2 against 3.4, so not below TR_SOLO),
+  // or of eight where they are too few for the GPU or four CTAs' shared memory does not hold X; where eight do not
+  // either, X lives in global memory.  Further tiles fill the GPU one CTA each (152 of rank 64: 5.2 ms against 8.3 in
+  // clusters) unless X does not fit one, in rank classes (so that a group's shared memory, sized by its largest
+  // rank, does not hold many small tiles to one CTA per SM).
+  static const int cls[] = {8, 16, 24, 32, TR_SOLO, 64, 96, 128, 1 << 30};
+  std::vector<int> by_rank;
+  for (const TrimTile& t : tiles) by_rank.push_back(t.r);
+  std::sort(by_rank.begin(), by_rank.end(), std::greater<int>());
+  const size_t most = (size_t)std::max(1, ctx->sm_count / 2);  // clusters of four
+  const int top = std::max(TR_SOLO, (int)by_rank.size() > (int)most ? by_rank[most] : 0);
+  auto spread = [&](int r) { return r > top || (r > TR_SOLO && trim_smem(b, r, 1, true) > TRIM_SMEM_MAX); };
   int nbig = 0;
-  for (const TrimTile& t : tiles) nbig += t.r > TR_SOLO;
+  for (const TrimTile& t : tiles) nbig += spread(t.r);
   struct Group {
     int cs = 1;
     bool sm = true;
@@ -334,7 +342,7 @@ void trim_tiles(tlr_ctx* ctx, int b, const std::vector<TrimTile>& tiles, double 
     Zs[t] = d.Zs;
     int key, cs = 1;
     bool sm;
-    if (r > TR_SOLO) {
+    if (spread(r)) {
       cs = nbig * 8 <= ctx->sm_count || trim_smem(b, r, 4, true) > TRIM_SMEM_MAX ? 8 : 4;
       sm = trim_smem(b, r, cs, true) <= TRIM_SMEM_MAX;
       key = !sm ? 0 : cs == 8 ? 1 : 2;
@@ -342,7 +350,7 @@ void trim_tiles(tlr_ctx* ctx, int b, const std::vector<TrimTile>& tiles, double 
       int c = 0;
       while (cls[c] < r) ++c;
       sm = trim_smem(b, r, 1, true) <= TRIM_SMEM_MAX;
-      key = sm ? 10 - c : 3;
+      key = sm ? 20 - c : 3;
     }
     Group& g = groups[key];
     g.cs = cs;

@@ -19,6 +19,7 @@ def T():
     (3, 96, 48),     # the highest rank of a single CTA
     (2, 96, 49),     # the lowest of a cluster (of eight: few tiles), an odd number of columns
     (24, 128, 57),   # enough tiles for clusters of four
+    (160, 96, 50),   # more tiles of one rank than clusters fill the GPU with: one CTA each
     (1, 512, 480),   # R^T larger than eight CTAs' shared memory
 ])
 def test_singular_values_and_products(T, nt, b, r):
