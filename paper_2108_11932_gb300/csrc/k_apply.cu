@@ -20,7 +20,8 @@
 // tiles, which this replaces, did 16 columns' work for one and left the GPU nearly empty in each launch.
 // Measured before -> now: A X, 2D, eps = 1e-6, N = 4096 (b = 256), 1 column 952 -> 60 us; N = 131072
 // (b = 1024), 8 columns 25.2 -> 9.15 ms (0.94 of the DFMA rate); L D L^T X, 3D N = 20011, b = 512,
-// eps = 1e-4, 1 column 6.50 -> 0.32 ms.
+// eps = 1e-4, 1 column 6.50 -> 0.32 ms.  Several columns of a large matrix go to the tensor cores (below): the
+// 8 columns of N = 131072 9.15 -> 2.20 ms.
 //
 // Sums run in a fixed order: results do not depend on timing.
 #include <cooperative_groups.h>
@@ -54,6 +55,7 @@ struct ApTab {
   const int* voff;  // [j (nb + 1) + i]: first column of tile i in V panel j
   const int* uoff;  // [i (nb + 1) + j]: first column of tile j in U panel i
   int npan, nb, b, unit;
+  const int* gate;  // if set: the kernel runs only if *gate is not zero
 };
 
 // coefficient vectors are row-major with this many doubles per row (16-byte rows past one column)
@@ -87,12 +89,24 @@ __device__ __forceinline__ void ap_ld_a(const double* p, double (&a)[VEC]) {
 
 // X (original order) -> Xp (KD order, padded with zeros, row-major)
 __global__ void k_apply_gather(int64_t N, int64_t np, int nr, int ld, const int64_t* __restrict__ perm,
-                               const double* __restrict__ X, int64_t ldx, double* __restrict__ Xp) {
+                               const double* __restrict__ X, int64_t ldx, double* __restrict__ Xp, int* bad) {
+  if (bad && blockIdx.x == 0 && threadIdx.x == 0) *bad = 0;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < np * ld; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t p = e / ld;
     const int c = (int)(e % ld);
     Xp[e] = p < N && c < nr ? X[perm[p] + (int64_t)c * ldx] : 0.0;
   }
+}
+
+// the panel of CTA c of a list
+__device__ __forceinline__ int ap_panel(const ApTab& T, int c) {
+  int lo = 0, hi = T.npan - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (T.pan[mid].cta0 <= c) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
 }
 
 template <int NR, int VEC>
@@ -101,15 +115,8 @@ __global__ void __launch_bounds__(AP_T) k_apply_tn(ApTab T, const double* __rest
   constexpr int LD = ap_ld<NR>(), UN = NR <= 4 ? 2 : 1, STEP = 32 * VEC;
   constexpr int P = AP_CW * (NR == 3 ? 4 : NR == 6 ? 8 : NR), LANES = 32 / P;  // lanes that share a sum
   __shared__ int panel;
-  if (threadIdx.x == 0) {
-    int lo = 0, hi = T.npan - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (T.pan[mid].cta0 <= (int)blockIdx.x) lo = mid;
-      else hi = mid - 1;
-    }
-    panel = lo;
-  }
+  if (T.gate && *T.gate == 0) return;
+  if (threadIdx.x == 0) panel = ap_panel(T, (int)blockIdx.x);
   __syncthreads();
   const ApPanel pn = T.pan[panel];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, b = T.b;
@@ -220,6 +227,7 @@ __global__ void __launch_bounds__(AP_T) k_apply_nn(ApTab T, int dmode, int use_u
   constexpr int LD = ap_ld<NR>(), RB = 32 * VEC, UN = 4;
   __shared__ double red[AP_W * NR * RB];
   __shared__ double part[NR * RB];
+  if (T.gate && *T.gate == 0) return;
   const int b = T.b, rbs = (b + RB - 1) / RB;
   const int rank = (int)blockIdx.x % S, rb = (int)blockIdx.x / S;
   const int i = rb / rbs, r0 = (rb % rbs) * RB;
@@ -306,6 +314,522 @@ __global__ void __launch_bounds__(AP_T) k_apply_nn(ApTab T, int dmode, int use_u
   cl.sync();  // no CTA leaves while its part is still read
 }
 
+// ------------------------------------------------------------------ several columns: tensor cores
+// With two or more right-hand sides the DFMAs (one per entry and column, 2 per clock and SM) take several times
+// HBM's time.  The same contractions then run as exact integer products on the 16-bit tensor cores
+// (mma.sync.m16n8k16, FP16 in, FP32 accumulate: the eight columns are its N, and a fragment's FP64 entries
+// are split in the registers that loaded them, so that the factor is read as it lies; tcgen05 wants its
+// operands in shared or tensor memory and 128 rows, which a panel of a few columns does not fill).  The
+// splitting is that of k_ozaki.cu (Ozaki, Ogita, Oishi and Rump, 2012) with balanced digits:
+//   x = 2^(e - 57) F, F = round(x 2^(57 - e)) = sum_{i=1..7} d_i 256^(7 - i), |d_1| <= 512, -128 <= d_i <= 127
+// where 2^e bounds the operand's column: a panel column's own bound for the factor, the block's for each
+// right-hand side.  Pairs with i + j <= 9 are kept (34 products a step; the dropped ones are 2^-66 of the
+// bounds); a group of equal i + j sums below 13 2^14 4 16 < 2^24 over four steps, exact in FP32, and moves to
+// 64-bit integers then; one rounding at the end.  Error: 2^-58 of the bounds per entry and factor, against FP64's
+// 2^-53 of the running sum per term: of A X, L X, L^T X and L (D) L^T X in 2D and 3D, eps 1e-8 to 1e-2, normal,
+// positive and right-hand sides over eight decades it is 0.2 to 0.8 of the DFMA kernels' (norm against extended
+// precision; truncating F, two instructions less, would make it up to twice theirs).
+// Where the contraction index is the panel's column (Y_i += U_ij T_ij), the column's bound 2^e moves to the
+// coefficient: (A(m, k) 2^-e_k) (2^e_k T(k)).
+// Bound: the integer instructions that split (about 18 per entry, at half rate; the ALU is busy 57 % of the
+// time, the tensor pipe 32 %, 16 warps per SM at 126 registers).  34 products of 16 x 8 x 16 per 256 entries.
+// Latency: each lane copies its own fragments of the next steps into shared memory (cp.async, no barrier).
+constexpr int TC_P = 7;      // digits
+constexpr int TC_KS = 16;    // k per step
+constexpr int TC_WIN = 4;    // steps of an exact window
+constexpr int TC_STG = 3;    // steps in flight per warp
+constexpr int TC_SPC = 8;    // CTAs (a cluster) per block in k_apply_split
+constexpr int TC_FRAG = 64;  // uint4 per step of a split right-hand side: [2][lane], the words of tc_digits with the sign on top
+constexpr int TC_W = 4, TC_T = 32 * TC_W;  // warps of k_apply_tn_tc and k_apply_nn_tc
+constexpr int TC_SMEM = TC_W * TC_STG * 32 * (64 + 32 + 16);
+
+// Exponent e with |x| < 2^e for the largest |x| whose high word is hw (1 for a zero column: any bound will do)
+__device__ __forceinline__ int tc_exp(unsigned hw) { return hw == 0 ? 1 : (int)(hw >> 20) - 1022; }
+// a column of tiny, huge or non-finite numbers
+__device__ __forceinline__ bool tc_odd(int e) { return e < -900 || e > 900; }
+// What tc_pairs takes of a column with |x| < 2^e (-900 <= e <= 900)
+__device__ __forceinline__ int tc_shift(int e) { return (e + 1022) << 20; }
+// |F| + 0x6600808080808080 as two words: the bytes are d_7 + 128, ..., d_2 + 128 and the FP16 number 1536 + d_1.
+// Rounds to nearest; the sign of bad is set unless |x| < 2^e; zeros and denormals give 0.
+__device__ __forceinline__ uint2 tc_digits(double x, int shift, int& bad) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  // |x| 2^(58 - e) = (mantissa 2^5) >> (e + 1022 - exponent field)
+  const int t = shift - (int)(hi & 0x7ff00000u);
+  bad |= t;
+  unsigned long long w = ((unsigned long long)((__funnelshift_l(lo, hi, 5) & 0x01ffffffu) | 0x02000000u) << 32) | (lo << 5);
+  asm("shr.u64 %0, %0, %1;" : "+l"(w) : "r"((unsigned)t >> 20));  // 0 from 64 on
+  w = (w + (2 * 0x6600808080808080ull + 1)) >> 1;
+  return make_uint2((unsigned)w, (unsigned)(w >> 32));
+}
+__device__ __forceinline__ unsigned tc_fma2(unsigned a, unsigned b, unsigned c) {
+  unsigned r;
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  return r;
+}
+// the seven digit pairs of entries a, b with the signs of the high words sa, sb: FP16 (1024 + byte) s - (1024 + 128) s
+__device__ __forceinline__ void tc_pairs(uint2 a, uint2 b, unsigned sa, unsigned sb, unsigned (&d)[TC_P]) {
+  const unsigned p0 = __byte_perm(a.x, b.x, 0x5140u), p1 = __byte_perm(a.x, b.x, 0x7362u), p2 = __byte_perm(a.y, b.y, 0x5140u);
+  const unsigned sg = __byte_perm(sa, sb, 0x7632u) & 0x80008000u;
+  const unsigned one = 0x64646464u, s = sg ^ 0x3c003c00u, bias = sg ^ 0xe480e480u, bias1 = sg ^ 0xe600e600u;
+  d[6] = tc_fma2(__byte_perm(p0, one, 0x4140u), s, bias);  // byte 0: the least significant digit
+  d[5] = tc_fma2(__byte_perm(p0, one, 0x4342u), s, bias);
+  d[4] = tc_fma2(__byte_perm(p1, one, 0x4140u), s, bias);
+  d[3] = tc_fma2(__byte_perm(p1, one, 0x4342u), s, bias);
+  d[2] = tc_fma2(__byte_perm(p2, one, 0x4140u), s, bias);
+  d[1] = tc_fma2(__byte_perm(p2, one, 0x4342u), s, bias);
+  d[0] = tc_fma2(__byte_perm(a.y, b.y, 0x7632u), s, bias1);
+}
+__device__ __forceinline__ void tc_mma(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+struct TcAcc {  // group sums of a window; the totals: hi of the groups 0-3, lo of 4-7 (weights 256^-g)
+  float f[8][4];
+  long long hi[4], lo[4];
+  int win, bad;
+};
+__device__ __forceinline__ void tc_init(TcAcc& a) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    a.hi[c] = a.lo[c] = 0;
+#pragma unroll
+    for (int g = 0; g < 8; ++g) a.f[g][c] = 0.f;
+  }
+  a.win = a.bad = 0;
+}
+__device__ __forceinline__ void tc_drain(TcAcc& a) {
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    long long h = 0, l = 0;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      h = h * 256 + __float2int_rn(a.f[g][c]);
+      l = l * 256 + __float2int_rn(a.f[g + 4][c]);
+      a.f[g][c] = a.f[g + 4][c] = 0.f;
+    }
+    a.hi[c] += h;
+    a.lo[c] += l;
+  }
+  a.win = 0;
+}
+// One step (CHECK: notes entries outside their bounds): the tile's fragments x[row half][k half][2] (rows g, g + 8; k 2t, 2t + 1, 2t + 8, 2t + 9 of the lane
+// g = lane / 4, t = lane % 4) with shifts e, times the split right-hand side's step (column g; the same k)
+template <bool CHECK>
+__device__ __forceinline__ void tc_step(const double (&x)[2][2][2], const int (&e)[2][2][2], uint4 f0, uint4 f1, TcAcc& acc) {
+  int bad = 0;
+  unsigned d[2][2][TC_P], b0[TC_P], b1[TC_P];
+  tc_pairs(make_uint2(f0.x, f0.y & 0x7fffffffu), make_uint2(f0.z, f0.w & 0x7fffffffu), f0.y, f0.w, b0);
+  tc_pairs(make_uint2(f1.x, f1.y & 0x7fffffffu), make_uint2(f1.z, f1.w & 0x7fffffffu), f1.y, f1.w, b1);
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      tc_pairs(tc_digits(x[r][h][0], e[r][h][0], bad), tc_digits(x[r][h][1], e[r][h][1], bad),
+               (unsigned)__double2hiint(x[r][h][0]), (unsigned)__double2hiint(x[r][h][1]), d[r][h]);
+#pragma unroll
+  for (int i = 0; i < TC_P; ++i) {
+    const unsigned a[4] = {d[0][0][i], d[1][0][i], d[0][1][i], d[1][1][i]};
+#pragma unroll
+    for (int j = 0; j < TC_P; ++j)
+      if (i + j <= 7) tc_mma(acc.f[i + j], a, b0[j], b1[j]);
+  }
+  if (CHECK) acc.bad |= bad;
+  if (++acc.win == TC_WIN) tc_drain(acc);
+}
+// value of a total: digits i, j carry 2^(-1 - 8 i) each (i, j from 1): group g = i + j - 2 carries 2^(-18 - 8 g)
+__device__ __forceinline__ double tc_value(long long hi, long long lo, int e) {
+  return ldexp(fma((double)hi, 4294967296.0, (double)lo), e - 74);
+}
+// The warps' totals through shared memory: thread `threadIdx.x` < 128 gets entry (lane / 4 + 8 (c / 2), 2 (lane % 4) + c % 2)
+// of the fragment, lane = threadIdx.x / 4, c = threadIdx.x % 4
+__device__ __forceinline__ void tc_total(TcAcc& acc, long long* part, long long& h, long long& l) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  tc_drain(acc);
+  __syncthreads();  // the copies' buffers are free
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    part[(warp * 32 + lane) * 8 + c] = acc.hi[c];
+    part[(warp * 32 + lane) * 8 + 4 + c] = acc.lo[c];
+  }
+  __syncthreads();
+  h = l = 0;
+  if (threadIdx.x >= TC_T) return;
+#pragma unroll
+  for (int w = 0; w < TC_W; ++w) {
+    h += part[(w * 32 + (threadIdx.x >> 2)) * 8 + (threadIdx.x & 3)];
+    l += part[(w * 32 + (threadIdx.x >> 2)) * 8 + 4 + (threadIdx.x & 3)];
+  }
+}
+// copies of a lane's own bytes to shared memory, zeros if !ok (src must be readable memory all the same)
+__device__ __forceinline__ void tc_cp16(void* dst, const void* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(ok ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void tc_cp8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+struct TcLane {  // a lane's slots of a warp's ring
+  char* base;
+  __device__ __forceinline__ TcLane(char* smem) : base(smem + (threadIdx.x >> 5) * (TC_STG * 32 * 112)) {}
+  __device__ __forceinline__ double2* x(int st, int q) const {
+    return reinterpret_cast<double2*>(base + st * 32 * 112) + q * 32 + (threadIdx.x & 31);
+  }
+  __device__ __forceinline__ uint4* f(int st, int q) const {
+    return reinterpret_cast<uint4*>(base + st * 32 * 112 + 2048) + q * 32 + (threadIdx.x & 31);
+  }
+  __device__ __forceinline__ int2* e(int st, int q) const {
+    return reinterpret_cast<int2*>(base + st * 32 * 112 + 3072) + q * 32 + (threadIdx.x & 31);
+  }
+};
+// steps first, first + TC_W, ... < end of a warp: issue(step, stage) copies, use(step, stage) computes
+template <class I>
+__device__ __forceinline__ void tc_ring_begin(int first, int end, I issue) {
+#pragma unroll
+  for (int q = 0; q < TC_STG - 1; ++q) {
+    if (first + q * TC_W < end) issue(first + q * TC_W, q);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+}
+template <class I, class C>
+__device__ __forceinline__ void tc_ring(int first, int end, I issue, C use) {
+  int next = first + (TC_STG - 1) * TC_W, st = 0, sn = TC_STG - 1;
+  for (int s = first; s < end; s += TC_W) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(TC_STG - 2) : "memory");
+    if (next < end) issue(next, sn);
+    next += TC_W;
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    use(s, st);
+    st = st + 1 == TC_STG ? 0 : st + 1;
+    sn = sn + 1 == TC_STG ? 0 : sn + 1;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+struct TcSeg {  // a split right-hand side: a block's rows in up to three segments, each padded to whole steps
+  int64_t ks0;  // first step
+  int n0, n1, n2;
+};
+
+// Splits the right-hand sides of block blockIdx.x / TC_SPC: rows of X (SEG = 1: the block's b rows), or
+// [X_i; T_i; S_i] scaled by the panels' column bounds (SEG = 3; the bounds' shifts, by step, to ek).
+// Fragments to frag, the columns' exponents to ef.  A cluster per block finds the bounds together.
+template <int SEG>
+__global__ void __cluster_dims__(TC_SPC, 1, 1) __launch_bounds__(256)
+    k_apply_split(const TcSeg* __restrict__ segs, const ApRow* __restrict__ rows, int b, const double* __restrict__ X,
+                  const double* __restrict__ TR, const double* __restrict__ SC, const int* __restrict__ eD,
+                  const int* __restrict__ eU, const int* __restrict__ eV, uint4* __restrict__ frag, int* __restrict__ ek_out,
+                  int* __restrict__ ef, int* bad_out) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int i = blockIdx.x / TC_SPC, rank = blockIdx.x % TC_SPC, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const TcSeg sg = segs[i];
+  const int s0 = (sg.n0 + TC_KS - 1) / TC_KS, s1 = SEG > 1 ? (sg.n1 + TC_KS - 1) / TC_KS : 0,
+            s2 = SEG > 1 ? (sg.n2 + TC_KS - 1) / TC_KS : 0, steps = s0 + s1 + s2;
+  __shared__ int part[8], emax[8];
+  if (tid < 8) part[tid] = -100000;
+  __syncthreads();
+  // row k of step s: its coefficients and the exponent of its panel column
+  auto entry = [&](int s, int k, int& ek) -> const double* {
+    ek = SEG > 1 ? 1 : 0;
+    if (s < s0) {
+      k += s * TC_KS;
+      if (k >= sg.n0) return nullptr;
+      if (SEG > 1) ek = eD[(int64_t)i * b + k];
+      return X + ((int64_t)i * b + k) * 8;
+    }
+    if (s < s0 + s1) {
+      k += (s - s0) * TC_KS;
+      if (k >= sg.n1) return nullptr;
+      ek = eU[rows[i].tr0 + k];
+      return TR + (rows[i].tr0 + k) * 8;
+    }
+    k += (s - s0 - s1) * TC_KS;
+    if (k >= sg.n2) return nullptr;
+    ek = eV[rows[i].sc0 + k];
+    return SC + (rows[i].sc0 + k) * 8;
+  };
+  int m = -100000;  // of column tid % 8
+  for (int o = rank * 256 + tid; o < steps * 128; o += TC_SPC * 256) {
+    int ek;
+    const double* p = entry(o >> 7, (o >> 3) & 15, ek);
+    const unsigned hw = p ? (unsigned)__double2hiint(p[o & 7]) & 0x7fffffffu : 0u;
+    if (hw) m = max(m, tc_exp(hw) + ek);
+    if (SEG > 1 && (o & 7) == 0) ek_out[sg.ks0 * TC_KS + (o >> 3)] = tc_shift(ek);
+  }
+  atomicMax(&part[tid & 7], m);
+  cl.sync();
+  if (tid < 8) {
+    int v = -100000;
+#pragma unroll
+    for (int q = 0; q < TC_SPC; ++q) v = max(v, cl.map_shared_rank(part, q)[tid]);
+    if (v == -100000) v = 1;
+    else if (tc_odd(v)) *bad_out = 1;
+    emax[tid] = v;
+    if (rank == 0) ef[i * 8 + tid] = v;
+  }
+  cl.sync();
+  const int n = lane >> 2, t = lane & 3, en = emax[n];
+  for (int s = rank * 8 + warp; s < steps; s += TC_SPC * 8) {
+    uint2 q[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      int ek;
+      const double* p = entry(s, 2 * t + (u & 1) + (u >> 1) * 8, ek);
+      const double x = p ? p[n] : 0.0;
+      const int e = x == 0.0 ? 1 : en - ek;
+      if (tc_odd(e)) *bad_out = 1;
+      int bad = 0;  // |x| < 2^e by its making
+      q[u] = tc_digits(x, tc_shift(e), bad);
+      q[u].y |= (unsigned)__double2hiint(x) & 0x80000000u;
+    }
+    uint4* out = frag + (sg.ks0 + s) * TC_FRAG + lane;
+    out[0] = make_uint4(q[0].x, q[0].y, q[1].x, q[1].y);
+    out[32] = make_uint4(q[2].x, q[2].y, q[3].x, q[3].y);
+  }
+}
+
+// place of a panel column's exponent
+__device__ __forceinline__ int* tc_expof(const ApTab& T, const ApPanel& pn, int c, int* eU, int* eV, int* eD) {
+  return pn.kind == 0 ? eV + T.row[pn.blk].sc0 + c : pn.kind == 1 ? eU + T.row[pn.blk].tr0 + c : eD + (int64_t)pn.blk * T.b + c;
+}
+
+// the last q in [0, n) with at(q) <= c (at(0) <= c, at monotone), by a whole warp, 32 places at a time
+template <class F>
+__device__ __forceinline__ int tc_search(int c, int n, F at) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0;
+  while (n > 1) {
+    const int step = (n + 31) / 32, q = lane * step;
+    const unsigned m = __ballot_sync(0xffffffffu, q < n && at(lo + q) <= c);
+    const int k = 31 - __clz(m);
+    lo += k * step;
+    n = min(step, n - k * step);
+  }
+  return lo;
+}
+
+// k_apply_tn on the tensor cores: 16 columns of a panel per CTA, its warps sharing the b rows.  The columns'
+// bounds are found first (the second pass over the 16 columns comes from the caches) and kept for k_apply_nn_tc.
+__global__ void __launch_bounds__(TC_T, 4) k_apply_tn_tc(ApTab T, const TcSeg* __restrict__ segs, const uint4* __restrict__ frag,
+                                                         const int* __restrict__ ef, double* __restrict__ TR,
+                                                         double* __restrict__ SC, double* __restrict__ YD,
+                                                         int* __restrict__ eU, int* __restrict__ eV, int* __restrict__ eD,
+                                                         int* bad_out) {
+  extern __shared__ __align__(16) char tc_smem[];
+  __shared__ int64_t dst[16];  // row of a column's coefficients
+  __shared__ unsigned cmax[TC_W][16];
+  const ApPanel pn = T.pan[tc_search((int)blockIdx.x / 2, T.npan, [&](int q) { return __ldg(&T.pan[q].cta0); })];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, b = T.b;
+  const int c0 = ((int)blockIdx.x - 2 * pn.cta0) * 16, steps = (b + TC_KS - 1) / TC_KS;
+  if (c0 >= pn.ncols) return;
+  const bool tri = pn.kind == 2;
+  const double* A[2];
+  bool live[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    live[r] = c0 + g + 8 * r < pn.ncols;
+    A[r] = pn.A + (size_t)(live[r] ? c0 + g + 8 * r : c0) * b;
+  }
+  for (int q = warp; q < 16 && c0 + q < pn.ncols; q += TC_W) {
+    const int c = c0 + q, j = pn.blk;
+    int64_t d = (int64_t)j * b + c;
+    if (!tri) {  // tile a of the panel with off[a] <= c < off[a + 1] (tiles of rank 0 are empty ranges)
+      const int* off = (pn.kind == 0 ? T.voff : T.uoff) + (size_t)j * (T.nb + 1);
+      const int a = tc_search(c, T.nb, [&](int k) { return __ldg(off + k); });
+      const int at = c - off[a];
+      d = pn.kind == 0 ? T.row[a].tr0 + T.uoff[(size_t)a * (T.nb + 1) + j] + at : T.row[a].sc0 + T.voff[(size_t)a * (T.nb + 1) + j] + at;
+    }
+    if (lane == 0) dst[q] = d;
+  }
+  // lower triangle of a tile, unit diagonal for L D L^T
+  auto mask = [&](int r, int k, double2& v) {
+    const int c = c0 + g + 8 * r;
+    if (k < c) v.x = 0.0;
+    else if (k == c && T.unit) v.x = 1.0;
+    if (k + 1 < c) v.y = 0.0;
+    else if (k + 1 == c && T.unit) v.y = 1.0;
+  };
+  const int first = (tri ? c0 / TC_KS : 0) + warp;  // steps before the diagonal are zero
+  const uint4* fr = frag + segs[pn.blk].ks0 * TC_FRAG + lane;
+  const TcLane ring(tc_smem);
+  auto issue = [&](int s, int st) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = s * TC_KS + 2 * t + 8 * h;
+        tc_cp16(ring.x(st, 2 * r + h), A[r] + (k < b ? k : 0), live[r] && k < b);
+      }
+    tc_cp16(ring.f(st, 0), fr + (int64_t)s * TC_FRAG, true);
+    tc_cp16(ring.f(st, 1), fr + (int64_t)s * TC_FRAG + 32, true);
+  };
+  tc_ring_begin(first, steps, issue);
+  unsigned m[2] = {0, 0};
+#pragma unroll 4
+  for (int s = first; s < steps; s += TC_W) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = s * TC_KS + 2 * t + 8 * h;
+        double2 v = make_double2(0.0, 0.0);
+        if (live[r] && k < b) v = __ldg(reinterpret_cast<const double2*>(A[r] + k));  // b is even
+        if (tri) mask(r, k, v);
+        m[r] = max(m[r], max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+      }
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    m[r] = max(m[r], __shfl_xor_sync(0xffffffffu, m[r], 1));
+    m[r] = max(m[r], __shfl_xor_sync(0xffffffffu, m[r], 2));
+    if (t == 0) cmax[warp][g + 8 * r] = m[r];
+  }
+  __syncthreads();
+  auto bound = [&](int c) {
+    unsigned v = 0;
+#pragma unroll
+    for (int w = 0; w < TC_W; ++w) v = max(v, cmax[w][c]);
+    return tc_exp(v);
+  };
+  int ec[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    ec[r] = bound(g + 8 * r);
+    if (warp == 0 && t == 0 && live[r]) {
+      *tc_expof(T, pn, c0 + g + 8 * r, eU, eV, eD) = ec[r];
+      if (tc_odd(ec[r])) *bad_out = 1;
+    }
+  }
+  const int h0 = tc_shift(ec[0]), h1 = tc_shift(ec[1]), e[2][2][2] = {{{h0, h0}, {h0, h0}}, {{h1, h1}, {h1, h1}}};
+  TcAcc acc;
+  tc_init(acc);
+  tc_ring(
+      first, steps, issue,
+      [&](int s, int st) {
+        double x[2][2][2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            double2 v = *ring.x(st, 2 * r + h);
+            if (tri) mask(r, s * TC_KS + 2 * t + 8 * h, v);
+            x[r][h][0] = v.x;
+            x[r][h][1] = v.y;
+          }
+        tc_step<false>(x, e, *ring.f(st, 0), *ring.f(st, 1), acc);
+      });
+  long long h, l;
+  tc_total(acc, reinterpret_cast<long long*>(tc_smem), h, l);
+  const int ol = threadIdx.x >> 2, oc = threadIdx.x & 3, or_ = (ol >> 2) + 8 * (oc >> 1), cc = c0 + or_, n = 2 * (ol & 3) + (oc & 1);
+  if (cc >= pn.ncols) return;
+  const double y = tc_value(h, l, bound(or_) + ef[pn.blk * 8 + n]);
+  (tri ? YD : pn.kind == 0 ? TR : SC)[dst[or_] * 8 + n] = y;
+}
+
+// k_apply_nn on the tensor cores: 16 rows of a block row per CTA, its warps sharing the steps of
+// [D_i | Urow_i | Vcol_i] [X_i; T_i; S_i].  Rows 2 g and 2 g + 1 are the fragment's rows g and g + 8 (16-byte loads).
+__global__ void __launch_bounds__(TC_T, 4) k_apply_nn_tc(ApTab T, int dmode, const TcSeg* __restrict__ segs,
+                                                         const uint4* __restrict__ frag, const int* __restrict__ ek,
+                                                         const int* __restrict__ ef, ApOut out, int* bad_out) {
+  extern __shared__ __align__(16) char tc_smem[];
+  const int b = T.b, rbs = (b + 15) / 16, i = (int)blockIdx.x / rbs, r0 = ((int)blockIdx.x % rbs) * 16;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const ApRow row = T.row[i];
+  const TcSeg sg = segs[i];
+  const int s0 = (sg.n0 + TC_KS - 1) / TC_KS, s1 = (sg.n1 + TC_KS - 1) / TC_KS, s2 = (sg.n2 + TC_KS - 1) / TC_KS;
+  const int d0 = dmode == 2 ? min(s0, r0 / TC_KS + 1) : s0;  // steps past the diagonal are zero
+  const int mr = r0 + 2 * g;
+  TcAcc acc;
+  tc_init(acc);
+  const uint4* fr = frag + sg.ks0 * TC_FRAG + lane;
+  const int* er = ek + sg.ks0 * TC_KS + 2 * t;
+  const TcLane ring(tc_smem);
+  auto issue = [&](int v, int st) {
+    const int s = v < d0 ? v : v - d0 + s0;
+    const double* P = s < s0 ? row.D : s < s0 + s1 ? row.U : row.V;
+    const int kb = (s < s0 ? s : s < s0 + s1 ? s - s0 : s - s0 - s1) * TC_KS, len = s < s0 ? sg.n0 : s < s0 + s1 ? sg.n1 : sg.n2;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = kb + 2 * t + (q & 1) + 8 * (q >> 1);
+      const bool ok = k < len && mr < b;
+      tc_cp16(ring.x(st, q), ok ? P + mr + (size_t)k * b : P, ok);
+    }
+    tc_cp16(ring.f(st, 0), fr + (int64_t)s * TC_FRAG, true);
+    tc_cp16(ring.f(st, 1), fr + (int64_t)s * TC_FRAG + 32, true);
+    tc_cp8(ring.e(st, 0), er + (int64_t)s * TC_KS);
+    tc_cp8(ring.e(st, 1), er + (int64_t)s * TC_KS + 8);
+  };
+  tc_ring_begin(warp, d0 + s1 + s2, issue);
+  tc_ring(
+      warp, d0 + s1 + s2, issue,
+      [&](int v, int st) {
+        double x[2][2][2];
+        int e[2][2][2];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          double2 a = *ring.x(st, q);
+          if (dmode == 2 && v < d0) {
+            const int k = v * TC_KS + 2 * t + (q & 1) + 8 * (q >> 1);
+            if (mr < k) a.x = 0.0;
+            else if (mr == k && T.unit) a.x = 1.0;
+            if (mr + 1 < k) a.y = 0.0;
+            else if (mr + 1 == k && T.unit) a.y = 1.0;
+          }
+          x[0][q >> 1][q & 1] = a.x;
+          x[1][q >> 1][q & 1] = a.y;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int2 ev = *ring.e(st, h);
+          e[0][h][0] = e[1][h][0] = ev.x;  // shifts
+          e[0][h][1] = e[1][h][1] = ev.y;
+        }
+        if (dmode == 1) tc_step<true>(x, e, *ring.f(st, 0), *ring.f(st, 1), acc);
+        else tc_step<false>(x, e, *ring.f(st, 0), *ring.f(st, 1), acc);
+      });
+  if (acc.bad < 0) *bad_out = 1;
+  long long h, l;
+  tc_total(acc, reinterpret_cast<long long*>(tc_smem), h, l);
+  const int ol = threadIdx.x >> 2, oc = threadIdx.x & 3, m = r0 + 2 * (ol >> 2) + (oc >> 1), n = 2 * (ol & 3) + (oc & 1);
+  if (m >= b || (!out.Z && n >= out.nr)) return;
+  double v = tc_value(h, l, ef[i * 8 + n]);
+  const int64_t gr = (int64_t)i * b + m;
+  if (out.add) v += out.add[gr * 8 + n];
+  if (out.scale) v *= out.scale[gr];
+  if (out.Z) out.Z[gr * 8 + n] = v;
+  else if (gr < out.N) out.Y[out.perm[gr] + n * out.ldy] = v;
+}
+
+// exponents of the columns of a list's panels that k_apply_nn_tc reads and k_apply_tn_tc has not: a warp per column
+__global__ void __launch_bounds__(AP_T) k_apply_colexp(ApTab T, int* __restrict__ eU, int* __restrict__ eV,
+                                                       int* __restrict__ eD, int* bad_out) {
+  const ApPanel pn = T.pan[ap_panel(T, (int)blockIdx.x)];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, b = T.b;
+  for (int q = 0; q < AP_CW; ++q) {
+    const int c = ((int)blockIdx.x - pn.cta0) * AP_W * AP_CW + q * AP_W + warp;
+    if (c >= pn.ncols) return;
+    const double* A = pn.A + (size_t)c * b;
+    unsigned m = pn.kind == 2 && T.unit ? 0x3ff00000u : 0u;
+    const int first = pn.kind == 2 ? c + (T.unit ? 1 : 0) : 0;
+#pragma unroll 4
+    for (int k = 2 * lane; k < b; k += 64) {
+      const double2 v = __ldg(reinterpret_cast<const double2*>(A + k));
+      if (k >= first) m = max(m, (unsigned)__double2hiint(v.x) & 0x7fffffffu);
+      if (k + 1 >= first) m = max(m, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+    }
+    for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) {
+      *tc_expof(T, pn, c, eU, eV, eD) = tc_exp(m);
+      if (tc_odd(tc_exp(m))) *bad_out = 1;
+    }
+  }
+}
+__global__ void k_apply_fill(int64_t n, int e, int* __restrict__ eD) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) eD[i] = e;
+}
+
 unsigned blocks(int64_t n, int t) { return (unsigned)std::min<int64_t>((n + t - 1) / t, 8192); }
 
 template <int NR, int VEC>
@@ -342,10 +866,41 @@ void run_nn(tlr_ctx* ctx, const ApTab& T, int dmode, int use_u, int use_v, int64
 
 struct ApPlan {  // host side of one matrix's tables
   ApTab T;       // pan set per list
-  const ApPanel* lists[2];
-  int npan[2], ctas[2];
-  int64_t R, np, ktot_d;
+  const ApPanel* lists[3];  // of the contractions, and the columns whose exponents they don't find
+  int npan[3], ctas[3];
+  int64_t R, np;
+  // tensor-core path: the blocks' right-hand sides (X; what follows for L^T X: S; then [X; T; S] or [Z; T]) and their steps
+  bool tc;
+  const TcSeg* segs[3];
+  int64_t steps[3];
 };
+
+// The product from the gathered right-hand sides Xp
+template <int NR, int VEC>
+void apply_run(tlr_ctx* ctx, const tlr_mat* M, int op, const ApPlan& pl, ApTab T, int nr, const double* Xp, double* YD,
+               double* Z, double* TR, double* SC, double* Y, int64_t ldy) {
+  auto tn = [&](int l, const double* x) {
+    T.pan = pl.lists[l];
+    T.npan = pl.npan[l];
+    run_tn<NR, VEC>(ctx, T, pl.ctas[l], x, TR, SC, YD);
+  };
+  ApOut fin{nullptr, nullptr, nullptr, Y, M->dperm, ldy, M->N, nr};
+  const int64_t kd = (int64_t)M->nb * M->b;
+  tn(0, Xp);
+  if (op == TLR_OP_A) {
+    run_nn<NR, VEC>(ctx, T, 1, 1, 1, kd + 2 * pl.R, Xp, TR, SC, fin);
+  } else if (op == TLR_OP_L) {
+    run_nn<NR, VEC>(ctx, T, 2, 1, 0, kd / 2 + pl.R, Xp, TR, SC, fin);
+  } else if (op == TLR_OP_LT) {
+    fin.add = YD;
+    run_nn<NR, VEC>(ctx, T, 0, 0, 1, pl.R, Xp, TR, SC, fin);
+  } else {  // L (D) (L^T X)
+    ApOut mid{YD, M->state == 2 ? M->dvec : nullptr, Z, nullptr, nullptr, 0, 0, nr};
+    run_nn<NR, VEC>(ctx, T, 0, 0, 1, pl.R, Xp, TR, SC, mid);
+    tn(1, Z);
+    run_nn<NR, VEC>(ctx, T, 2, 1, 0, kd / 2 + pl.R, Z, TR, SC, fin);
+  }
+}
 
 template <int NR, int VEC>
 void apply_group(tlr_ctx* ctx, const tlr_mat* M, int op, const ApPlan& pl, int nr, const double* X, int64_t ldx, double* Y,
@@ -355,33 +910,83 @@ void apply_group(tlr_ctx* ctx, const tlr_mat* M, int op, const ApPlan& pl, int n
   double* Xp = work.need<double>((size_t)(3 * np + 2 * R) * LD);
   double *YD = Xp + np * LD, *Z = YD + np * LD, *TR = Z + np * LD, *SC = TR + R * LD;
   TLR_SITE_PRE(ctx);
-  k_apply_gather<<<blocks(np * LD, 256), 256, 0, ctx->stream>>>(M->N, np, nr, LD, M->dperm, X, ldx, Xp);
+  k_apply_gather<<<blocks(np * LD, 256), 256, 0, ctx->stream>>>(M->N, np, nr, LD, M->dperm, X, ldx, Xp, nullptr);
   TLR_LAUNCH_CHECK(ctx);
+  apply_run<NR, VEC>(ctx, M, op, pl, pl.T, nr, Xp, YD, Z, TR, SC, Y, ldy);
+}
+
+// The same on the tensor cores (8 columns, zero past nr).  Numbers outside what the digits hold (not finite, or a
+// column's largest below 2^-900 or above 2^900) set a flag, and then the FP64 kernels that follow run too.
+void apply_group_tc(tlr_ctx* ctx, const tlr_mat* M, int op, const ApPlan& pl, int nr, const double* X, int64_t ldx, double* Y,
+                    int64_t ldy, Buf& work) {
+  const int64_t np = pl.np, R = std::max<int64_t>(pl.R, 1);
+  const int64_t steps = std::max({pl.steps[0], pl.steps[1], pl.steps[2]});
+  const int nb = M->nb, b = M->b;
+  // doubles: Xp, YD, Z (np x 8), T, S (R x 8); fragments (16 bytes); ints: exponents by step, of U, V
+  // and tile columns, of the blocks' right-hand sides, the flag
+  const size_t nd = (size_t)(3 * np + 2 * R) * 8, nf = 2 * (size_t)steps * TC_FRAG,
+               ni = (size_t)(steps * TC_KS + 2 * R + np + 8 * (int64_t)nb + 1);
+  double* Xp = work.need<double>(nd + nf + (ni + 1) / 2);
+  double *YD = Xp + np * 8, *Z = YD + np * 8, *TR = Z + np * 8, *SC = TR + R * 8;
+  uint4* frag = reinterpret_cast<uint4*>(Xp + nd);
+  int* ek = reinterpret_cast<int*>(Xp + nd + nf);
+  int *eU = ek + steps * TC_KS, *eV = eU + R, *eD = eV + R, *ef = eD + np, *bad = ef + 8 * (int64_t)nb;
+  TLR_SITE_PRE(ctx);
+  k_apply_gather<<<blocks(np * 8, 256), 256, 0, ctx->stream>>>(M->N, np, nr, 8, M->dperm, X, ldx, Xp, bad);
+  TLR_LAUNCH_CHECK(ctx);
+  for (const void* f : {(const void*)k_apply_tn_tc, (const void*)k_apply_nn_tc})
+    TLR_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM));
   ApTab T = pl.T;
   auto tn = [&](int l, const double* x) {
+    TLR_SITE_PRE(ctx);
+    k_apply_split<1><<<(unsigned)nb * TC_SPC, 256, 0, ctx->stream>>>(pl.segs[0], T.row, b, x, TR, SC, eD, eU, eV, frag, ek, ef,
+                                                                             bad);
+    TLR_LAUNCH_CHECK(ctx);
+    if (pl.ctas[l] <= 0) return;
     T.pan = pl.lists[l];
     T.npan = pl.npan[l];
-    run_tn<NR, VEC>(ctx, T, pl.ctas[l], x, TR, SC, YD);
+    TLR_SITE_PRE(ctx);
+    k_apply_tn_tc<<<2 * (unsigned)pl.ctas[l], TC_T, TC_SMEM, ctx->stream>>>(T, pl.segs[0], frag, ef, TR, SC, YD, eU, eV, eD, bad);
+    TLR_LAUNCH_CHECK(ctx);
   };
-  ApOut fin{nullptr, nullptr, nullptr, Y, M->dperm, ldy, M->N, nr};
-  const int64_t kd = (int64_t)M->nb * M->b;
-  if (op == TLR_OP_A) {
-    tn(0, Xp);
-    run_nn<NR, VEC>(ctx, T, 1, 1, 1, kd + 2 * pl.R, Xp, TR, SC, fin);
-  } else if (op == TLR_OP_L) {
-    tn(0, Xp);
-    run_nn<NR, VEC>(ctx, T, 2, 1, 0, kd / 2 + pl.R, Xp, TR, SC, fin);
-  } else if (op == TLR_OP_LT) {
-    tn(0, Xp);
-    fin.add = YD;
-    run_nn<NR, VEC>(ctx, T, 0, 0, 1, pl.R, Xp, TR, SC, fin);
-  } else {  // L (D) (L^T X)
-    tn(0, Xp);
-    ApOut mid{YD, M->state == 2 ? M->dvec : nullptr, Z, nullptr, nullptr, 0, 0, nr};
-    run_nn<NR, VEC>(ctx, T, 0, 0, 1, pl.R, Xp, TR, SC, mid);
-    tn(1, Z);
-    run_nn<NR, VEC>(ctx, T, 2, 1, 0, kd / 2 + pl.R, Z, TR, SC, fin);
+  auto nn = [&](int q, int dmode, const double* x, const ApOut& o) {
+    TLR_SITE_PRE(ctx);
+    k_apply_split<3><<<(unsigned)nb * TC_SPC, 256, 0, ctx->stream>>>(pl.segs[q], T.row, b, x, TR, SC, eD, eU, eV, frag, ek, ef,
+                                                                             bad);
+    TLR_LAUNCH_CHECK(ctx);
+    TLR_SITE_PRE(ctx);
+    k_apply_nn_tc<<<(unsigned)((int64_t)nb * ((b + 15) / 16)), TC_T, TC_SMEM, ctx->stream>>>(T, dmode, pl.segs[q], frag, ek,
+                                                                                          ef, o, bad);
+    TLR_LAUNCH_CHECK(ctx);
+  };
+  if (op == TLR_OP_A) {  // kernel entries are at most 1, the diagonal's 1 + nugget
+    TLR_SITE_PRE(ctx);
+    k_apply_fill<<<blocks(np, 256), 256, 0, ctx->stream>>>(np, ilogb(std::max(1.0, 1.0 + M->kern.nugget)) + 1, eD);
+    TLR_LAUNCH_CHECK(ctx);
+  } else if (pl.ctas[2] > 0) {
+    T.pan = pl.lists[2];
+    T.npan = pl.npan[2];
+    TLR_SITE_PRE(ctx);
+    k_apply_colexp<<<(unsigned)pl.ctas[2], AP_T, 0, ctx->stream>>>(T, eU, eV, eD, bad);
+    TLR_LAUNCH_CHECK(ctx);
   }
+  ApOut fin{nullptr, nullptr, nullptr, Y, M->dperm, ldy, M->N, nr};
+  tn(0, Xp);
+  if (op == TLR_OP_A) {
+    nn(2, 1, Xp, fin);
+  } else if (op == TLR_OP_L) {
+    nn(2, 2, Xp, fin);
+  } else if (op == TLR_OP_LT) {
+    fin.add = YD;
+    nn(1, 0, Xp, fin);
+  } else {  // L (D) (L^T X); the first contraction has left the exponents of U's and the tiles' columns
+    ApOut mid{YD, M->state == 2 ? M->dvec : nullptr, Z, nullptr, nullptr, 0, 0, nr};
+    nn(1, 0, Xp, mid);
+    tn(1, Z);
+    nn(2, 2, Z, fin);
+  }
+  T.gate = bad;
+  apply_run<8, 2>(ctx, M, op, pl, T, nr, Xp, YD, Z, TR, SC, Y, ldy);
 }
 
 template <int VEC>
@@ -425,8 +1030,15 @@ void tlr_apply(tlr_ctx* ctx, const tlr_mat* M, int op, int nrhs, const double* X
     al(M->Urow[i]);
     al(M->Vcol[i]);
   }
+  // Tensor cores where the DFMAs (1.67 ps per entry and column) take longer than the tensor cores' passes (3.2 ps
+  // per entry for up to eight columns) and their five further launches (45 us): measured, DFMA / tensor cores, us:
+  // 6.7e8 entries 2412 / 2200 (2 columns), 9134 / 2202 (8); 3.6e7 213 / 241 (2), 284 / 241 (3), 608 / 240 (8);
+  // 4.8e6 108 / 121 (4), 132 / 123 (6), 155 / 124 (8); 1.4e6 101 / 106 (8).
+  const int ng = (nrhs + 7) / 8;  // right-hand sides in equal groups of at most eight
+  const double entries = 4.0 * b * (double)tr + (double)nb * b * b;
+  pl.tc = aligned && entries * (1.67 * ((nrhs + ng - 1) / ng) - 3.2) > 45e6;
   std::vector<ApPanel> pans;
-  int n0[3] = {0, 0, 0};
+  int n0[4] = {0, 0, 0, 0};
   auto list = [&](int l, bool v, bool u, bool dg) {
     int cta = 0;
     auto add = [&](const double* A, int64_t ncols, int blk, int kind) {
@@ -446,13 +1058,33 @@ void tlr_apply(tlr_ctx* ctx, const tlr_mat* M, int op, int nrhs, const double* X
   if (op == TLR_OP_A) list(0, true, true, false);
   else if (op == TLR_OP_L) list(0, true, false, false);
   else list(0, false, true, true);
-  if (op == TLR_OP_LLT) list(1, true, false, false);
+  list(1, op == TLR_OP_LLT, false, false);
+  list(2, pl.tc && (op == TLR_OP_LT || op == TLR_OP_LLT), pl.tc && op == TLR_OP_L, pl.tc && op == TLR_OP_L);
   // one table on the device: rows, panels, offsets
-  const size_t br = sizeof(ApRow) * nb, bp = sizeof(ApPanel) * pans.size(), bo = sizeof(int) * off.size();
-  std::vector<char> tab(br + bp + bo);
+  std::vector<TcSeg> segs;
+  for (int q = 0; pl.tc && q < 3; ++q) {
+    int64_t ks = 0;
+    for (int i = 0; i < nb; ++i) {
+      TcSeg g{ks, 0, 0, 0};
+      if (q == 0) g.n0 = b;                          // X
+      else if (q == 1) g.n2 = (int)M->vlen[i];       // S
+      else {                                         // [X; T; S] of A, [X; T] of L
+        g.n0 = b;
+        g.n1 = (int)M->ulen[i];
+        g.n2 = op == TLR_OP_A ? (int)M->vlen[i] : 0;
+      }
+      for (int n : {g.n0, g.n1, g.n2}) ks += (n + TC_KS - 1) / TC_KS;
+      segs.push_back(g);
+    }
+    pl.steps[q] = ks;
+  }
+  const size_t br = sizeof(ApRow) * nb, bp = sizeof(ApPanel) * pans.size(), bg = sizeof(TcSeg) * segs.size(),
+               bo = sizeof(int) * off.size();
+  std::vector<char> tab(br + bp + bg + bo);
   memcpy(tab.data(), rows.data(), br);
   if (bp) memcpy(tab.data() + br, pans.data(), bp);
-  memcpy(tab.data() + br + bp, off.data(), bo);
+  if (bg) memcpy(tab.data() + br + bp, segs.data(), bg);
+  memcpy(tab.data() + br + bp + bg, off.data(), bo);
   Buf btab(ctx), work(ctx);
   const char* dt;
   const size_t chunk = (size_t)16 << 20;
@@ -469,20 +1101,21 @@ void tlr_apply(tlr_ctx* ctx, const tlr_mat* M, int op, int nrhs, const double* X
   pl.T.row = reinterpret_cast<const ApRow*>(dt);
   pl.lists[0] = reinterpret_cast<const ApPanel*>(dt + br);
   pl.lists[1] = pl.lists[0] + n0[1];
-  pl.T.voff = reinterpret_cast<const int*>(dt + br + bp);
+  pl.lists[2] = pl.lists[0] + n0[2];
+  for (int q = 0; q < 3; ++q) pl.segs[q] = reinterpret_cast<const TcSeg*>(dt + br + bp) + (pl.tc ? (size_t)q * nb : 0);
+  pl.T.voff = reinterpret_cast<const int*>(dt + br + bp + bg);
   pl.T.uoff = pl.T.voff + tabn;
   pl.T.nb = nb;
   pl.T.b = b;
   pl.T.unit = M->state == 2;
   pl.R = tr;
   pl.np = (int64_t)nb * b;
-  // right-hand sides in equal groups of at most eight
-  const int ng = (nrhs + 7) / 8;
   for (int g = 0; g < ng; ++g) {
     const int c0 = (int)((int64_t)nrhs * g / ng), nr = (int)((int64_t)nrhs * (g + 1) / ng) - c0;
     const double* Xg = X + (size_t)c0 * ldx;
     double* Yg = Y + (size_t)c0 * ldy;
-    if (aligned) apply_width<2>(ctx, M, op, pl, nr, Xg, ldx, Yg, ldy, work);
+    if (pl.tc) apply_group_tc(ctx, M, op, pl, nr, Xg, ldx, Yg, ldy, work);
+    else if (aligned) apply_width<2>(ctx, M, op, pl, nr, Xg, ldx, Yg, ldy, work);
     else apply_width<1>(ctx, M, op, pl, nr, Xg, ldx, Yg, ldy, work);
   }
 }

@@ -84,6 +84,56 @@ def test_products_match_the_exported_tiles(T, N, d, b, eps, ldl):
 
 
 @pytest.mark.parametrize("N,d,b,eps,ldl", [
+    (3000, 3, 250, 1e-6, True),     # tiles and segments that end inside a step of 16
+    (4100, 2, 514, 1e-6, False),
+])
+def test_products_of_several_columns_on_the_tensor_cores(T, N, d, b, eps, ldl):
+    """Entries and coefficients are rounded to 2^-58 of their columns' bounds (at most twice the largest), so a term's
+    error is at most 2^-55.4 of the largest |a| |x| of its row block: n u max(|A| |X|) in all per contraction.
+    Columns that the digits cannot hold go through the FP64 kernels: they match the columns one by one."""
+    import torch
+    ctx = T.Context(0)
+    o = T.default_opts(bs=16, seed=N)
+    A = ctx.compress(inputs.points(N, d, N), b, eps, 0.1, 1e-3, o)
+    F = A.copy()
+    (F.ldlt if ldl else F.potrf)(eps, o)
+    DA, PA, _ = _dense(A, False)
+    L, PL, dv = _dense(F, True)
+    perm = A.perm()
+    u = 2.0 ** -53
+    rng = np.random.default_rng(N)
+    for nrhs, scale in ((7, 1.0), (8, 1e-200), (16, 1e200)):
+        X = rng.standard_normal((N, nrhs)) * scale * 10.0 ** rng.uniform(-3, 0, nrhs)
+        Xp = np.zeros((DA.shape[0], nrhs))
+        Xp[:N] = X[perm]
+        n = DA.shape[0] + int(max(A.ranks().sum(), F.ranks().sum()))
+        want = {
+            "A": (A, T.OP_A, DA @ Xp, PA @ np.abs(Xp), 1),
+            "L": (F, T.OP_L, L @ Xp, PL @ np.abs(Xp), 1),
+            "Lt": (F, T.OP_LT, L.T @ Xp, PL.T @ np.abs(Xp), 1),
+            "LLt": (F, T.OP_LLT, L @ (dv[:, None] * (L.T @ Xp)),
+                    PL @ (np.abs(dv)[:, None] * (PL.T @ np.abs(Xp))), 2),
+        }
+        for name, (M, op, Y, B, times) in want.items():
+            g = M.matvec(T.fortran(torch.tensor(X, device="cuda:0")), op).cpu().numpy()[perm]
+            assert np.all(np.abs(g - Y[:N]) <= 2 * times * n * u * B.max(0)), (name, nrhs)
+    X = rng.standard_normal((N, 8))
+    X[7, 1], X[N // 2, 2], X[N - 1, 3] = np.nan, np.inf, -np.inf
+    X[:, 4] *= 1e-300
+    X[:, 5] = 0
+    for M, op in ((A, T.OP_A), (F, T.OP_L), (F, T.OP_LT), (F, T.OP_LLT)):
+        g = M.matvec(T.fortran(torch.tensor(X, device="cuda:0")), op).cpu().numpy()
+        for c in range(8):
+            w = M.matvec(T.fortran(torch.tensor(X[:, c:c + 1], device="cuda:0")), op).cpu().numpy()[:, 0]
+            assert np.array_equal(np.isnan(g[:, c]), np.isnan(w)), (op, c)
+            f = np.isfinite(w)
+            assert np.array_equal(g[~f, c], w[~f], equal_nan=True), (op, c)
+            if f.any():
+                assert np.allclose(g[f, c], w[f], rtol=0, atol=1e-12 * np.abs(w[f]).max()), (op, c)
+    ctx.close()
+
+
+@pytest.mark.parametrize("N,d,b,eps,ldl", [
     (100, 2, 128, 1e-6, False),     # one tile, ragged
     (1000, 3, 64, 1e-4, True),      # L D L^T, ragged last tile
     (700, 2, 75, 1e-6, False),      # odd tile size: columns on 8-byte boundaries
