@@ -274,8 +274,10 @@ void add_rowsum_abs(tlr_ctx* ctx, int n, const double* E, int lde, double* A, in
 void logdet_reduce(tlr_ctx* ctx, int n, const double* diag_tiles, int b, int nb, const double* dvec,
                    double* out2 /*device: [sum log|.|, count negative]*/);
 // gi, grid: device workspace (N d) for the points' grid
+// work (device): kernel_matvec_work() bytes, or null for none
+size_t kernel_matvec_work(int64_t N);
 void kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell, double nugget,
-                   int nrhs, const double* X, int64_t ldx, double* Y, int64_t ldy, GridInfo* gi, long long* grid);
+                   int nrhs, const double* X, int64_t ldx, double* Y, int64_t ldy, GridInfo* gi, long long* grid, void* work);
 void copy_matrix(tlr_ctx* ctx, int m, int n, const double* X, int ldx, double* Y, int ldy);
 void to_float(tlr_ctx* ctx, int64_t n, const double* x, float* y);
 void to_double(tlr_ctx* ctx, int64_t n, const float* x, double* y);

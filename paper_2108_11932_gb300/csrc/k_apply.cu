@@ -29,6 +29,7 @@
 #include <cstring>
 
 #include "internal.h"
+#include "tcdigits.cuh"
 #include "warpsum.cuh"
 
 namespace cg = cooperative_groups;
@@ -320,10 +321,8 @@ __global__ void __launch_bounds__(AP_T) k_apply_nn(ApTab T, int dmode, int use_u
 // (mma.sync.m16n8k16, FP16 in, FP32 accumulate: the eight columns are its N, and a fragment's FP64 entries
 // are split in the registers that loaded them, so that the factor is read as it lies; tcgen05 wants its
 // operands in shared or tensor memory and 128 rows, which a panel of a few columns does not fill).  The
-// splitting is that of k_ozaki.cu (Ozaki, Ogita, Oishi and Rump, 2012) with balanced digits:
-//   x = 2^(e - 57) F, F = round(x 2^(57 - e)) = sum_{i=1..7} d_i 256^(7 - i), |d_1| <= 512, -128 <= d_i <= 127
-// where 2^e bounds the operand's column: a panel column's own bound for the factor, the block's for each
-// right-hand side.  Pairs with i + j <= 9 are kept (34 products a step; the dropped ones are 2^-66 of the
+// splitting is that of tcdigits.cuh, seven digits below a bound 2^e of the operand's column: a panel column's own
+// bound for the factor, the block's for each right-hand side.  Pairs with i + j <= 9 are kept (34 products a step; the dropped ones are 2^-66 of the
 // bounds); a group of equal i + j sums below 13 2^14 4 16 < 2^24 over four steps, exact in FP32, and moves to
 // 64-bit integers then; one rounding at the end.  Error: 2^-58 of the bounds per entry and factor, against FP64's
 // 2^-53 of the running sum per term: of A X, L X, L^T X and L (D) L^T X in 2D and 3D, eps 1e-8 to 1e-2, normal,
@@ -334,85 +333,18 @@ __global__ void __launch_bounds__(AP_T) k_apply_nn(ApTab T, int dmode, int use_u
 // Bound: the integer instructions that split (about 18 per entry, at half rate; the ALU is busy 57 % of the
 // time, the tensor pipe 32 %, 16 warps per SM at 126 registers).  34 products of 16 x 8 x 16 per 256 entries.
 // Latency: each lane copies its own fragments of the next steps into shared memory (cp.async, no barrier).
-constexpr int TC_P = 7;      // digits
 constexpr int TC_KS = 16;    // k per step
-constexpr int TC_WIN = 4;    // steps of an exact window
 constexpr int TC_STG = 3;    // steps in flight per warp
 constexpr int TC_SPC = 8;    // CTAs (a cluster) per block in k_apply_split
 constexpr int TC_FRAG = 64;  // uint4 per step of a split right-hand side: [2][lane], the words of tc_digits with the sign on top
 constexpr int TC_W = 4, TC_T = 32 * TC_W;  // warps of k_apply_tn_tc and k_apply_nn_tc
 constexpr int TC_SMEM = TC_W * TC_STG * 32 * (64 + 32 + 16);
 
-// Exponent e with |x| < 2^e for the largest |x| whose high word is hw (1 for a zero column: any bound will do)
-__device__ __forceinline__ int tc_exp(unsigned hw) { return hw == 0 ? 1 : (int)(hw >> 20) - 1022; }
-// a column of tiny, huge or non-finite numbers
-__device__ __forceinline__ bool tc_odd(int e) { return e < -900 || e > 900; }
-// What tc_pairs takes of a column with |x| < 2^e (-900 <= e <= 900)
-__device__ __forceinline__ int tc_shift(int e) { return (e + 1022) << 20; }
-// |F| + 0x6600808080808080 as two words: the bytes are d_7 + 128, ..., d_2 + 128 and the FP16 number 1536 + d_1.
-// Rounds to nearest; the sign of bad is set unless |x| < 2^e; zeros and denormals give 0.
-__device__ __forceinline__ uint2 tc_digits(double x, int shift, int& bad) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  // |x| 2^(58 - e) = (mantissa 2^5) >> (e + 1022 - exponent field)
-  const int t = shift - (int)(hi & 0x7ff00000u);
-  bad |= t;
-  unsigned long long w = ((unsigned long long)((__funnelshift_l(lo, hi, 5) & 0x01ffffffu) | 0x02000000u) << 32) | (lo << 5);
-  asm("shr.u64 %0, %0, %1;" : "+l"(w) : "r"((unsigned)t >> 20));  // 0 from 64 on
-  w = (w + (2 * 0x6600808080808080ull + 1)) >> 1;
-  return make_uint2((unsigned)w, (unsigned)(w >> 32));
-}
-__device__ __forceinline__ unsigned tc_fma2(unsigned a, unsigned b, unsigned c) {
-  unsigned r;
-  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
-  return r;
-}
-// the seven digit pairs of entries a, b with the signs of the high words sa, sb: FP16 (1024 + byte) s - (1024 + 128) s
-__device__ __forceinline__ void tc_pairs(uint2 a, uint2 b, unsigned sa, unsigned sb, unsigned (&d)[TC_P]) {
-  const unsigned p0 = __byte_perm(a.x, b.x, 0x5140u), p1 = __byte_perm(a.x, b.x, 0x7362u), p2 = __byte_perm(a.y, b.y, 0x5140u);
-  const unsigned sg = __byte_perm(sa, sb, 0x7632u) & 0x80008000u;
-  const unsigned one = 0x64646464u, s = sg ^ 0x3c003c00u, bias = sg ^ 0xe480e480u, bias1 = sg ^ 0xe600e600u;
-  d[6] = tc_fma2(__byte_perm(p0, one, 0x4140u), s, bias);  // byte 0: the least significant digit
-  d[5] = tc_fma2(__byte_perm(p0, one, 0x4342u), s, bias);
-  d[4] = tc_fma2(__byte_perm(p1, one, 0x4140u), s, bias);
-  d[3] = tc_fma2(__byte_perm(p1, one, 0x4342u), s, bias);
-  d[2] = tc_fma2(__byte_perm(p2, one, 0x4140u), s, bias);
-  d[1] = tc_fma2(__byte_perm(p2, one, 0x4342u), s, bias);
-  d[0] = tc_fma2(__byte_perm(a.y, b.y, 0x7632u), s, bias1);
-}
 __device__ __forceinline__ void tc_mma(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-struct TcAcc {  // group sums of a window; the totals: hi of the groups 0-3, lo of 4-7 (weights 256^-g)
-  float f[8][4];
-  long long hi[4], lo[4];
-  int win, bad;
-};
-__device__ __forceinline__ void tc_init(TcAcc& a) {
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    a.hi[c] = a.lo[c] = 0;
-#pragma unroll
-    for (int g = 0; g < 8; ++g) a.f[g][c] = 0.f;
-  }
-  a.win = a.bad = 0;
-}
-__device__ __forceinline__ void tc_drain(TcAcc& a) {
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    long long h = 0, l = 0;
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      h = h * 256 + __float2int_rn(a.f[g][c]);
-      l = l * 256 + __float2int_rn(a.f[g + 4][c]);
-      a.f[g][c] = a.f[g + 4][c] = 0.f;
-    }
-    a.hi[c] += h;
-    a.lo[c] += l;
-  }
-  a.win = 0;
 }
 // One step (CHECK: notes entries outside their bounds): the tile's fragments x[row half][k half][2] (rows g, g + 8; k 2t, 2t + 1, 2t + 8, 2t + 9 of the lane
 // g = lane / 4, t = lane % 4) with shifts e, times the split right-hand side's step (column g; the same k)
@@ -437,10 +369,6 @@ __device__ __forceinline__ void tc_step(const double (&x)[2][2][2], const int (&
   }
   if (CHECK) acc.bad |= bad;
   if (++acc.win == TC_WIN) tc_drain(acc);
-}
-// value of a total: digits i, j carry 2^(-1 - 8 i) each (i, j from 1): group g = i + j - 2 carries 2^(-18 - 8 g)
-__device__ __forceinline__ double tc_value(long long hi, long long lo, int e) {
-  return ldexp(fma((double)hi, 4294967296.0, (double)lo), e - 74);
 }
 // The warps' totals through shared memory: thread `threadIdx.x` < 128 gets entry (lane / 4 + 8 (c / 2), 2 (lane % 4) + c % 2)
 // of the fragment, lane = threadIdx.x / 4, c = threadIdx.x % 4

@@ -5,6 +5,7 @@
 
 #include "common.h"
 #include "cholqr.cuh"
+#include "tcdigits.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -148,6 +149,50 @@ __device__ __forceinline__ double entry(uint64_t hi, uint64_t lo, int ezb, uint6
   const uint64_t M53 = (Vn >> 11) + ((Vn >> 10) & 1ull);                      // nearest, may carry to 2^53
   const uint64_t bits = ((uint64_t)(1025 - lzv - (int)(n >> 6)) << 52) + (M53 - (1ull << 52));
   return __longlong_as_double((long long)bits);
+}
+
+// The same as a digit word of tcdigits.cuh: exp(-c sqrt(S) 2^-q) 2^57, rounded, for the products that add entries up in
+// fixed point (absolute error below 2^-57: 2^-58 of rounding, 2^-60 of the steps taken in 32 bits).
+// c 64/ln2 = Cm 2^(e - 63) (Cm in [2^63, 2^64)), ezb = e + 63 - q; needs z < 2^8 (GridInfo::ok).
+__device__ __forceinline__ uint64_t shr(uint64_t x, int n) {  // 0 from 64 on
+  uint64_t r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"((unsigned)n));
+  return r;
+}
+__device__ __forceinline__ uint2 entry_word(uint64_t hi, uint64_t lo, int ezb, uint64_t Cm, const uint64_t* tab) {
+  int lz = hi ? __clzll((long long)hi) : 64 + __clzll((long long)lo);
+  lz &= ~1;
+  uint64_t H;
+  if (lz == 0) H = hi;
+  else if (lz < 64) H = (hi << lz) | (lo >> (64 - lz));
+  else H = lo << (lz & 63);
+  const unsigned top = (unsigned)(H >> 63);
+  const unsigned fb = ((127u + top) << 23) | (unsigned)((H >> (39 + top)) & 0x7fffffu);
+  const unsigned yb = __float_as_uint(rsqrtf(__uint_as_float(fb)));
+  const int ey = (int)((yb >> 23) & 0xffu) - 127;
+  const uint64_t Y0 = (uint64_t)((yb & 0x7fffffu) | 0x800000u) << (39 + ey);  // Q62
+  const uint64_t G0 = __umul64hi(H, Y0);                                      // F y0, Q60
+  const long long h = (long long)((1ull << 58) - __umul64hi(G0, Y0));         // 1 - F y0^2, Q58, below 2^39
+  const int hs = (int)(h >> 12);                                              // Q46
+  const long long corr = h * 8 + ((3 * ((long long)hs * hs)) >> 33);          // h/2 + 3h^2/8, Q62
+  const uint64_t G = G0 + (uint64_t)(__mul64hi((long long)G0, corr) * 4);     // sqrt(F), Q60
+  const uint64_t P = __umul64hi(G, Cm);                                       // z 64/ln2 = P 2^(ez - 59)
+  const int ez = ezb - lz / 2, fs = 5 + ez;
+  const int n = (int)shr(P, 59 - ez);
+  const uint64_t frac = fs >= 0 ? P << (fs & 63) : shr(P, -fs);               // Q64 fraction of n
+  // exp(-rho): the innermost steps of the Horner form matter by rho^3 and less and take 32-bit operands
+  const uint64_t rho = __umul64hi(frac, L70);                                 // Q70
+  const unsigned r32 = (unsigned)(rho >> 32);                                 // Q38
+  const unsigned a5 = 2290649225u - (__umulhi(r32, 3054198967u) >> 9);        // 1/5! (Q38) - rho / 6! (Q41)
+  const uint64_t a4 = F4 - (((uint64_t)r32 * a5) >> 14);                      // Q62
+  const uint64_t a3 = F3 - (((uint64_t)r32 * (unsigned)(a4 >> 26)) >> 12);
+  const uint64_t a2 = F2 - (__umul64hi(rho, a3) >> 6);
+  const uint64_t a1 = F1 - (__umul64hi(rho, a2) >> 6);
+  const uint64_t E = (1ull << 62) - (__umul64hi(rho, a1) >> 6);
+  const uint64_t V = __umul64hi(tab[n & 63], E);                              // Q61
+  uint64_t w = (hi | lo) ? shr(V, 3 + (n >> 6)) : 1ull << 58;                 // Q58
+  w = (w + (2 * 0x6600808080808080ull + 1)) >> 1;
+  return make_uint2((unsigned)w, (unsigned)(w >> 32));
 }
 }  // namespace fx
 
@@ -799,15 +844,214 @@ void logdet_reduce(tlr_ctx* ctx, int n, const double* diag_tiles, int b, int nb,
 // A lane owns a row and the CTA's eight warps share the columns (each stages 32 of them at a time for
 // itself, no CTA barrier in the loop), a cluster of S CTAs splits them further so that small N fills the
 // GPU; partial sums are added in warp and rank order.
-// Measured: N = 32768, 3D, 4 right-hand sides 81.3 -> 16.3 ms (the FP64 products of 4 columns are 6.9 ms of it).
+// Measured: N = 32768, 3D, 4 right-hand sides 81.3 -> 16.3 ms.  Large products go through k_kernel_tc (below) and come
+// here only with points or right-hand sides that it does not take (ef: the bounds that decide).
 constexpr int KMV_W = 8, KMV_T = 32 * KMV_W, KMV_R = 8;
+
+// Large products: an entry is formed once for itself and its mirror image, and the products leave the FP64 unit.  A
+// warp forms 16 rows x 8 columns of entries as digit words (fx::entry_word) in the layout of an mma.m16n8k8 fragment
+// and multiplies their digits with those of up to eight right-hand sides (tcdigits.cuh); the transposed digits serve
+// the mirror image.  Integer totals: neither the split over CTAs nor the order of the additions changes a bit.
+// Bound: the integer pipe (about 230 instructions an entry; the digits and their products 70).  Measured: N = 32768,
+// 3D, 4 columns 16.3 -> 10.2 ms (k_kernel_matvec alone; without the mirror images 15.8); error against extended
+// precision 0.1 to 0.8 of k_kernel_matvec's (1D to 3D, ell 0.02 to 3, right-hand sides over eight decades).
+constexpr int KTC_NONE = (int)0x80808080;  // exponent of a column without a nonzero entry, as memset leaves it
+__device__ __forceinline__ int kmv_exp(int e) { return e == KTC_NONE ? 1 : e; }
+// the grid resolves the points and the digits hold the right-hand sides; otherwise k_kernel_matvec does it all
+__device__ __forceinline__ bool kmv_tc_ok(const GridInfo* gi, const int* ef) {
+  bool ok = gi->ok;
+#pragma unroll
+  for (int n = 0; n < 8; ++n) ok &= !tc_odd(kmv_exp(ef[n]));
+  return ok;
+}
+// ef[n]: exponent of column n's bound
+__global__ void __launch_bounds__(256) k_kernel_bound(int64_t N, const double* __restrict__ X, int64_t ldx, int* ef) {
+  const int n = blockIdx.y;
+  unsigned m = 0;
+  for (int64_t i = blockIdx.x * 256 + threadIdx.x; i < N; i += (int64_t)gridDim.x * 256)
+    m = max(m, (unsigned)__double2hiint(X[i + n * ldx]) & 0x7fffffffu);
+  for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(ef + n, tc_exp(m));
+}
+// digit words of the right-hand sides, [step of 8 rows][lane]: rows 2 t and 2 t + 1 of column lane / 4, t = lane % 4
+__global__ void __launch_bounds__(256) k_kernel_split(int64_t N, int nr, const double* __restrict__ X, int64_t ldx,
+                                                      const int* __restrict__ ef, uint4* __restrict__ frag) {
+  const int64_t e = blockIdx.x * (int64_t)256 + threadIdx.x;
+  const int64_t i = e / 32 * 8 + 2 * (e & 3);
+  const int n = (int)(e >> 2) & 7;
+  if (e / 32 * 8 >= N) return;
+  uint2 w[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const double x = i + u < N && n < nr ? X[i + u + n * ldx] : 0.0;
+    const int ex = kmv_exp(ef[n]);
+    int bad = 0;
+    w[u] = tc_digits(x, tc_shift(tc_odd(ex) ? 1 : ex), bad);
+    w[u].y |= (unsigned)__double2hiint(x) & 0x80000000u;
+  }
+  frag[e] = make_uint4(w[0].x, w[0].y, w[1].x, w[1].y);
+}
+__device__ __forceinline__ unsigned ktc_trans(unsigned a) {
+  unsigned r;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(a));
+  return r;
+}
+// CTA (I, c): 128 rows I (a warp 16 of them) times the column blocks c CH .. of 128, up to the diagonal block.  Left of the
+// diagonal block each entry serves its mirror image as well: the transposed fragments (movmatrix) are the B operand of the
+// right-hand sides' rows, and a step's eight columns go to the totals at once.
+template <int D>
+__global__ void __launch_bounds__(KMV_T, 2) k_kernel_tc(const long long* __restrict__ grid, const GridInfo* __restrict__ gi,
+                                                        int64_t N, uint64_t Cm, int ec, int nr, int CH,
+                                                        const uint4* __restrict__ frag, const int* __restrict__ ef,
+                                                        unsigned long long* __restrict__ sums) {
+  if (!kmv_tc_ok(gi, ef)) return;
+  __shared__ uint64_t tab[64];
+  __shared__ uint4 xrow[KMV_W][4][32];  // digit pairs of the right-hand sides' rows (A operand): [digit / 2][lane]
+  if (threadIdx.x < 64) tab[threadIdx.x] = fx::TAB[threadIdx.x];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  // row blocks a CH .. (a + 1) CH - 1 have a + 1 chunks of columns each
+  const int64_t idx = blockIdx.x;
+  int64_t a = (int64_t)((sqrtf(8.f * (float)idx / (float)CH + 1.f) - 1.f) * 0.5f);
+  while (a > 0 && CH * a * (a + 1) / 2 > idx) --a;
+  while (CH * (a + 1) * (a + 2) / 2 <= idx) ++a;
+  const int rem = (int)(idx - CH * a * (a + 1) / 2), I = (int)a * CH + rem / (int)(a + 1), chunk = rem % (int)(a + 1);
+  const int64_t r0 = ((int64_t)I * KMV_W + warp) * 16;
+  const int steps = (int)((N + 7) / 8);
+  {
+    unsigned d[2][TC_P + 1];
+    d[0][TC_P] = d[1][TC_P] = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int64_t s = r0 / 8 + h;
+      const uint4 f = s < steps ? __ldg(frag + s * 32 + lane) : make_uint4(0x80808080u, 0x66008080u, 0x80808080u, 0x66008080u);
+      unsigned e[TC_P];
+      tc_pairs(make_uint2(f.x, f.y & 0x7fffffffu), make_uint2(f.z, f.w & 0x7fffffffu), f.y, f.w, e);
+#pragma unroll
+      for (int i = 0; i < TC_P; ++i) d[h][i] = e[i];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) xrow[warp][q][lane] = make_uint4(d[0][2 * q], d[1][2 * q], d[0][2 * q + 1], d[1][2 * q + 1]);
+  }
+  __syncthreads();
+  if (r0 >= N) return;
+  const int ezb = ec + 63 - gi->q;
+  long long xr[2][D];
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int k = 0; k < D; ++k) xr[r][k] = grid[min(r0 + g + 8 * r, N - 1) * D + k];
+  TcAcc acc;
+  tc_init(acc);
+  const int s1 = min(min((chunk + 1) * CH, I + 1) * 16, steps);
+#pragma unroll 1
+  for (int s = chunk * CH * 16; s < s1; ++s) {
+    const uint4 f = __ldg(frag + (int64_t)s * 32 + lane);
+    unsigned d0[TC_P], d1[TC_P];
+    {
+      uint2 w[2][2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        long long xc[D];
+#pragma unroll
+        for (int k = 0; k < D; ++k) xc[k] = __ldg(grid + min((int64_t)s * 8 + 2 * t + q, N - 1) * D + k);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          uint64_t hi = 0, lo = 0;
+#pragma unroll
+          for (int k = 0; k < D; ++k) {
+            const long long df = xr[r][k] - xc[k];
+            const uint64_t v = (uint64_t)(df < 0 ? -df : df);
+            const uint64_t l = v * v;
+            lo += l;
+            hi += __umul64hi(v, v) + (lo < l ? 1ull : 0ull);
+          }
+          w[r][q] = fx::entry_word(hi, lo, ezb, Cm, tab);
+        }
+      }
+      tc_pairs(w[0][0], w[0][1], 0u, 0u, d0);
+      tc_pairs(w[1][0], w[1][1], 0u, 0u, d1);
+    }
+    unsigned b[TC_P];
+    tc_pairs(make_uint2(f.x, f.y & 0x7fffffffu), make_uint2(f.z, f.w & 0x7fffffffu), f.y, f.w, b);
+#pragma unroll
+    for (int i = 0; i < TC_P; ++i)
+#pragma unroll
+      for (int j = 0; j < TC_P; ++j)
+        if (i + j <= 7)
+          asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+                       : "+f"(acc.f[i + j][0]), "+f"(acc.f[i + j][1]), "+f"(acc.f[i + j][2]), "+f"(acc.f[i + j][3])
+                       : "r"(d0[i]), "r"(d1[i]), "r"(b[j]));
+    if (++acc.win == 2 * TC_WIN) tc_drain(acc);
+    if (s >= I * 16) continue;  // the diagonal block has its mirror image itself
+    float cf[8][2];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) cf[q][0] = cf[q][1] = 0.f;
+#pragma unroll
+    for (int i = 0; i < TC_P; ++i) {
+      d0[i] = ktc_trans(d0[i]);
+      d1[i] = ktc_trans(d1[i]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint4 x = xrow[warp][q][lane];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int j = 2 * q + u;
+        const unsigned x0 = u ? x.z : x.x, x1 = u ? x.w : x.y;
+#pragma unroll
+        for (int i = 0; i < TC_P; ++i)
+          if (j < TC_P && i + j <= 7) {
+            float n0, n1;
+            asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%8,%5,%8}, {%6,%7}, {%0,%1,%9,%9};"
+                         : "+f"(cf[i + j][0]), "+f"(cf[i + j][1]), "=f"(n0), "=f"(n1)
+                         : "r"(x0), "r"(x1), "r"(d0[i]), "r"(d1[i]), "r"(0u), "f"(0.f));
+          }
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      long long h = 0, l = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        h = h * 256 + __float2int_rn(cf[q][c]);
+        l = l * 256 + __float2int_rn(cf[q + 4][c]);
+      }
+      if (g < nr) {
+        unsigned long long* o = sums + ((int64_t)(s * 8 + 2 * t + c) * 8 + g) * 2;
+        atomicAdd(o, (unsigned long long)h);
+        atomicAdd(o + 1, (unsigned long long)l);
+      }
+    }
+  }
+  tc_drain(acc);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int64_t i = r0 + g + 8 * (c >> 1);
+    const int n = 2 * t + (c & 1);
+    if (i < N && n < nr) {
+      atomicAdd(sums + (i * 8 + n) * 2, (unsigned long long)acc.hi[c]);
+      atomicAdd(sums + (i * 8 + n) * 2 + 1, (unsigned long long)acc.lo[c]);
+    }
+  }
+}
+__global__ void __launch_bounds__(256) k_kernel_join(const GridInfo* __restrict__ gi, int64_t N, int nr, double nugget,
+                                                     const unsigned long long* __restrict__ sums, const int* __restrict__ ef,
+                                                     const double* __restrict__ X, int64_t ldx, double* __restrict__ Y, int64_t ldy) {
+  const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
+  if (i >= N || !kmv_tc_ok(gi, ef)) return;
+  for (int n = 0; n < nr; ++n)
+    Y[i + n * ldy] = tc_value((long long)sums[(i * 8 + n) * 2], (long long)sums[(i * 8 + n) * 2 + 1], kmv_exp(ef[n])) +
+                     nugget * X[i + n * ldx];
+}
+
 template <int D, int NR>
 __global__ void __launch_bounds__(KMV_T) k_kernel_matvec(const double* __restrict__ pts,
                                                         const long long* __restrict__ grid,
                                                         const GridInfo* __restrict__ gi, int64_t N, uint64_t Cm, int ec,
                                                         double inv_ell, double nugget, int nr, int S,
                                                         const double* __restrict__ X, int64_t ldx,
-                                                        double* __restrict__ Y, int64_t ldy) {
+                                                        double* __restrict__ Y, int64_t ldy, const int* ef) {
+  if (ef && kmv_tc_ok(gi, ef)) return;  // done on the tensor cores
   __shared__ uint64_t tab[64];
   __shared__ long long sp[KMV_W][32][D];  // grid points, or the bits of the coordinates
   __shared__ __align__(16) double sx[KMV_W][32][NR];
@@ -895,7 +1139,7 @@ __global__ void __launch_bounds__(KMV_T) k_kernel_matvec(const double* __restric
 template <int D, int NR>
 static void kernel_matvec_launch(tlr_ctx* ctx, const double* pts, const long long* grid, const GridInfo* gi, int64_t N,
                                  uint64_t Cm, int ec, double ell, double nugget, int nr, const double* X, int64_t ldx,
-                                 double* Y, int64_t ldy) {
+                                 double* Y, int64_t ldy, const int* ef) {
   const int64_t rbs = (N + 31) / 32;
   // CTAs sharing 32 rows: about 32 per SM in all (a CTA's work is then small against the whole, so the
   // last wave is short), while each keeps a 32-column block for every warp
@@ -913,35 +1157,70 @@ static void kernel_matvec_launch(tlr_ctx* ctx, const double* pts, const long lon
   cf.numAttrs = 1;
   TLR_SITE_PRE(ctx);
   TLR_CUDA(cudaLaunchKernelEx(&cf, k_kernel_matvec<D, NR>, pts, grid, gi, N, Cm, ec, 1.0 / ell, nugget, nr, S, X, ldx, Y,
-                              ldy));
+                              ldy, ef));
   TLR_LAUNCH_CHECK(ctx);
 }
 
 template <int D>
 static void kernel_matvec_d(tlr_ctx* ctx, const double* pts, const long long* grid, const GridInfo* gi, int64_t N,
                             uint64_t Cm, int ec, double ell, double nugget, int nr, const double* X, int64_t ldx,
-                            double* Y, int64_t ldy) {
-  if (nr == 1) kernel_matvec_launch<D, 1>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy);
-  else if (nr == 2) kernel_matvec_launch<D, 2>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy);
-  else if (nr <= 4) kernel_matvec_launch<D, 4>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy);
-  else kernel_matvec_launch<D, KMV_R>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy);
+                            double* Y, int64_t ldy, const int* ef) {
+  if (nr == 1) kernel_matvec_launch<D, 1>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef);
+  else if (nr == 2) kernel_matvec_launch<D, 2>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef);
+  else if (nr <= 4) kernel_matvec_launch<D, 4>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef);
+  else kernel_matvec_launch<D, KMV_R>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef);
+}
+
+// Tensor cores from 3000 points on (DFMA / tensor cores, 4 columns, us: N = 2048, 3D 161 / 170; 4096, 2D 358 / 282;
+// 8192, 3D 1140 / 754; 32768, 3D 16277 / 10257; the same within 10 % for 1 and 8 columns); the totals of 2^20 points
+// stay below 2^63.
+size_t kernel_matvec_work(int64_t N) {
+  return N >= 3000 && N <= (1 << 20) ? (size_t)((N + 7) / 8 * 512 + N * 128 + 256) : 0;
 }
 
 void kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell, double nugget, int nrhs,
-                   const double* X, int64_t ldx, double* Y, int64_t ldy, GridInfo* gi, long long* grid) {
+                   const double* X, int64_t ldx, double* Y, int64_t ldy, GridInfo* gi, long long* grid, void* work) {
   if (nrhs <= 0) return;
   grid_points(ctx, pts, N, d, ell, gi, grid);
   int ec;
   uint64_t Cm;
   fx_scale(ell, Cm, ec);
+  const unsigned __int128 c64 = (unsigned __int128)Cm * fx::KQ;  // 64/ln2 of it: 2^126 or a little less
+  const int lz = c64 >> 127 ? 0 : c64 >> 126 ? 1 : 2;
+  const uint64_t Ct = (uint64_t)((c64 << lz) >> 64);
+  const int et = ec + 8 - lz;
   const int ng = (nrhs + KMV_R - 1) / KMV_R;  // right-hand sides in equal groups
   for (int g = 0; g < ng; ++g) {
     const int c0 = (int)((int64_t)nrhs * g / ng), nr = (int)((int64_t)nrhs * (g + 1) / ng) - c0;
     const double* Xg = X + c0 * ldx;
     double* Yg = Y + c0 * ldy;
-    if (d == 1) kernel_matvec_d<1>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy);
-    else if (d == 2) kernel_matvec_d<2>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy);
-    else kernel_matvec_d<3>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy);
+    int* ef = static_cast<int*>(work);
+    if (work) {
+      uint4* frag = reinterpret_cast<uint4*>(static_cast<char*>(work) + 256);
+      unsigned long long* sums = reinterpret_cast<unsigned long long*>(frag + (N + 7) / 8 * 32);
+      TLR_CUDA(cudaMemsetAsync(ef, 0x80, 32, ctx->stream));
+      TLR_CUDA(cudaMemsetAsync(sums, 0, (size_t)N * 128, ctx->stream));
+      TLR_SITE_PRE(ctx);
+      k_kernel_bound<<<dim3(std::min(cdiv(N, 1024), 128u), (unsigned)nr), 256, 0, ctx->stream>>>(N, Xg, ldx, ef);
+      TLR_LAUNCH_CHECK(ctx);
+      TLR_SITE_PRE(ctx);
+      k_kernel_split<<<cdiv((N + 7) / 8 * 32, 256), 256, 0, ctx->stream>>>(N, nr, Xg, ldx, ef, frag);
+      TLR_LAUNCH_CHECK(ctx);
+      // column blocks per CTA: at least 8 CTAs per SM in all, and at most 16 blocks
+      const int64_t rbs = (N + 127) / 128;
+      const int CH = (int)std::max<int64_t>(1, std::min<int64_t>(16, rbs * rbs / 2 / (8 * 152)));
+      const int64_t na = rbs / CH, ctas = CH * na * (na + 1) / 2 + (rbs - na * CH) * (na + 1);
+      auto kern = d == 1 ? k_kernel_tc<1> : d == 2 ? k_kernel_tc<2> : k_kernel_tc<3>;
+      TLR_SITE_PRE(ctx);
+      kern<<<(unsigned)ctas, KMV_T, 0, ctx->stream>>>(grid, gi, N, Ct, et, nr, CH, frag, ef, sums);
+      TLR_LAUNCH_CHECK(ctx);
+      TLR_SITE_PRE(ctx);
+      k_kernel_join<<<cdiv(N, 256), 256, 0, ctx->stream>>>(gi, N, nr, nugget, sums, ef, Xg, ldx, Yg, ldy);
+      TLR_LAUNCH_CHECK(ctx);
+    }
+    if (d == 1) kernel_matvec_d<1>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy, ef);
+    else if (d == 2) kernel_matvec_d<2>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy, ef);
+    else kernel_matvec_d<3>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy, ef);
   }
 }
 

@@ -81,7 +81,7 @@ extern "C" tlr_status tlr_kernel_matvec_noalloc(void* cuda_stream, const double*
   launch_ctx.stream = stream;
   try {
     tlr::kernel_matvec(&launch_ctx, pts, N, d, kern->ell, kern->nugget, nrhs, X, ldx, Y, ldy,
-                       info, grid);
+                       info, grid, nullptr);
   } catch (const tlr::Error& e) {
     cudaGetLastError();  // a failed launch leaves its error pending: do not hand it to the caller's next call
     return e.status;

@@ -1299,7 +1299,9 @@ tlr_status tlr_kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, 
   long long* grid = reinterpret_cast<long long*>(dp + (size_t)N * d);
   GridInfo* gi = reinterpret_cast<GridInfo*>(dp + (size_t)2 * N * d);
   TLR_CUDA(cudaMemcpyAsync(dp, pts, sizeof(double) * N * d, cudaMemcpyHostToDevice, ctx->stream));
-  kernel_matvec(ctx, dp, N, d, kern->ell, kern->nugget, nrhs, X, ldx, Y, ldy, gi, grid);
+  Buf bw(ctx);
+  const size_t work = kernel_matvec_work(N);
+  kernel_matvec(ctx, dp, N, d, kern->ell, kern->nugget, nrhs, X, ldx, Y, ldy, gi, grid, work ? bw.need<char>(work) : nullptr);
   TLR_CUDA(cudaStreamSynchronize(ctx->stream));
   return TLR_OK;
   ABI_END

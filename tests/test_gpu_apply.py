@@ -193,6 +193,40 @@ def test_kernel_product_matches_dense(T, N, d, ell, scale, nrhs):
     ctx.close()
 
 
+@pytest.mark.parametrize("N,d,ell,nrhs", [
+    (3000, 2, 0.1, 1),            # ragged last row block
+    (3073, 1, 0.02, 9),           # one row in the last block; two groups
+    (4096, 3, 0.2, 8),
+    (3300, 3, 0.01, 3),           # extent above 64 ell: FP64 entries
+])
+def test_large_kernel_products_match_dense(T, N, d, ell, nrhs):
+    """As above, plus the fixed-point rounding of entries (2^-57) and right-hand sides (2^-58 of a bound of at most twice
+    the largest): N 2^-55 of the largest."""
+    import torch
+    ctx = T.Context(0)
+    x = inputs.points(N, d, N)
+    x[7] = x[60]  # coincident points
+    z = np.sqrt(((x[:, None, :] - x[None, :, :]) ** 2).sum(-1)) / ell
+    A = np.exp(-z) + 1e-3 * np.eye(N)
+    rng = np.random.default_rng(N)
+    for scale in (1.0, 1e-150, 1e200, 1e-305):
+        X = rng.standard_normal((N, nrhs)) * scale * 10.0 ** rng.uniform(-2, 0, nrhs)
+        g = ctx.kernel_matvec(x, ell, 1e-3, T.fortran(torch.tensor(X, device="cuda:0"))).cpu().numpy()
+        B = (A * 2 * (N + 4 * (1 + z) + 4) * 2.0 ** -52) @ np.abs(X) + N * 2.0 ** -55 * np.abs(X).max(0)
+        assert np.all(np.abs(g - A @ X) <= B), scale
+    X = np.abs(rng.standard_normal((N, nrhs)))
+    X[N // 2, 0] = np.inf
+    if nrhs > 1:
+        X[N - 1, 1] = np.nan
+    g = ctx.kernel_matvec(x, ell, 1e-3, T.fortran(torch.tensor(X, device="cuda:0"))).cpu().numpy()
+    want = A @ X
+    assert np.array_equal(np.isnan(g[:, 1:]), np.isnan(want[:, 1:]))
+    assert np.isinf(g[:, 0]).all() and np.all(g[:, 0] > 0)
+    f = np.isfinite(want)
+    assert np.allclose(g[f], want[f], rtol=1e-10, atol=0)
+    ctx.close()
+
+
 def test_kernel_product_of_non_finite_points_is_nan(T):
     import torch
     ctx = T.Context(0)
