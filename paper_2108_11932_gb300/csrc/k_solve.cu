@@ -264,19 +264,19 @@ __global__ void __launch_bounds__(SV_T, 1) k_solve(SvTab T, SvVec v) {
         if (lane < RB) red[((n << rsh) + lane) * SV_RLD + warp] = acc[n];
       }
       __syncthreads();
-      // warp partials: four lanes per output
+      // warp partials: four lanes per output, whole warps (the lanes leave the waits below at different times)
 #pragma unroll 1
-      for (int o = tid >> 2; o < RB * NR; o += SV_T / 4) {
-        const double* r = red + o * SV_RLD + (tid & 3) * (SV_W / 4);
-        const bool out = is_out(o);
+      for (int o0 = warp * 8; o0 < RB * NR; o0 += SV_T / 4) {
+        const int o = o0 + (lane >> 2);
+        const bool live = o < RB * NR, out = live && is_out(o);
+        const double* r = red + (live ? o : 0) * SV_RLD + (tid & 3) * (SV_W / 4);
         double old = old0;
         if (out && o >= SV_T / 4) old = before(o);
         double z = r[0];
 #pragma unroll
         for (int w = 1; w < SV_W / 4; ++w) z += r[w];
-        const unsigned mask = __activemask();  // whole groups of four
-        z += __shfl_xor_sync(mask, z, 1);
-        z += __shfl_xor_sync(mask, z, 2);
+        z += __shfl_xor_sync(0xffffffffu, z, 1);
+        z += __shfl_xor_sync(0xffffffffu, z, 2);
         if (out) {
           if (s.kind == 1) {
             sv_st(v.Z + at(o), z);
