@@ -264,8 +264,9 @@ tlr_status tlr_poll(tlr_ctx* ctx, uint64_t ticket, tlr_result* res, double* x, i
  * The factor keeps its step list and the work arrays of the widest solve so far
  * (allocated on the first solve, freed with the factor).  Solves with one factor
  * must not run concurrently (they share the work arrays).  Every device wait is
- * bounded: should one run out, the result is NaN and the context's next solve
- * returns TLR_ERR_TIMEOUT. */
+ * bounded: should one run out, the result is NaN and the context's next tlr_solve
+ * or tlr_pcg returns TLR_ERR_TIMEOUT.  (tlr_pcg and the serving queue wait for
+ * their own solves and report them themselves.) */
 tlr_status tlr_solve(tlr_ctx* ctx, const tlr_mat* F, int nrhs, double* B, int64_t ldb);
 
 /* Preconditioned conjugate gradients (Section 6: a low-accuracy TLR factor of

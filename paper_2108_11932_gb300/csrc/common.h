@@ -112,7 +112,7 @@ struct tlr_ctx {
   size_t split_ctr_cap[2] = {0, 0};
   // grid-barrier words of the fused orthogonalization kernel: {arrivals, generation} per stream
   unsigned* orth_bar = nullptr;
-  // host-visible word that a solve's grid barrier sets when its bounded wait runs out
+  // host-visible word that a solve sets when one of its bounded waits runs out
   int* wait_out = nullptr;
   // Small host-pinned status buffer for per-round device->host reads.
   void* hstatus = nullptr;

@@ -138,7 +138,9 @@ inline double* Vptr(const tlr_mat* M, int i, int j) { return M->Vcol[j] + (size_
 void mat_free_storage(tlr_ctx* ctx, tlr_mat* M);
 void mat_drop_plans(tlr_ctx* ctx, tlr_mat* M);  // solve plan of M
 void plan_destroy(tlr_ctx* ctx, SolvePlan* P);
-// B <- F^-1 B, original point order (k_solve.cu)
+// 1 if a bounded wait of a solve that the caller has waited for ran out since the last call (then cleared)
+bool solve_timeout_flag(tlr_ctx* ctx);
+// B <- F^-1 B, original point order (k_solve.cu); reports a wait that ran out in an earlier solve
 void tlr_solve_factor(tlr_ctx* ctx, tlr_mat* F, int nrhs, double* B, int64_t ldb);
 void mat_destroy(tlr_ctx* ctx, tlr_mat* M);
 tlr_mat* mat_new(int64_t N, int d, int b);

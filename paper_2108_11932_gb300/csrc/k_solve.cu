@@ -551,11 +551,15 @@ static void solve_launch(tlr_ctx* ctx, const SolvePlan* P, SvVec v) {
   TLR_LAUNCH_CHECK(ctx);
 }
 
+bool solve_timeout_flag(tlr_ctx* ctx) {
+  volatile int* out = ctx->wait_out;
+  if (!*out) return false;
+  *out = 0;
+  return true;
+}
+
 void tlr_solve_factor(tlr_ctx* ctx, tlr_mat* F, int nrhs, double* B, int64_t ldb) {
-  if (*ctx->wait_out) {
-    *ctx->wait_out = 0;
-    throw Error(TLR_ERR_TIMEOUT, "solve: a bounded device wait of an earlier solve ran out");
-  }
+  TLR_REQUIRE(!solve_timeout_flag(ctx), TLR_ERR_TIMEOUT, "solve: a bounded device wait of an earlier solve ran out");
   if (!F->plan) F->plan = plan_build(ctx, F);
   SolvePlan* P = F->plan;
   const int ng32 = (nrhs + SV_NRHS - 1) / SV_NRHS;
@@ -676,3 +680,6 @@ void pcg_update_p(tlr_ctx* ctx, int64_t n, int ncols, const double* num, const d
 }
 
 }  // namespace tlr
+
+// The word that a solve's bounded waits set, for tests that set it from the host (not part of the C API).
+extern "C" int* tlr_solve_wait_word(tlr_ctx* ctx) { return ctx->wait_out; }

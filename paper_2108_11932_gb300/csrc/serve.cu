@@ -98,6 +98,7 @@ struct Server {
         q.x.resize(n);
         TLR_CUDA(cudaMemcpyAsync(q.x.data(), B, sizeof(double) * n, cudaMemcpyDeviceToHost, ctx->stream));
         TLR_CUDA(cudaStreamSynchronize(ctx->stream));
+        if (solve_timeout_flag(ctx)) st = TLR_ERR_TIMEOUT;  // this request's own solve
       }
       dfree(ctx, B);
       q.rhs.clear();

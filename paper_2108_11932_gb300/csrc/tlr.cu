@@ -1197,6 +1197,9 @@ tlr_status tlr_pcg(tlr_ctx* ctx, const tlr_mat* A, const tlr_mat* F, int nrhs, c
   auto check = [](tlr_status st, const char* what) {
     if (st != TLR_OK) throw Error(st, what);
   };
+  auto check_solves = [&]() {  // after a synchronization: the preconditioner's solves so far
+    TLR_REQUIRE(!solve_timeout_flag(ctx), TLR_ERR_TIMEOUT, "pcg: a bounded device wait of a solve ran out");
+  };
   Buf bR(ctx), bP(ctx), bQ(ctx), bZ(ctx), bS(ctx);
   double* R = bR.need<double>((size_t)n * nrhs);
   double* P = bP.need<double>((size_t)n * nrhs);
@@ -1234,6 +1237,7 @@ tlr_status tlr_pcg(tlr_ctx* ctx, const tlr_mat* A, const tlr_mat* F, int nrhs, c
     pcg_update_xr(ctx, n, nrhs, rz[cur], pq, da, X, ldx, P, R, Q, n);
     coldot(ctx, n, nrhs, R, n, R, n, rr);
     d2h_sync(ctx, h, rr, sizeof(double) * nrhs);
+    check_solves();
     for (int c = 0; c < nrhs; ++c)
       if (act[c] && (std::sqrt(h[c]) <= tol * std::sqrt(hb[c]) || it == maxit)) {
         act[c] = 0;
@@ -1254,6 +1258,7 @@ tlr_status tlr_pcg(tlr_ctx* ctx, const tlr_mat* A, const tlr_mat* F, int nrhs, c
   axpy_matrix(ctx, (int)n, nrhs, -1.0, Q, (int)n, R, (int)n);
   coldot(ctx, n, nrhs, R, n, R, n, rr);
   d2h_sync(ctx, h, rr, sizeof(double) * nrhs);
+  check_solves();
   for (int c = 0; c < nrhs; ++c) relres[c] = hb[c] > 0.0 ? std::sqrt(h[c] / hb[c]) : 0.0;
   return TLR_OK;
   ABI_END
