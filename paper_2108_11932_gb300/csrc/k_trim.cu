@@ -359,37 +359,46 @@ void trim_tiles(tlr_ctx* ctx, int b, const std::vector<TrimTile>& tiles, double 
     g.js.push_back(d);
   }
   // the clusters on the main stream, the single-CTA tiles beside them on the side stream
-  const bool fork = nbig > 0 && nbig < nt && ctx->side && ctx->stream == ctx->main;
-  if (fork) {
+  // (joined on every way out: the side stream's launches read the workspace and the job tables)
+  struct Side {
+    tlr_ctx* ctx;
+    cudaStream_t saved;
+    bool open = false;
+    void join() {
+      if (!open) return;
+      open = false;
+      TLR_CUDA(cudaEventRecord(ctx->ev_join, ctx->side));
+      TLR_CUDA(cudaStreamWaitEvent(ctx->main, ctx->ev_join, 0));
+    }
+    ~Side() {
+      ctx->stream = saved;
+      if (open && (cudaEventRecord(ctx->ev_join, ctx->side) != cudaSuccess ||
+                   cudaStreamWaitEvent(ctx->main, ctx->ev_join, 0) != cudaSuccess))
+        cudaStreamSynchronize(ctx->side);
+    }
+  } side{ctx, ctx->stream};
+  if (nbig > 0 && nbig < nt && ctx->side && ctx->stream == ctx->main) {
     TLR_CUDA(cudaEventRecord(ctx->ev_fork, ctx->main));
     TLR_CUDA(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+    side.open = true;
   }
   for (auto& kv : groups) {
     Group& g = kv.second;
     std::stable_sort(g.js.begin(), g.js.end(), [](const TrimDev& x, const TrimDev& y) { return x.r > y.r; });
     const size_t sm = trim_smem(b, g.rmax, g.cs, g.sm);
-    cudaStream_t saved = ctx->stream;
-    if (fork && g.cs == 1) ctx->stream = ctx->side;
-    try {
-      for (size_t o = 0; o < g.js.size(); o += 65535) {
-        const int cnt = (int)std::min<size_t>(65535, g.js.size() - o);
-        const TrimDev* dj = static_cast<const TrimDev*>(upload(ctx, g.js.data() + o, sizeof(TrimDev) * cnt));
-        if (g.cs == 8 && g.sm) trim_launch<8, true>(ctx, dj, cnt, sm, b, eps);
-        else if (g.cs == 8) trim_launch<8, false>(ctx, dj, cnt, sm, b, eps);
-        else if (g.cs == 4) trim_launch<4, true>(ctx, dj, cnt, sm, b, eps);
-        else if (g.sm) trim_launch<1, true>(ctx, dj, cnt, sm, b, eps);
-        else trim_launch<1, false>(ctx, dj, cnt, sm, b, eps);
-      }
-    } catch (...) {
-      ctx->stream = saved;
-      throw;
+    ctx->stream = side.open && g.cs == 1 ? ctx->side : side.saved;
+    for (size_t o = 0; o < g.js.size(); o += 65535) {
+      const int cnt = (int)std::min<size_t>(65535, g.js.size() - o);
+      const TrimDev* dj = static_cast<const TrimDev*>(upload(ctx, g.js.data() + o, sizeof(TrimDev) * cnt));
+      if (g.cs == 8 && g.sm) trim_launch<8, true>(ctx, dj, cnt, sm, b, eps);
+      else if (g.cs == 8) trim_launch<8, false>(ctx, dj, cnt, sm, b, eps);
+      else if (g.cs == 4) trim_launch<4, true>(ctx, dj, cnt, sm, b, eps);
+      else if (g.sm) trim_launch<1, true>(ctx, dj, cnt, sm, b, eps);
+      else trim_launch<1, false>(ctx, dj, cnt, sm, b, eps);
     }
-    ctx->stream = saved;
   }
-  if (fork) {
-    TLR_CUDA(cudaEventRecord(ctx->ev_join, ctx->side));
-    TLR_CUDA(cudaStreamWaitEvent(ctx->main, ctx->ev_join, 0));
-  }
+  ctx->stream = side.saved;
+  side.join();
   TLR_CUDA(cudaMemcpyAsync(rank.data(), dr, sizeof(int) * nt, cudaMemcpyDeviceToHost, ctx->stream));
   TLR_CUDA(cudaStreamSynchronize(ctx->stream));
 }
