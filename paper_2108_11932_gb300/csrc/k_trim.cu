@@ -74,6 +74,30 @@ __device__ __forceinline__ double recip_approx(double v) {
   return fma(y, fma(-v, y, 1.0), y);
 }
 
+// Lane gl's share, of L lanes, of the inner product of two columns of r entries, to be added up over the lanes by
+// halving exchanges (o = L / 2, .., 1).  The sum is that of 32 chains, chain c of the rows c, c + 32, .., added in
+// halves whatever L is: lane gl holds the chains gl, gl + L, ..
+template <int L, class LD>
+__device__ __forceinline__ double pair_dot(const double* x, const double* y, int r, int gl, LD ld) {
+  constexpr int C = 32 / L;
+  double a[C];
+#pragma unroll
+  for (int u = 0; u < C; ++u) a[u] = 0.0;
+  int m = gl;
+#pragma unroll(C < 4 ? 4 / C : 1)
+  for (; m + (C - 1) * L < r; m += 32)
+#pragma unroll
+    for (int u = 0; u < C; ++u) a[u] = fma(ld(x + m + u * L), ld(y + m + u * L), a[u]);
+#pragma unroll
+  for (int u = 0; u < C - 1; ++u)
+    if (m + u * L < r) a[u] = fma(ld(x + m + u * L), ld(y + m + u * L), a[u]);
+#pragma unroll
+  for (int h = C / 2; h; h /= 2)
+#pragma unroll
+    for (int u = 0; u < h; ++u) a[u] += a[u + h];
+  return a[0];
+}
+
 // CS: CTAs of the tile's cluster.  SM: X and the norms live in shared memory, column c in CTA c % CS at place
 // c / CS; otherwise in global memory.
 template <int CS, bool SM>
@@ -148,8 +172,8 @@ __global__ void __launch_bounds__(TR_T) k_trim(const TrimDev* __restrict__ jobs,
   }
   // ---- one-sided Jacobi on X, round-robin pairs (position 0 fixed, 1 .. n-1 rotating); pair k is CTA k % CS's
   const int n = r + (r & 1), np = n / 2, mine = (np - rank + CS - 1) / CS;
-  int L = 32;  // lanes of a pair
-  while (L > 1 && mine * L > TR_T) L >>= 1;
+  int L = 32;  // lanes of a pair (pair_dot)
+  while (L > 4 && mine * L > TR_T) L >>= 1;
   const int G = TR_T / L, grp = tid / L, gl = tid % L;
   const double tol2 = ((double)r * 0x1p-53) * ((double)r * 0x1p-53);
   auto norms = [&]() {  // squared norms of this CTA's columns
@@ -189,8 +213,10 @@ __global__ void __launch_bounds__(TR_T) k_trim(const TrimDev* __restrict__ jobs,
         if (live) {
           xp = col(p);
           xq = col(q);
-#pragma unroll 4
-          for (int m = gl; m < r; m += L) g = fma(ld(xp + m), ld(xq + m), g);
+          g = L == 32   ? pair_dot<32>(xp, xq, r, gl, ld)
+              : L == 16 ? pair_dot<16>(xp, xq, r, gl, ld)
+              : L == 8  ? pair_dot<8>(xp, xq, r, gl, ld)
+                        : pair_dot<4>(xp, xq, r, gl, ld);
         }
         for (int o = L >> 1; o; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
         if (gl == 0) gs[grp] = g;
