@@ -66,12 +66,41 @@ __device__ double block_sum(double v, double* red) {
   return s;
 }
 
-// 1 / v to an ulp or two by two Newton steps (the angle it enters is corrected by later rotations); v normal
+// 1 / v by two Newton steps, v normal.  (Any tangent makes an orthogonal rotation; one that is off by a few ulps is
+// corrected by later rotations.)
 __device__ __forceinline__ double recip_approx(double v) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
   y = fma(y, fma(-v, y, 1.0), y);
   return fma(y, fma(-v, y, 1.0), y);
+}
+
+// Whether columns with squared norms a, b and inner product g are to be rotated (g^2 > tol2 a b), and the tangent of
+// the rotation, 2 g / (d + sign(d) sqrt(d^2 + 4 g^2)) with d = b - a
+__device__ __forceinline__ bool rotation_in_range(double a, double b, double g, double tol2, double& t) {
+  const double d = b - a, g2 = 2.0 * g, h = fma(d, d, g2 * g2);
+  if (!(g * g > tol2 * (a * b))) return false;
+  const double hs = h * rsqrt(h);
+  t = (d >= 0.0 ? g2 : -g2) * recip_approx(fabs(d) + hs);
+  return true;
+}
+__device__ __forceinline__ int exp_field(double x) { return (int)((unsigned)__double2hiint(x) >> 20 & 0x7ffu); }
+// 2^(1023 - f) for a biased exponent f in 1 .. 2045
+__device__ __forceinline__ double pow2_inv(int f) { return __hiloint2double((2046 - f) << 20, 0); }
+// The squares of a, b and g leave FP64's range (norms beyond about 2^+-225): the same on numbers scaled by powers of
+// two, a and b to order one each for the test and to the larger of them for the angle
+__device__ __noinline__ bool rotation_scaled(double a, double b, double g, double tol2, double& t) {
+  const int fa = min(max(exp_field(a), 1), 2045), fb = min(max(exp_field(b), 1), 2045), odd = (fa ^ fb) & 1;
+  const double gn = g * pow2_inv((fa + fb + odd) / 2), an = a * pow2_inv(fa), bn = b * pow2_inv(min(fb + odd, 2045));
+  if (!(gn * gn > tol2 * (an * bn))) return false;
+  const double sc = pow2_inv(max(fa, fb));
+  t = 0.0;
+  return rotation_in_range(a * sc, b * sc, g * sc, -1.0, t);
+}
+__device__ __forceinline__ bool rotation(double a, double b, double g, double tol2, double& t) {
+  const unsigned fa = exp_field(a) - 573, fb = exp_field(b) - 573;  // 2^-450 .. 2^450
+  if (max(fa, fb) <= 900u) return rotation_in_range(a, b, g, tol2, t);
+  return rotation_scaled(a, b, g, tol2, t);
 }
 
 // Lane gl's share, of L lanes, of the inner product of two columns of r entries, to be added up over the lanes by
@@ -229,10 +258,8 @@ __global__ void __launch_bounds__(TR_T) k_trim(const TrimDev* __restrict__ jobs,
           if (i2 < mine && q2 < r) {
             double *ap = nrm(p2), *bp = nrm(q2);
             const double aa = ld(ap), bb = ld(bp), gg = gs[tid];
-            if (gg * gg > tol2 * (aa * bb)) {
-              // tan of the rotation: 2 g / (d + sign(d) sqrt(d^2 + 4 g^2)), d = b - a
-              const double d = bb - aa, g2 = 2.0 * gg, h = fma(d, d, g2 * g2);
-              const double hs = h * rsqrt(h), tt = (d >= 0.0 ? g2 : -g2) * recip_approx(fabs(d) + hs);
+            double tt;
+            if (rotation(aa, bb, gg, tol2, tt)) {
               c = rsqrt(fma(tt, tt, 1.0));
               s = c * tt;
               *ap = fma(-tt, gg, aa);

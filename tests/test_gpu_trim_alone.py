@@ -36,3 +36,15 @@ def test_a_tile_alone_and_among_others(T, b, r, counts):
         for (q0, b0), (q1, b1) in zip(got[0], g):
             assert np.array_equal(q0, q1) and np.array_equal(b0, b1)
     ctx.close()
+
+
+@pytest.mark.parametrize("nt,b,r", [(2, 96, 40), (1, 128, 75), (24, 128, 57)])
+@pytest.mark.parametrize("k", [-290, 300])
+def test_powers_of_two_scale_the_result(T, nt, b, r, k):
+    """2^k B has the singular values and vectors of B, the former times 2^k: no square leaves the range of FP64 that a
+    column's norm (and its square) stays in."""
+    ctx = T.Context(0)
+    Q, B, _ = inputs.lowrank_tiles(nt, b, r, seed=b + r, smin=1e-6)
+    for (q0, b0), (q1, b1) in zip(_trim(T, ctx, Q, B, 1e-5), _trim(T, ctx, Q, np.ldexp(B, k), np.ldexp(1e-5, k))):
+        assert np.array_equal(q0, q1) and np.array_equal(np.ldexp(b0, k), b1)
+    ctx.close()
