@@ -114,6 +114,8 @@ struct tlr_ctx {
   unsigned* orth_bar = nullptr;
   // host-visible word that a solve sets when one of its bounded waits runs out
   int* wait_out = nullptr;
+  // most rounds per slot that the blocks of samples formed ahead have held in a run (ara_run)
+  double sample_rounds_per_slot = 0;
   // Small host-pinned status buffer for per-round device->host reads.
   void* hstatus = nullptr;
   size_t hstatus_cap = 0;

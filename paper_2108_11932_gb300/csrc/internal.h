@@ -25,6 +25,14 @@ struct Buf {
     cap = 0;
   }
   template <typename T>
+  T* exact(size_t elems) {  // anew, without the room that need() adds
+    release();
+    const size_t bytes = std::max<size_t>(elems * sizeof(T), 256);
+    p = dalloc(ctx, bytes);
+    cap = bytes;
+    return static_cast<T*>(p);
+  }
+  template <typename T>
   T* need(size_t elems) {
     const size_t bytes = std::max<size_t>(elems * sizeof(T), 256);
     if (bytes > cap) {

@@ -436,26 +436,51 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
   std::vector<double> thr_h(slots);
 
   // Samples of m rounds of an operand, formed in one product; rounds next .. m - 1 are still to be used.
-  // Their blocks are kept by size and handed on (everything runs on one stream).
+  // A block that an operand has done with serves the next request of as many rounds or fewer (everything runs on one
+  // stream).  The blocks hold at most `most` rounds per slot, the largest request so far: past that a request gets a
+  // smaller block, and with it fewer rounds ahead, which changes no result.
   struct Ahead {
     double* Y = nullptr;
-    int m = 0, next = 0;
+    int m = 0, next = 0, size = 0;  // size: rounds of the block
   };
   std::vector<Ahead> have(nops);
   std::vector<std::unique_ptr<Buf>> pool;
-  std::map<int, std::vector<double*>> spare;
-  auto take = [&](int m) -> double* {
-    std::vector<double*>& f = spare[m];
-    if (f.empty()) {
-      const int64_t one = (int64_t)m * nmax * bs * (int64_t)sizeof(double);
-      const int n = (int)std::max<int64_t>(1, std::min<int64_t>(slots, ((int64_t)64 << 20) / one));  // allocated together
-      pool.emplace_back(new Buf(ctx));
-      double* p = pool.back()->need<double>((size_t)n * m * nmax * bs);
-      for (int i = 0; i < n; ++i) f.push_back(p + (size_t)i * m * nmax * bs);
+  std::multimap<int, double*> spare;  // free blocks by size
+  int64_t held = 0;                   // rounds of all blocks
+  int most = 1;
+  // blocks for the requests of h[.].m rounds (their largest first); new ones in one allocation
+  auto take = [&](std::vector<Ahead*>& hs) {
+    std::vector<Ahead*> fresh;
+    int64_t rounds = 0;
+    for (const Ahead* h : hs) most = std::max(most, h->m);
+    std::stable_sort(hs.begin(), hs.end(), [](const Ahead* a, const Ahead* c) { return a->m > c->m; });
+    for (Ahead* h : hs) {
+      auto it = spare.lower_bound(h->m);
+      if (it == spare.end() && held + rounds + h->m > (int64_t)most * slots) {
+        if (!spare.empty()) it = std::prev(spare.end());
+        else h->m = 1;
+      }
+      if (it == spare.end()) {
+        h->size = h->m;
+        rounds += h->m;
+        fresh.push_back(h);
+        continue;
+      }
+      h->size = it->first;
+      h->m = std::min(h->m, h->size);
+      h->Y = it->second;
+      spare.erase(it);
     }
-    double* p = f.back();
-    f.pop_back();
-    return p;
+    if (fresh.empty()) return;
+    const size_t one = (size_t)nmax * bs;
+    pool.emplace_back(new Buf(ctx));
+    double* p = pool.back()->exact<double>((size_t)rounds * one);
+    for (Ahead* h : fresh) {
+      h->Y = p;
+      p += h->m * one;
+    }
+    held += rounds;
+    ctx->sample_rounds_per_slot = std::max(ctx->sample_rounds_per_slot, (double)held / slots);
   };
 
   std::vector<int> active;
@@ -473,16 +498,20 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
     {
       std::vector<int> ops, ts, ms;
       std::vector<double*> ydst;
+      std::vector<Ahead*> need;
       for (int op : active) {
         Ahead& h = have[op];
         if (h.next < h.m) continue;
         h.next = 0;
         h.m = std::max(1, S.ahead(op, round[op], ns));
-        h.Y = take(h.m);
+        need.push_back(&h);
         ops.push_back(op);
         ts.push_back(round[op]);
-        ms.push_back(h.m);
-        ydst.push_back(h.Y);
+      }
+      take(need);
+      for (int op : ops) {
+        ms.push_back(have[op].m);
+        ydst.push_back(have[op].Y);
       }
       if (!Om) {
         if (!ops.empty()) S.sample(ops, ts, ms, nullptr, ydst);
@@ -612,7 +641,7 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
       Ahead& h = have[op];
       if (done || h.next == h.m) {
         if (h.next < h.m) S.unused(op, h.m - h.next);
-        spare[h.m].push_back(h.Y);
+        spare.emplace(h.size, h.Y);
         h = Ahead();
       }
     }
@@ -1573,6 +1602,9 @@ tlr_status tlr_fp64_peak(tlr_ctx* ctx, double* tflops) {
 }
 
 int64_t tlr_launch_count(const tlr_ctx* ctx) { return ctx ? ctx->launches : -1; }
+
+// The largest sample_rounds_per_slot of a context, for tests (not part of the C API).
+double tlr_sample_rounds_per_slot(const tlr_ctx* ctx) { return ctx->sample_rounds_per_slot; }
 
 tlr_status tlr_gemm_stats(tlr_ctx* ctx, int enable, double* ms, double* flops, double* bytes, int64_t* launches) {
   if (!ctx) return TLR_ERR_ARG;
