@@ -146,6 +146,8 @@ inline double* Vptr(const tlr_mat* M, int i, int j) { return M->Vcol[j] + (size_
 void mat_free_storage(tlr_ctx* ctx, tlr_mat* M);
 void mat_drop_plans(tlr_ctx* ctx, tlr_mat* M);  // solve plan of M
 void plan_destroy(tlr_ctx* ctx, SolvePlan* P);
+// doubles of a solve's work vectors for a factor of np (padded) rows and R columns in its U panels
+size_t solve_doubles(int64_t np, int64_t R, bool ldl, int nrhs);
 // 1 if a bounded wait of a solve that the caller has waited for ran out since the last call (then cleared)
 bool solve_timeout_flag(tlr_ctx* ctx);
 // B <- F^-1 B, original point order (k_solve.cu); reports a wait that ran out in an earlier solve

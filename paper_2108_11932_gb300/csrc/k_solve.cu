@@ -551,6 +551,22 @@ static void solve_launch(tlr_ctx* ctx, const SolvePlan* P, SvVec v) {
   TLR_LAUNCH_CHECK(ctx);
 }
 
+// Right-hand sides go in equal launches of at most 32 columns, each in equal groups of at most 8: launches, the groups of
+// a launch of nc columns, and the columns that a group is computed in
+static int solve_launches(int nrhs) { return (nrhs + SV_NRHS - 1) / SV_NRHS; }
+static int solve_groups(int nc) { return (nc + 7) / 8; }
+static int solve_width(int nc) {
+  const int w = (nc + solve_groups(nc) - 1) / solve_groups(nc);
+  return w <= 4 ? w : w <= 6 ? 6 : 8;
+}
+static size_t solve_vectors(int64_t np, int64_t ldt, bool ldl) { return (ldl ? 6 : 5) * (size_t)np + 2 * (size_t)ldt; }
+
+size_t solve_doubles(int64_t np, int64_t R, bool ldl, int nrhs) {
+  if (nrhs <= 0) return 0;
+  const int nc = (nrhs + solve_launches(nrhs) - 1) / solve_launches(nrhs);  // the widest launch
+  return solve_vectors(np, std::max<int64_t>(R, 1), ldl) * solve_groups(nc) * solve_width(nc) + 32;
+}
+
 bool solve_timeout_flag(tlr_ctx* ctx) {
   volatile int* out = ctx->wait_out;
   if (!*out) return false;
@@ -562,11 +578,11 @@ void tlr_solve_factor(tlr_ctx* ctx, tlr_mat* F, int nrhs, double* B, int64_t ldb
   TLR_REQUIRE(!solve_timeout_flag(ctx), TLR_ERR_TIMEOUT, "solve: a bounded device wait of an earlier solve ran out");
   if (!F->plan) F->plan = plan_build(ctx, F);
   SolvePlan* P = F->plan;
-  const int ng32 = (nrhs + SV_NRHS - 1) / SV_NRHS;
-  for (int h = 0; h < ng32; ++h) {  // equal launches of at most 32 columns, each in equal groups of at most 8
+  const int ng32 = solve_launches(nrhs);
+  for (int h = 0; h < ng32; ++h) {
     const int c0 = (int)((int64_t)nrhs * h / ng32), nc = (int)((int64_t)nrhs * (h + 1) / ng32) - c0;
-    const int ng = (nc + 7) / 8, w = (nc + ng - 1) / ng, nr = w <= 4 ? w : w <= 6 ? 6 : 8, cols = ng * nr;
-    const size_t one = (P->T.dvec ? 6 : 5) * (size_t)P->np + 2 * (size_t)P->ldt;
+    const int ng = solve_groups(nc), nr = solve_width(nc), cols = ng * nr;
+    const size_t one = solve_vectors(P->np, P->ldt, P->T.dvec != nullptr);
     if (cols > P->cols) {
       dfree(ctx, P->vec);
       P->vec = nullptr;

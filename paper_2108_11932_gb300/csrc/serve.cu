@@ -52,14 +52,17 @@ struct Server {
   // and the inverses of the factor's diagonal tiles (3 N b), the low-rank factors of A and of L at a
   // mean rank estimated from eps and the dimension (exponential kernels: ranks grow like log(1/eps),
   // roughly twice as fast in 3D), their 7-bit chunk planes for the tensor-core products, the ARA
-  // workspace, the points and right-hand sides.
+  // workspace with the samples formed ahead, the points and right-hand sides, and the solve's vectors.
   static size_t footprint(const tlr_request& r) {
     const double nb = std::ceil((double)r.N / r.b);
     const double rbar = std::max(4.0, 3.0 * std::log10(1.0 / r.eps)) * (r.d >= 3 ? 2.0 : 1.0);
     const double lowrank = 2.0 * 2.0 * (nb * (nb - 1.0) / 2.0) * r.b * rbar;  // A and L, U and V
     const double planes = 3.0 * (nb * (nb - 1.0) / 2.0) * r.b * rbar;         // int8: 3 bytes per 8
-    const double work = nb * r.b * (double)(r.b + 64);
-    return (size_t)(8.0 * (3.0 * nb * r.b * r.b + lowrank + work + (double)r.N * (r.d + r.nrhs)) + planes);
+    const int bs = r.opts.bs > 0 ? r.opts.bs : 16;
+    const double ahead = std::min(8.0, std::ceil(0.9 * rbar / bs) + 1.0);     // rounds sampled in one product
+    const double work = nb * r.b * (double)(r.b + 64 + ahead * bs);
+    const double solve = solve_doubles((int64_t)nb * r.b, (int64_t)(nb * (nb - 1.0) / 2.0 * rbar), r.ldl != 0, r.nrhs);
+    return (size_t)(8.0 * (3.0 * nb * r.b * r.b + lowrank + work + solve + (double)r.N * (r.d + r.nrhs)) + planes);
   }
 
   tlr_status build(Req& q, bool shifted) {
@@ -160,6 +163,9 @@ void server_destroy(tlr_ctx* ctx) {
 using namespace tlr;
 
 extern "C" {
+
+// The admission's estimate of a request's device bytes, for tests (not part of the C API).
+size_t tlr_request_footprint(const tlr_request* r) { return Server::footprint(*r); }
 
 tlr_status tlr_submit(tlr_ctx* ctx, const tlr_request* r, uint64_t* ticket) {
   if (!ctx || !r || !ticket || !r->points || r->N <= 0 || r->d < 1 || r->d > 3 || r->b < 1 || !(r->eps > 0) ||
