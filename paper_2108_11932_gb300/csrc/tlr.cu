@@ -632,6 +632,14 @@ void ara_run(tlr_ctx* ctx, Sampler& S, const std::vector<int>& nrow, const std::
       st.rounds++;
       const int conv = hs[2 * s], nk2 = hs[2 * s + 1];
       bool done = conv != 0;
+      if (conv && !fused) {  // the products that the slot skipped above
+        const double nq = 2.0 * n * q[op] * bs, nn = 2.0 * n * bs * bs;
+        st.flops -= 2.0 * nq + 2.0 * nn;
+        if (ctx->kprof) {
+          ctx->kfam_flops[NN] -= nq + 2.0 * nn;
+          ctx->kfam_flops[TN] -= nq + nn;
+        }
+      }
       if (!done) {
         q[op] = std::min(q[op] + nk2, n);
         if (q[op] >= n || nk2 == 0) done = true;  // full basis, or no progress possible
