@@ -853,8 +853,14 @@ constexpr int KMV_W = 8, KMV_T = 32 * KMV_W, KMV_R = 8;
 // and multiplies their digits with those of up to eight right-hand sides (tcdigits.cuh); the transposed digits serve
 // the mirror image.  Integer totals: neither the split over CTAs nor the order of the additions changes a bit.
 // Bound: the integer pipe (about 230 instructions an entry; the digits and their products 70).  Measured: N = 32768,
-// 3D, 4 columns 16.3 -> 10.2 ms (k_kernel_matvec alone; without the mirror images 15.8); error against extended
+// 3D, 4 columns 16.3 -> 10.3 ms (k_kernel_matvec alone; without the mirror images 15.8); error against extended
 // precision 0.1 to 0.8 of k_kernel_matvec's (1D to 3D, ell 0.02 to 3, right-hand sides over eight decades).
+//
+// Accuracy, row by row: an entry is off by up to 2^-58 and a right-hand side by 2^-58 of its column's bound 2^e, so a
+// result by up to N 2^-57 2^e whatever its own terms are, where FP64 has N 2^-53 sum_j |a_ij x_j|.  So the sums of
+// |a_ij x_j| are estimated on the way (one product more per step, of the leading digits' absolute values: nothing of a
+// number below 2^-10 of its bound, at most twice a larger one, four times the sum), and blocks of 32 rows with one
+// below 2^e / 2 are computed by k_kernel_matvec (a unit vector's far rows, values of very different sizes).
 constexpr int KTC_NONE = (int)0x80808080;  // exponent of a column without a nonzero entry, as memset leaves it
 __device__ __forceinline__ int kmv_exp(int e) { return e == KTC_NONE ? 1 : e; }
 // the grid resolves the points and the digits hold the right-hand sides; otherwise k_kernel_matvec does it all
@@ -903,7 +909,8 @@ template <int D>
 __global__ void __launch_bounds__(KMV_T, 2) k_kernel_tc(const long long* __restrict__ grid, const GridInfo* __restrict__ gi,
                                                         int64_t N, uint64_t Cm, int ec, int nr, int CH,
                                                         const uint4* __restrict__ frag, const int* __restrict__ ef,
-                                                        unsigned long long* __restrict__ sums) {
+                                                        unsigned long long* __restrict__ sums, unsigned* __restrict__ est,
+                                                        int sh) {
   if (!kmv_tc_ok(gi, ef)) return;
   __shared__ uint64_t tab[64];
   __shared__ uint4 xrow[KMV_W][4][32];  // digit pairs of the right-hand sides' rows (A operand): [digit / 2][lane]
@@ -942,6 +949,7 @@ __global__ void __launch_bounds__(KMV_T, 2) k_kernel_tc(const long long* __restr
     for (int k = 0; k < D; ++k) xr[r][k] = grid[min(r0 + g + 8 * r, N - 1) * D + k];
   TcAcc acc;
   tc_init(acc);
+  unsigned sa = 0, sb = 0;  // FP16 sums of |a x| 2^11 below 2^e: columns 2 t and 2 t + 1 of rows g and g + 8
   const int s1 = min(min((chunk + 1) * CH, I + 1) * 16, steps);
 #pragma unroll 1
   for (int s = chunk * CH * 16; s < s1; ++s) {
@@ -981,9 +989,12 @@ __global__ void __launch_bounds__(KMV_T, 2) k_kernel_tc(const long long* __restr
           asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
                        : "+f"(acc.f[i + j][0]), "+f"(acc.f[i + j][1]), "+f"(acc.f[i + j][2]), "+f"(acc.f[i + j][3])
                        : "r"(d0[i]), "r"(d1[i]), "r"(b[j]));
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f16.f16.f16.f16 {%0,%1}, {%2,%3}, {%4}, {%0,%1};"
+                 : "+r"(sa), "+r"(sb)
+                 : "r"(d0[0]), "r"(d1[0]), "r"(tc_mul2(b[0] & 0x7fff7fffu, 0x20002000u)));  // 2^-7
     if (++acc.win == 2 * TC_WIN) tc_drain(acc);
     if (s >= I * 16) continue;  // the diagonal block has its mirror image itself
-    float cf[8][2];
+    float cf[8][2], ce[2];
 #pragma unroll
     for (int q = 0; q < 8; ++q) cf[q][0] = cf[q][1] = 0.f;
 #pragma unroll
@@ -994,6 +1005,12 @@ __global__ void __launch_bounds__(KMV_T, 2) k_kernel_tc(const long long* __restr
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const uint4 x = xrow[warp][q][lane];
+      if (q == 0) {
+        float n0, n1;
+        asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%8,%5,%8}, {%6,%7}, {%9,%9,%9,%9};"
+                     : "=f"(ce[0]), "=f"(ce[1]), "=f"(n0), "=f"(n1)
+                     : "r"(x.x & 0x7fff7fffu), "r"(x.y & 0x7fff7fffu), "r"(d0[0]), "r"(d1[0]), "r"(0u), "f"(0.f));
+      }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int j = 2 * q + u;
@@ -1020,6 +1037,7 @@ __global__ void __launch_bounds__(KMV_T, 2) k_kernel_tc(const long long* __restr
         unsigned long long* o = sums + ((int64_t)(s * 8 + 2 * t + c) * 8 + g) * 2;
         atomicAdd(o, (unsigned long long)h);
         atomicAdd(o + 1, (unsigned long long)l);
+        atomicAdd(est + (int64_t)(s * 8 + 2 * t + c) * 8 + g, __float2uint_rz(ce[c]) >> sh);
       }
     }
   }
@@ -1031,17 +1049,27 @@ __global__ void __launch_bounds__(KMV_T, 2) k_kernel_tc(const long long* __restr
     if (i < N && n < nr) {
       atomicAdd(sums + (i * 8 + n) * 2, (unsigned long long)acc.hi[c]);
       atomicAdd(sums + (i * 8 + n) * 2 + 1, (unsigned long long)acc.lo[c]);
+      const float v = tc_half(c >> 1 ? sb : sa, c & 1);  // infinite past 2^5 of 2^e
+      atomicAdd(est + i * 8 + n, __float2uint_rz(fminf(v, 65504.f) * 128.f) >> sh);
     }
   }
 }
+// results, and the blocks of 32 rows with one whose sum of |a x| is below 2^e / 2 (least: the estimate of that)
 __global__ void __launch_bounds__(256) k_kernel_join(const GridInfo* __restrict__ gi, int64_t N, int nr, double nugget,
-                                                     const unsigned long long* __restrict__ sums, const int* __restrict__ ef,
+                                                     const unsigned long long* __restrict__ sums,
+                                                     const unsigned* __restrict__ est, unsigned least,
+                                                     const int* __restrict__ ef, int* __restrict__ redo,
                                                      const double* __restrict__ X, int64_t ldx, double* __restrict__ Y, int64_t ldy) {
   const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
-  if (i >= N || !kmv_tc_ok(gi, ef)) return;
-  for (int n = 0; n < nr; ++n)
+  if (!kmv_tc_ok(gi, ef)) return;
+  bool low = false;
+  for (int n = 0; n < nr && i < N; ++n) {
+    low |= est[i * 8 + n] < least && ef[n] != KTC_NONE;
     Y[i + n * ldy] = tc_value((long long)sums[(i * 8 + n) * 2], (long long)sums[(i * 8 + n) * 2 + 1], kmv_exp(ef[n])) +
                      nugget * X[i + n * ldx];
+  }
+  const bool any = __any_sync(0xffffffffu, low);
+  if ((threadIdx.x & 31) == 0 && i < N) redo[i / 32] = any;
 }
 
 template <int D, int NR>
@@ -1050,8 +1078,9 @@ __global__ void __launch_bounds__(KMV_T) k_kernel_matvec(const double* __restric
                                                         const GridInfo* __restrict__ gi, int64_t N, uint64_t Cm, int ec,
                                                         double inv_ell, double nugget, int nr, int S,
                                                         const double* __restrict__ X, int64_t ldx,
-                                                        double* __restrict__ Y, int64_t ldy, const int* ef) {
-  if (ef && kmv_tc_ok(gi, ef)) return;  // done on the tensor cores
+                                                        double* __restrict__ Y, int64_t ldy, const int* ef,
+                                                        const int* redo) {
+  if (ef && kmv_tc_ok(gi, ef) && !redo[(int)blockIdx.x / S]) return;  // done on the tensor cores
   __shared__ uint64_t tab[64];
   __shared__ long long sp[KMV_W][32][D];  // grid points, or the bits of the coordinates
   __shared__ __align__(16) double sx[KMV_W][32][NR];
@@ -1139,7 +1168,7 @@ __global__ void __launch_bounds__(KMV_T) k_kernel_matvec(const double* __restric
 template <int D, int NR>
 static void kernel_matvec_launch(tlr_ctx* ctx, const double* pts, const long long* grid, const GridInfo* gi, int64_t N,
                                  uint64_t Cm, int ec, double ell, double nugget, int nr, const double* X, int64_t ldx,
-                                 double* Y, int64_t ldy, const int* ef) {
+                                 double* Y, int64_t ldy, const int* ef, const int* redo) {
   const int64_t rbs = (N + 31) / 32;
   // CTAs sharing 32 rows: about 32 per SM in all (a CTA's work is then small against the whole, so the
   // last wave is short), while each keeps a 32-column block for every warp
@@ -1157,25 +1186,25 @@ static void kernel_matvec_launch(tlr_ctx* ctx, const double* pts, const long lon
   cf.numAttrs = 1;
   TLR_SITE_PRE(ctx);
   TLR_CUDA(cudaLaunchKernelEx(&cf, k_kernel_matvec<D, NR>, pts, grid, gi, N, Cm, ec, 1.0 / ell, nugget, nr, S, X, ldx, Y,
-                              ldy, ef));
+                              ldy, ef, redo));
   TLR_LAUNCH_CHECK(ctx);
 }
 
 template <int D>
 static void kernel_matvec_d(tlr_ctx* ctx, const double* pts, const long long* grid, const GridInfo* gi, int64_t N,
                             uint64_t Cm, int ec, double ell, double nugget, int nr, const double* X, int64_t ldx,
-                            double* Y, int64_t ldy, const int* ef) {
-  if (nr == 1) kernel_matvec_launch<D, 1>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef);
-  else if (nr == 2) kernel_matvec_launch<D, 2>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef);
-  else if (nr <= 4) kernel_matvec_launch<D, 4>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef);
-  else kernel_matvec_launch<D, KMV_R>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef);
+                            double* Y, int64_t ldy, const int* ef, const int* redo) {
+  if (nr == 1) kernel_matvec_launch<D, 1>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef, redo);
+  else if (nr == 2) kernel_matvec_launch<D, 2>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef, redo);
+  else if (nr <= 4) kernel_matvec_launch<D, 4>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef, redo);
+  else kernel_matvec_launch<D, KMV_R>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, X, ldx, Y, ldy, ef, redo);
 }
 
 // Tensor cores from 3000 points on (DFMA / tensor cores, 4 columns, us: N = 2048, 3D 161 / 170; 4096, 2D 358 / 282;
 // 8192, 3D 1140 / 754; 32768, 3D 16277 / 10257; the same within 10 % for 1 and 8 columns); the totals of 2^20 points
 // stay below 2^63.
 size_t kernel_matvec_work(int64_t N) {
-  return N >= 3000 && N <= (1 << 20) ? (size_t)((N + 7) / 8 * 512 + N * 128 + 256) : 0;
+  return N >= 3000 && N <= (1 << 20) ? (size_t)((N + 7) / 8 * 512 + N * 160 + (N + 31) / 32 * 4 + 256) : 0;
 }
 
 void kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell, double nugget, int nrhs,
@@ -1194,12 +1223,14 @@ void kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell
     const int c0 = (int)((int64_t)nrhs * g / ng), nr = (int)((int64_t)nrhs * (g + 1) / ng) - c0;
     const double* Xg = X + c0 * ldx;
     double* Yg = Y + c0 * ldy;
-    int* ef = static_cast<int*>(work);
+    int *ef = static_cast<int*>(work), *redo = nullptr;
     if (work) {
       uint4* frag = reinterpret_cast<uint4*>(static_cast<char*>(work) + 256);
       unsigned long long* sums = reinterpret_cast<unsigned long long*>(frag + (N + 7) / 8 * 32);
       TLR_CUDA(cudaMemsetAsync(ef, 0x80, 32, ctx->stream));
-      TLR_CUDA(cudaMemsetAsync(sums, 0, (size_t)N * 128, ctx->stream));
+      unsigned* est = reinterpret_cast<unsigned*>(sums + N * 16);
+      redo = reinterpret_cast<int*>(est + N * 8);
+      TLR_CUDA(cudaMemsetAsync(sums, 0, (size_t)N * 160, ctx->stream));
       TLR_SITE_PRE(ctx);
       k_kernel_bound<<<dim3(std::min(cdiv(N, 1024), 128u), (unsigned)nr), 256, 0, ctx->stream>>>(N, Xg, ldx, ef);
       TLR_LAUNCH_CHECK(ctx);
@@ -1210,17 +1241,21 @@ void kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell
       const int64_t rbs = (N + 127) / 128;
       const int CH = (int)std::max<int64_t>(1, std::min<int64_t>(16, rbs * rbs / 2 / (8 * 152)));
       const int64_t na = rbs / CH, ctas = CH * na * (na + 1) / 2 + (rbs - na * CH) * (na + 1);
+      // the estimates in units of 2^(sh - 18): a step of 16 rows adds at most 2^22, N of them at most 2^(18 - sh) N < 2^32
+      int sh = 0;
+      while ((N << 18 >> sh) >= (1ll << 32)) ++sh;
       auto kern = d == 1 ? k_kernel_tc<1> : d == 2 ? k_kernel_tc<2> : k_kernel_tc<3>;
       TLR_SITE_PRE(ctx);
-      kern<<<(unsigned)ctas, KMV_T, 0, ctx->stream>>>(grid, gi, N, Ct, et, nr, CH, frag, ef, sums);
+      kern<<<(unsigned)ctas, KMV_T, 0, ctx->stream>>>(grid, gi, N, Ct, et, nr, CH, frag, ef, sums, est, sh);
       TLR_LAUNCH_CHECK(ctx);
       TLR_SITE_PRE(ctx);
-      k_kernel_join<<<cdiv(N, 256), 256, 0, ctx->stream>>>(gi, N, nr, nugget, sums, ef, Xg, ldx, Yg, ldy);
+      k_kernel_join<<<cdiv(N, 256), 256, 0, ctx->stream>>>(gi, N, nr, nugget, sums, est, 1u << (17 - sh), ef, redo, Xg, ldx, Yg,
+                                                             ldy);
       TLR_LAUNCH_CHECK(ctx);
     }
-    if (d == 1) kernel_matvec_d<1>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy, ef);
-    else if (d == 2) kernel_matvec_d<2>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy, ef);
-    else kernel_matvec_d<3>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy, ef);
+    if (d == 1) kernel_matvec_d<1>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy, ef, redo);
+    else if (d == 2) kernel_matvec_d<2>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy, ef, redo);
+    else kernel_matvec_d<3>(ctx, pts, grid, gi, N, Cm, ec, ell, nugget, nr, Xg, ldx, Yg, ldy, ef, redo);
   }
 }
 

@@ -33,6 +33,16 @@ __device__ __forceinline__ unsigned tc_fma2(unsigned a, unsigned b, unsigned c) 
   asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
   return r;
 }
+__device__ __forceinline__ unsigned tc_mul2(unsigned a, unsigned b) {
+  unsigned r;
+  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ float tc_half(unsigned a, int high) {
+  float r;
+  asm("cvt.f32.f16 %0, %1;" : "=f"(r) : "h"((unsigned short)(high ? a >> 16 : a)));
+  return r;
+}
 // the seven digit pairs of entries a, b with the signs of the high words sa, sb: FP16 (1024 + byte) s - (1024 + 128) s
 __device__ __forceinline__ void tc_pairs(uint2 a, uint2 b, unsigned sa, unsigned sb, unsigned (&d)[TC_P]) {
   const unsigned p0 = __byte_perm(a.x, b.x, 0x5140u), p1 = __byte_perm(a.x, b.x, 0x7362u), p2 = __byte_perm(a.y, b.y, 0x5140u);
