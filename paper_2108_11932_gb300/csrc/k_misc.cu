@@ -856,11 +856,10 @@ constexpr int KMV_W = 8, KMV_T = 32 * KMV_W, KMV_R = 8;
 // 3D, 4 columns 16.3 -> 10.3 ms (k_kernel_matvec alone; without the mirror images 15.8); error against extended
 // precision 0.1 to 0.8 of k_kernel_matvec's (1D to 3D, ell 0.02 to 3, right-hand sides over eight decades).
 //
-// Accuracy, row by row: an entry is off by up to 2^-58 and a right-hand side by 2^-58 of its column's bound 2^e, so a
-// result by up to N 2^-57 2^e whatever its own terms are, where FP64 has N 2^-53 sum_j |a_ij x_j|.  So the sums of
-// |a_ij x_j| are estimated on the way (one product more per step, of the leading digits' absolute values: nothing of a
-// number below 2^-10 of its bound, at most twice a larger one, four times the sum), and blocks of 32 rows with one
-// below 2^e / 2 are computed by k_kernel_matvec (a unit vector's far rows, values of very different sizes).
+// Accuracy, row by row: entries are off by up to 2^-58 and right-hand sides by 2^-58 of their column's bound 2^e,
+// whatever a row's own terms are.  So the sums of |a_ij x_j| are estimated on the way (one product more per step, of the
+// leading digits), and blocks of 32 rows with one below sqrt(N) / 64 2^e (tcdigits.cuh) are computed by k_kernel_matvec:
+// a unit vector's rows, values of very different sizes.
 constexpr int KTC_NONE = (int)0x80808080;  // exponent of a column without a nonzero entry, as memset leaves it
 __device__ __forceinline__ int kmv_exp(int e) { return e == KTC_NONE ? 1 : e; }
 // the grid resolves the points and the digits hold the right-hand sides; otherwise k_kernel_matvec does it all
@@ -949,7 +948,6 @@ __global__ void __launch_bounds__(KMV_T, 2) k_kernel_tc(const long long* __restr
     for (int k = 0; k < D; ++k) xr[r][k] = grid[min(r0 + g + 8 * r, N - 1) * D + k];
   TcAcc acc;
   tc_init(acc);
-  unsigned sa = 0, sb = 0;  // FP16 sums of |a x| 2^11 below 2^e: columns 2 t and 2 t + 1 of rows g and g + 8
   const int s1 = min(min((chunk + 1) * CH, I + 1) * 16, steps);
 #pragma unroll 1
   for (int s = chunk * CH * 16; s < s1; ++s) {
@@ -990,8 +988,8 @@ __global__ void __launch_bounds__(KMV_T, 2) k_kernel_tc(const long long* __restr
                        : "+f"(acc.f[i + j][0]), "+f"(acc.f[i + j][1]), "+f"(acc.f[i + j][2]), "+f"(acc.f[i + j][3])
                        : "r"(d0[i]), "r"(d1[i]), "r"(b[j]));
     asm volatile("mma.sync.aligned.m16n8k8.row.col.f16.f16.f16.f16 {%0,%1}, {%2,%3}, {%4}, {%0,%1};"
-                 : "+r"(sa), "+r"(sb)
-                 : "r"(d0[0]), "r"(d1[0]), "r"(tc_mul2(b[0] & 0x7fff7fffu, 0x20002000u)));  // 2^-7
+                 : "+r"(acc.est[0]), "+r"(acc.est[1])
+                 : "r"(d0[0]), "r"(d1[0]), "r"(tc_abs2s(b[0])));
     if (++acc.win == 2 * TC_WIN) tc_drain(acc);
     if (s >= I * 16) continue;  // the diagonal block has its mirror image itself
     float cf[8][2], ce[2];
@@ -1009,7 +1007,7 @@ __global__ void __launch_bounds__(KMV_T, 2) k_kernel_tc(const long long* __restr
         float n0, n1;
         asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%8,%5,%8}, {%6,%7}, {%9,%9,%9,%9};"
                      : "=f"(ce[0]), "=f"(ce[1]), "=f"(n0), "=f"(n1)
-                     : "r"(x.x & 0x7fff7fffu), "r"(x.y & 0x7fff7fffu), "r"(d0[0]), "r"(d1[0]), "r"(0u), "f"(0.f));
+                     : "r"(tc_abs2(x.x)), "r"(tc_abs2(x.y)), "r"(d0[0]), "r"(d1[0]), "r"(0u), "f"(0.f));
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
@@ -1049,12 +1047,11 @@ __global__ void __launch_bounds__(KMV_T, 2) k_kernel_tc(const long long* __restr
     if (i < N && n < nr) {
       atomicAdd(sums + (i * 8 + n) * 2, (unsigned long long)acc.hi[c]);
       atomicAdd(sums + (i * 8 + n) * 2 + 1, (unsigned long long)acc.lo[c]);
-      const float v = tc_half(c >> 1 ? sb : sa, c & 1);  // infinite past 2^5 of 2^e
-      atomicAdd(est + i * 8 + n, __float2uint_rz(fminf(v, 65504.f) * 128.f) >> sh);
+      atomicAdd(est + i * 8 + n, __float2uint_rz(fminf(tc_half(acc.est[c >> 1], c & 1), 65504.f) * 128.f) >> sh);
     }
   }
 }
-// results, and the blocks of 32 rows with one whose sum of |a x| is below 2^e / 2 (least: the estimate of that)
+// results, and the blocks of 32 rows with one whose estimate is below `least`
 __global__ void __launch_bounds__(256) k_kernel_join(const GridInfo* __restrict__ gi, int64_t N, int nr, double nugget,
                                                      const unsigned long long* __restrict__ sums,
                                                      const unsigned* __restrict__ est, unsigned least,
@@ -1244,12 +1241,13 @@ void kernel_matvec(tlr_ctx* ctx, const double* pts, int64_t N, int d, double ell
       // the estimates in units of 2^(sh - 18): a step of 16 rows adds at most 2^22, N of them at most 2^(18 - sh) N < 2^32
       int sh = 0;
       while ((N << 18 >> sh) >= (1ll << 32)) ++sh;
+      const unsigned least = (unsigned)(ldexp(tc_least((float)N), 18 - 11 - sh));
       auto kern = d == 1 ? k_kernel_tc<1> : d == 2 ? k_kernel_tc<2> : k_kernel_tc<3>;
       TLR_SITE_PRE(ctx);
       kern<<<(unsigned)ctas, KMV_T, 0, ctx->stream>>>(grid, gi, N, Ct, et, nr, CH, frag, ef, sums, est, sh);
       TLR_LAUNCH_CHECK(ctx);
       TLR_SITE_PRE(ctx);
-      k_kernel_join<<<cdiv(N, 256), 256, 0, ctx->stream>>>(gi, N, nr, nugget, sums, est, 1u << (17 - sh), ef, redo, Xg, ldx, Yg,
+      k_kernel_join<<<cdiv(N, 256), 256, 0, ctx->stream>>>(gi, N, nr, nugget, sums, est, least, ef, redo, Xg, ldx, Yg,
                                                              ldy);
       TLR_LAUNCH_CHECK(ctx);
     }

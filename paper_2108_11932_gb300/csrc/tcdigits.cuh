@@ -56,11 +56,25 @@ __device__ __forceinline__ void tc_pairs(uint2 a, uint2 b, unsigned sa, unsigned
   d[1] = tc_fma2(__byte_perm(p2, one, 0x4342u), s, bias);
   d[0] = tc_fma2(__byte_perm(a.y, b.y, 0x7632u), s, bias1);
 }
-struct TcAcc {  // group sums of a window; the totals: hi of the groups 0-3, lo of 4-7 (weights 256^-g)
+// Group sums of a window; the totals: hi of the groups 0-3, lo of 4-7 (weights 256^-g); est: estimates of the sums of
+// |x y|, FP16 in the layout of the products, 2^11 for the product of the two bounds (infinite past 2^5 of them).  The
+// estimate multiplies the leading digits: nothing of a number below 2^-10 of its bound, at most twice a larger one.
+//
+// What an estimate has to reach for a result to be as accurate as an FP64 sum: K terms x y in units of the two bounds are
+// off by the roundings of x and y, 2^-58 / sqrt(3) in the mean square each, so the result by
+// 2^-58.8 sqrt(sum x^2 + y^2), up to 2^-58.3 sqrt(K) and for entries spread over their range about 2^-60 sqrt(K); an FP64
+// sum by 2^-53 / sqrt(3) of its size s from its last rounding and about as much again from the others.  Hence
+// s >= sqrt(K) / 64 (tc_least; in the worst case, all roundings of one sign, K 2^-57 against FP64's K 2^-53 s).
+struct TcAcc {
   float f[8][4];
   long long hi[4], lo[4];
+  unsigned est[2];
   int win, bad;
 };
+__host__ __device__ __forceinline__ float tc_least(float K) { return 32.f * sqrtf(K); }  // in the estimates' units
+// |leading digits|, of the second factor times 2^-7
+__device__ __forceinline__ unsigned tc_abs2(unsigned d) { return d & 0x7fff7fffu; }
+__device__ __forceinline__ unsigned tc_abs2s(unsigned d) { return tc_mul2(d & 0x7fff7fffu, 0x20002000u); }
 __device__ __forceinline__ void tc_init(TcAcc& a) {
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
@@ -68,6 +82,7 @@ __device__ __forceinline__ void tc_init(TcAcc& a) {
 #pragma unroll
     for (int g = 0; g < 8; ++g) a.f[g][c] = 0.f;
   }
+  a.est[0] = a.est[1] = 0;
   a.win = a.bad = 0;
 }
 __device__ __forceinline__ void tc_drain(TcAcc& a) {
