@@ -21,7 +21,7 @@
 // Measured before -> now: A X, 2D, eps = 1e-6, N = 4096 (b = 256), 1 column 952 -> 60 us; N = 131072
 // (b = 1024), 8 columns 25.2 -> 9.15 ms (0.94 of the DFMA rate); L D L^T X, 3D N = 20011, b = 512,
 // eps = 1e-4, 1 column 6.50 -> 0.32 ms.  Several columns of a large matrix go to the tensor cores (below): the
-// 8 columns of N = 131072 9.15 -> 2.20 ms.
+// 8 columns of N = 131072 9.15 -> 2.26 ms.
 //
 // Sums run in a fixed order: results do not depend on timing.
 #include <cooperative_groups.h>
@@ -56,7 +56,10 @@ struct ApTab {
   const int* voff;  // [j (nb + 1) + i]: first column of tile i in V panel j
   const int* uoff;  // [i (nb + 1) + j]: first column of tile j in U panel i
   int npan, nb, b, unit;
-  const int* gate;  // if set: the kernel runs only if *gate is not zero
+  int64_t N;
+  // if set: the kernel (of FP64 products) runs only if *gate is not zero, and those CTAs (of k_apply_tn, row blocks of
+  // k_apply_nn) whose entry of redo is not
+  const int *gate, *redo;
 };
 
 // coefficient vectors are row-major with this many doubles per row (16-byte rows past one column)
@@ -90,8 +93,9 @@ __device__ __forceinline__ void ap_ld_a(const double* p, double (&a)[VEC]) {
 
 // X (original order) -> Xp (KD order, padded with zeros, row-major)
 __global__ void k_apply_gather(int64_t N, int64_t np, int nr, int ld, const int64_t* __restrict__ perm,
-                               const double* __restrict__ X, int64_t ldx, double* __restrict__ Xp, int* bad) {
-  if (bad && blockIdx.x == 0 && threadIdx.x == 0) *bad = 0;
+                               const double* __restrict__ X, int64_t ldx, double* __restrict__ Xp, int* flags,
+                               int64_t nflags) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nflags; e += (int64_t)gridDim.x * blockDim.x) flags[e] = 0;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < np * ld; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t p = e / ld;
     const int c = (int)(e % ld);
@@ -116,7 +120,7 @@ __global__ void __launch_bounds__(AP_T) k_apply_tn(ApTab T, const double* __rest
   constexpr int LD = ap_ld<NR>(), UN = NR <= 4 ? 2 : 1, STEP = 32 * VEC;
   constexpr int P = AP_CW * (NR == 3 ? 4 : NR == 6 ? 8 : NR), LANES = 32 / P;  // lanes that share a sum
   __shared__ int panel;
-  if (T.gate && *T.gate == 0) return;
+  if (T.gate && *T.gate == 0 && T.redo[blockIdx.x] == 0) return;
   if (threadIdx.x == 0) panel = ap_panel(T, (int)blockIdx.x);
   __syncthreads();
   const ApPanel pn = T.pan[panel];
@@ -228,9 +232,9 @@ __global__ void __launch_bounds__(AP_T) k_apply_nn(ApTab T, int dmode, int use_u
   constexpr int LD = ap_ld<NR>(), RB = 32 * VEC, UN = 4;
   __shared__ double red[AP_W * NR * RB];
   __shared__ double part[NR * RB];
-  if (T.gate && *T.gate == 0) return;
   const int b = T.b, rbs = (b + RB - 1) / RB;
   const int rank = (int)blockIdx.x % S, rb = (int)blockIdx.x / S;
+  if (T.gate && *T.gate == 0 && T.redo[rb] == 0) return;  // the whole cluster
   const int i = rb / rbs, r0 = (rb % rbs) * RB;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = r0 + lane * VEC;
   const ApRow row = T.row[i];
@@ -322,21 +326,29 @@ __global__ void __launch_bounds__(AP_T) k_apply_nn(ApTab T, int dmode, int use_u
 // are split in the registers that loaded them, so that the factor is read as it lies; tcgen05 wants its
 // operands in shared or tensor memory and 128 rows, which a panel of a few columns does not fill).  The
 // splitting is that of tcdigits.cuh, seven digits below a bound 2^e of the operand's column: a panel column's own
-// bound for the factor, the block's for each right-hand side.  Pairs with i + j <= 9 are kept (34 products a step; the dropped ones are 2^-66 of the
-// bounds); a group of equal i + j sums below 13 2^14 4 16 < 2^24 over four steps, exact in FP32, and moves to
-// 64-bit integers then; one rounding at the end.  Error: 2^-58 of the bounds per entry and factor, against FP64's
-// 2^-53 of the running sum per term: of A X, L X, L^T X and L (D) L^T X in 2D and 3D, eps 1e-8 to 1e-2, normal,
-// positive and right-hand sides over eight decades it is 0.2 to 0.8 of the DFMA kernels' (norm against extended
-// precision; truncating F, two instructions less, would make it up to twice theirs).
+// bound for the factor, the block's for each right-hand side.  Pairs with i + j <= 9 are kept (34 products a step;
+// the dropped ones are 2^-66 of the bounds); a group of equal i + j sums below 13 2^14 4 16 < 2^24 over four steps,
+// exact in FP32, and moves to 64-bit integers then; one rounding at the end.
 // Where the contraction index is the panel's column (Y_i += U_ij T_ij), the column's bound 2^e moves to the
 // coefficient: (A(m, k) 2^-e_k) (2^e_k T(k)).
+// Error: 2^-58 of the bounds per entry and factor, whatever the size of a result's own terms, where FP64 has 2^-53 of
+// the running sum per term.  So the sum of the terms' sizes is estimated too (one product more a step, of the leading
+// digits), and where it is small against the bounds (tcdigits.cuh; the first rows of a triangle, the far rows of a unit
+// vector's product, right-hand sides with small entries beside large ones) the FP64 kernel that follows each
+// contraction computes the 32 columns or 64 rows that the result is among, decided on the device.  Of A X, L X, L^T X
+// and L (D) L^T X in 2D and 3D, N = 6000 and 8192, normal, positive and smooth right-hand sides, unit vectors and values
+// over eight decades, against extended precision: in norm 0.2 to 1.0 of the DFMA kernels' error; row by row, over
+// u |A| |X|, the mean square at most theirs and the largest at most 1.15 of it.  (Truncating F instead of rounding, two
+// instructions less, would make it up to twice theirs.)
 // Bound: the integer instructions that split (about 18 per entry, at half rate; the ALU is busy 57 % of the
-// time, the tensor pipe 32 %, 16 warps per SM at 126 registers).  34 products of 16 x 8 x 16 per 256 entries.
+// time, the tensor pipe 32 %, 16 warps per SM at 128 registers).  35 products of 16 x 8 x 16 per 256 entries.
 // Latency: each lane copies its own fragments of the next steps into shared memory (cp.async, no barrier).
+// The estimates and what follows from them cost 3 % of A X (N = 131072, 8 columns 2.19 -> 2.26 ms).
 constexpr int TC_KS = 16;    // k per step
 constexpr int TC_STG = 3;    // steps in flight per warp
 constexpr int TC_SPC = 8;    // CTAs (a cluster) per block in k_apply_split
-constexpr int TC_FRAG = 64;  // uint4 per step of a split right-hand side: [2][lane], the words of tc_digits with the sign on top
+constexpr int TC_FRAG = 64;  // uint4 per step of a split right-hand side: [2][lane], tc_digits' words, the sign on top
+constexpr int TC_ZERO = -100000;  // exponent of a column of zeros
 constexpr int TC_W = 4, TC_T = 32 * TC_W;  // warps of k_apply_tn_tc and k_apply_nn_tc
 constexpr int TC_SMEM = TC_W * TC_STG * 32 * (64 + 32 + 16);
 
@@ -346,8 +358,9 @@ __device__ __forceinline__ void tc_mma(float (&c)[4], const unsigned (&a)[4], un
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// One step (CHECK: notes entries outside their bounds): the tile's fragments x[row half][k half][2] (rows g, g + 8; k 2t, 2t + 1, 2t + 8, 2t + 9 of the lane
-// g = lane / 4, t = lane % 4) with shifts e, times the split right-hand side's step (column g; the same k)
+// One step (CHECK: notes entries outside their bounds): the tile's fragments x[row half][k half][2] (rows g, g + 8;
+// k 2t, 2t + 1, 2t + 8, 2t + 9 of the lane g = lane / 4, t = lane % 4) with shifts e, times the split right-hand side's
+// step (column g; the same k)
 template <bool CHECK>
 __device__ __forceinline__ void tc_step(const double (&x)[2][2][2], const int (&e)[2][2][2], uint4 f0, uint4 f1, TcAcc& acc) {
   int bad = 0;
@@ -367,27 +380,37 @@ __device__ __forceinline__ void tc_step(const double (&x)[2][2][2], const int (&
     for (int j = 0; j < TC_P; ++j)
       if (i + j <= 7) tc_mma(acc.f[i + j], a, b0[j], b1[j]);
   }
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f16.f16.f16.f16 {%0,%1}, {%2,%3,%4,%5}, {%6,%7}, {%0,%1};"
+               : "+r"(acc.est[0]), "+r"(acc.est[1])
+               : "r"(tc_abs2(d[0][0][0])), "r"(tc_abs2(d[1][0][0])), "r"(tc_abs2(d[0][1][0])), "r"(tc_abs2(d[1][1][0])),
+                 "r"(tc_abs2s(b0[0])), "r"(tc_abs2s(b1[0])));
   if (CHECK) acc.bad |= bad;
   if (++acc.win == TC_WIN) tc_drain(acc);
 }
 // The warps' totals through shared memory: thread `threadIdx.x` < 128 gets entry (lane / 4 + 8 (c / 2), 2 (lane % 4) + c % 2)
 // of the fragment, lane = threadIdx.x / 4, c = threadIdx.x % 4
-__device__ __forceinline__ void tc_total(TcAcc& acc, long long* part, long long& h, long long& l) {
+// (est: the same of the estimates)
+__device__ __forceinline__ void tc_total(TcAcc& acc, long long* part, long long& h, long long& l, float& est) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* pest = reinterpret_cast<float*>(part + TC_W * 32 * 8);
+  static_assert(TC_W * 32 * (8 * sizeof(long long) + 4 * sizeof(float)) <= TC_SMEM, "the totals fit the buffers");
   tc_drain(acc);
   __syncthreads();  // the copies' buffers are free
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     part[(warp * 32 + lane) * 8 + c] = acc.hi[c];
     part[(warp * 32 + lane) * 8 + 4 + c] = acc.lo[c];
+    pest[(warp * 32 + lane) * 4 + c] = tc_half(acc.est[c >> 1], c & 1);
   }
   __syncthreads();
   h = l = 0;
+  est = 0.f;
   if (threadIdx.x >= TC_T) return;
 #pragma unroll
   for (int w = 0; w < TC_W; ++w) {
     h += part[(w * 32 + (threadIdx.x >> 2)) * 8 + (threadIdx.x & 3)];
     l += part[(w * 32 + (threadIdx.x >> 2)) * 8 + 4 + (threadIdx.x & 3)];
+    est += pest[(w * 32 + (threadIdx.x >> 2)) * 4 + (threadIdx.x & 3)];
   }
 }
 // copies of a lane's own bytes to shared memory, zeros if !ok (src must be readable memory all the same)
@@ -444,19 +467,24 @@ struct TcSeg {  // a split right-hand side: a block's rows in up to three segmen
 // Splits the right-hand sides of block blockIdx.x / TC_SPC: rows of X (SEG = 1: the block's b rows), or
 // [X_i; T_i; S_i] scaled by the panels' column bounds (SEG = 3; the bounds' shifts, by step, to ek).
 // Fragments to frag, the columns' exponents to ef.  A cluster per block finds the bounds together.
+// SEG = 3: a coefficient whose row is below 4^-d of the columns' bounds goes up by 2^d and its panel column down, so that
+// their roundings, 2^-58 of the bounds each, weigh the same in a product: a term's error falls with the root of its size
+// (T and S fall off by orders of magnitude).  least: what an estimate has to
+// reach (tcdigits.cuh), with the bounds themselves for the entries, 4 tc_least(sum 4^-d).
 template <int SEG>
 __global__ void __cluster_dims__(TC_SPC, 1, 1) __launch_bounds__(256)
     k_apply_split(const TcSeg* __restrict__ segs, const ApRow* __restrict__ rows, int b, const double* __restrict__ X,
                   const double* __restrict__ TR, const double* __restrict__ SC, const int* __restrict__ eD,
                   const int* __restrict__ eU, const int* __restrict__ eV, uint4* __restrict__ frag, int* __restrict__ ek_out,
-                  int* __restrict__ ef, int* bad_out) {
+                  int* __restrict__ ef, float* __restrict__ least, int* bad_out) {
   cg::cluster_group cl = cg::this_cluster();
   const int i = blockIdx.x / TC_SPC, rank = blockIdx.x % TC_SPC, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const TcSeg sg = segs[i];
   const int s0 = (sg.n0 + TC_KS - 1) / TC_KS, s1 = SEG > 1 ? (sg.n1 + TC_KS - 1) / TC_KS : 0,
             s2 = SEG > 1 ? (sg.n2 + TC_KS - 1) / TC_KS : 0, steps = s0 + s1 + s2;
   __shared__ int part[8], emax[8];
-  if (tid < 8) part[tid] = -100000;
+  __shared__ float wsum[SEG > 1 ? 8 : 1];
+  if (tid < 8) part[tid] = TC_ZERO;
   __syncthreads();
   // row k of step s: its coefficients and the exponent of its panel column
   auto entry = [&](int s, int k, int& ek) -> const double* {
@@ -478,34 +506,46 @@ __global__ void __cluster_dims__(TC_SPC, 1, 1) __launch_bounds__(256)
     ek = eV[rows[i].sc0 + k];
     return SC + (rows[i].sc0 + k) * 8;
   };
-  int m = -100000;  // of column tid % 8
+  int m = TC_ZERO;  // of column tid % 8
   for (int o = rank * 256 + tid; o < steps * 128; o += TC_SPC * 256) {
     int ek;
     const double* p = entry(o >> 7, (o >> 3) & 15, ek);
     const unsigned hw = p ? (unsigned)__double2hiint(p[o & 7]) & 0x7fffffffu : 0u;
     if (hw) m = max(m, tc_exp(hw) + ek);
-    if (SEG > 1 && (o & 7) == 0) ek_out[sg.ks0 * TC_KS + (o >> 3)] = tc_shift(ek);
   }
   atomicMax(&part[tid & 7], m);
   cl.sync();
   if (tid < 8) {
-    int v = -100000;
+    int v = TC_ZERO;
 #pragma unroll
     for (int q = 0; q < TC_SPC; ++q) v = max(v, cl.map_shared_rank(part, q)[tid]);
-    if (v == -100000) v = 1;
+    if (rank == 0) ef[i * 8 + tid] = v;  // TC_ZERO for a column of zeros
+    if (v == TC_ZERO) v = 1;
     else if (tc_odd(v)) *bad_out = 1;
     emax[tid] = v;
-    if (rank == 0) ef[i * 8 + tid] = v;
   }
   cl.sync();
   const int n = lane >> 2, t = lane & 3, en = emax[n];
+  float w = 0.f;
   for (int s = rank * 8 + warp; s < steps; s += TC_SPC * 8) {
     uint2 q[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       int ek;
-      const double* p = entry(s, 2 * t + (u & 1) + (u >> 1) * 8, ek);
+      const int k = 2 * t + (u & 1) + (u >> 1) * 8;
+      const double* p = entry(s, k, ek);
       const double x = p ? p[n] : 0.0;
+      if constexpr (SEG > 1) {
+        int g = x == 0.0 ? -48 : max(-48, tc_exp((unsigned)__double2hiint(x) & 0x7fffffffu) + ek - en);
+#pragma unroll
+        for (int o = 4; o < 32; o *= 2) g = max(g, __shfl_xor_sync(0xffffffffu, g, o));
+        const int d = max(0, -g / 2);
+        ek += d;
+        if (n == 0) {
+          ek_out[(sg.ks0 + s) * TC_KS + k] = tc_shift(ek);
+          if (p) w += exp2f(-2.f * (float)d);
+        }
+      }
       const int e = x == 0.0 ? 1 : en - ek;
       if (tc_odd(e)) *bad_out = 1;
       int bad = 0;  // |x| < 2^e by its making
@@ -515,6 +555,18 @@ __global__ void __cluster_dims__(TC_SPC, 1, 1) __launch_bounds__(256)
     uint4* out = frag + (sg.ks0 + s) * TC_FRAG + lane;
     out[0] = make_uint4(q[0].x, q[0].y, q[1].x, q[1].y);
     out[32] = make_uint4(q[2].x, q[2].y, q[3].x, q[3].y);
+  }
+  if constexpr (SEG > 1) {
+    for (int o = 16; o; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    if (lane == 0) wsum[warp] = w;
+    cl.sync();
+    if (rank == 0 && tid == 0) {
+      float v = 0.f;
+      for (int q = 0; q < TC_SPC; ++q)
+        for (int u = 0; u < 8; ++u) v += cl.map_shared_rank(wsum, q)[u];
+      least[i] = 4.f * tc_least(v);
+    }
+    cl.sync();  // no CTA leaves while its sums are still read
   }
 }
 
@@ -544,7 +596,7 @@ __global__ void __launch_bounds__(TC_T, 4) k_apply_tn_tc(ApTab T, const TcSeg* _
                                                          const int* __restrict__ ef, double* __restrict__ TR,
                                                          double* __restrict__ SC, double* __restrict__ YD,
                                                          int* __restrict__ eU, int* __restrict__ eV, int* __restrict__ eD,
-                                                         int* bad_out) {
+                                                         float least, int* bad_out, int* __restrict__ redo) {
   extern __shared__ __align__(16) char tc_smem[];
   __shared__ int64_t dst[16];  // row of a column's coefficients
   __shared__ unsigned cmax[TC_W][16];
@@ -649,10 +701,13 @@ __global__ void __launch_bounds__(TC_T, 4) k_apply_tn_tc(ApTab T, const TcSeg* _
         tc_step<false>(x, e, *ring.f(st, 0), *ring.f(st, 1), acc);
       });
   long long h, l;
-  tc_total(acc, reinterpret_cast<long long*>(tc_smem), h, l);
+  float est;
+  tc_total(acc, reinterpret_cast<long long*>(tc_smem), h, l, est);
   const int ol = threadIdx.x >> 2, oc = threadIdx.x & 3, or_ = (ol >> 2) + 8 * (oc >> 1), cc = c0 + or_, n = 2 * (ol & 3) + (oc & 1);
   if (cc >= pn.ncols) return;
-  const double y = tc_value(h, l, bound(or_) + ef[pn.blk * 8 + n]);
+  const int en = ef[pn.blk * 8 + n];
+  if (est < least && en != TC_ZERO && !(tri && (int64_t)pn.blk * b + cc >= T.N)) redo[blockIdx.x / 2] = 1;
+  const double y = tc_value(h, l, bound(or_) + en);
   (tri ? YD : pn.kind == 0 ? TR : SC)[dst[or_] * 8 + n] = y;
 }
 
@@ -660,7 +715,9 @@ __global__ void __launch_bounds__(TC_T, 4) k_apply_tn_tc(ApTab T, const TcSeg* _
 // [D_i | Urow_i | Vcol_i] [X_i; T_i; S_i].  Rows 2 g and 2 g + 1 are the fragment's rows g and g + 8 (16-byte loads).
 __global__ void __launch_bounds__(TC_T, 4) k_apply_nn_tc(ApTab T, int dmode, const TcSeg* __restrict__ segs,
                                                          const uint4* __restrict__ frag, const int* __restrict__ ek,
-                                                         const int* __restrict__ ef, ApOut out, int* bad_out) {
+                                                         const int* __restrict__ ef, const float* __restrict__ least,
+                                                         ApOut out, int* bad_out,
+                                                         int* __restrict__ redo) {
   extern __shared__ __align__(16) char tc_smem[];
   const int b = T.b, rbs = (b + 15) / 16, i = (int)blockIdx.x / rbs, r0 = ((int)blockIdx.x % rbs) * 16;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -719,12 +776,19 @@ __global__ void __launch_bounds__(TC_T, 4) k_apply_nn_tc(ApTab T, int dmode, con
       });
   if (acc.bad < 0) *bad_out = 1;
   long long h, l;
-  tc_total(acc, reinterpret_cast<long long*>(tc_smem), h, l);
+  float est;
+  tc_total(acc, reinterpret_cast<long long*>(tc_smem), h, l, est);
   const int ol = threadIdx.x >> 2, oc = threadIdx.x & 3, m = r0 + 2 * (ol >> 2) + (oc >> 1), n = 2 * (ol & 3) + (oc & 1);
   if (m >= b || (!out.Z && n >= out.nr)) return;
-  double v = tc_value(h, l, ef[i * 8 + n]);
+  const int en = ef[i * 8 + n];
+  double v = tc_value(h, l, en);
   const int64_t gr = (int64_t)i * b + m;
-  if (out.add) v += out.add[gr * 8 + n];
+  if (out.add) {
+    const double a = out.add[gr * 8 + n];
+    if (en != TC_ZERO) est += (float)fmin(ldexp(fabs(a), 11 - en), 65504.0);  // a term like the others
+    v += a;
+  }
+  if (est < least[i] && en != TC_ZERO && gr < T.N) redo[i * ((b + 63) / 64) + m / 64] = 1;
   if (out.scale) v *= out.scale[gr];
   if (out.Z) out.Z[gr * 8 + n] = v;
   else if (gr < out.N) out.Y[out.perm[gr] + n * out.ldy] = v;
@@ -803,17 +867,25 @@ struct ApPlan {  // host side of one matrix's tables
   int64_t steps[3];
 };
 
-// The product from the gathered right-hand sides Xp
 template <int NR, int VEC>
-void apply_run(tlr_ctx* ctx, const tlr_mat* M, int op, const ApPlan& pl, ApTab T, int nr, const double* Xp, double* YD,
-               double* Z, double* TR, double* SC, double* Y, int64_t ldy) {
+void apply_group(tlr_ctx* ctx, const tlr_mat* M, int op, const ApPlan& pl, int nr, const double* X, int64_t ldx, double* Y,
+                 int64_t ldy, Buf& work) {
+  constexpr int LD = ap_ld<NR>();
+  const int64_t np = pl.np, R = std::max<int64_t>(pl.R, 1);
+  double* Xp = work.need<double>((size_t)(3 * np + 2 * R) * LD);
+  double *YD = Xp + np * LD, *Z = YD + np * LD, *TR = Z + np * LD, *SC = TR + R * LD;
+  TLR_SITE_PRE(ctx);
+  k_apply_gather<<<blocks(np * LD, 256), 256, 0, ctx->stream>>>(M->N, np, nr, LD, M->dperm, X, ldx, Xp, nullptr, 0);
+  TLR_LAUNCH_CHECK(ctx);
+  const int64_t kd = (int64_t)M->nb * M->b;
+  const ApTab& T = pl.T;
   auto tn = [&](int l, const double* x) {
-    T.pan = pl.lists[l];
-    T.npan = pl.npan[l];
-    run_tn<NR, VEC>(ctx, T, pl.ctas[l], x, TR, SC, YD);
+    ApTab Tl = T;
+    Tl.pan = pl.lists[l];
+    Tl.npan = pl.npan[l];
+    run_tn<NR, VEC>(ctx, Tl, pl.ctas[l], x, TR, SC, YD);
   };
   ApOut fin{nullptr, nullptr, nullptr, Y, M->dperm, ldy, M->N, nr};
-  const int64_t kd = (int64_t)M->nb * M->b;
   tn(0, Xp);
   if (op == TLR_OP_A) {
     run_nn<NR, VEC>(ctx, T, 1, 1, 1, kd + 2 * pl.R, Xp, TR, SC, fin);
@@ -830,62 +902,61 @@ void apply_run(tlr_ctx* ctx, const tlr_mat* M, int op, const ApPlan& pl, ApTab T
   }
 }
 
-template <int NR, int VEC>
-void apply_group(tlr_ctx* ctx, const tlr_mat* M, int op, const ApPlan& pl, int nr, const double* X, int64_t ldx, double* Y,
-                 int64_t ldy, Buf& work) {
-  constexpr int LD = ap_ld<NR>();
-  const int64_t np = pl.np, R = std::max<int64_t>(pl.R, 1);
-  double* Xp = work.need<double>((size_t)(3 * np + 2 * R) * LD);
-  double *YD = Xp + np * LD, *Z = YD + np * LD, *TR = Z + np * LD, *SC = TR + R * LD;
-  TLR_SITE_PRE(ctx);
-  k_apply_gather<<<blocks(np * LD, 256), 256, 0, ctx->stream>>>(M->N, np, nr, LD, M->dperm, X, ldx, Xp, nullptr);
-  TLR_LAUNCH_CHECK(ctx);
-  apply_run<NR, VEC>(ctx, M, op, pl, pl.T, nr, Xp, YD, Z, TR, SC, Y, ldy);
-}
-
-// The same on the tensor cores (8 columns, zero past nr).  Numbers outside what the digits hold (not finite, or a
-// column's largest below 2^-900 or above 2^900) set a flag, and then the FP64 kernels that follow run too.
+// The same on the tensor cores (8 columns, zero past nr).  After each contraction the FP64 kernel computes what would have
+// fewer digits (redo), or all of it if numbers are outside what the digits hold (bad: not finite, or a column's largest
+// below 2^-900 or above 2^900).
 void apply_group_tc(tlr_ctx* ctx, const tlr_mat* M, int op, const ApPlan& pl, int nr, const double* X, int64_t ldx, double* Y,
                     int64_t ldy, Buf& work) {
-  const int64_t np = pl.np, R = std::max<int64_t>(pl.R, 1);
+  const int64_t np = pl.np, R = std::max<int64_t>(pl.R, 1), kd = np;
   const int64_t steps = std::max({pl.steps[0], pl.steps[1], pl.steps[2]});
   const int nb = M->nb, b = M->b;
+  // flags: bad, then redo of the contractions of list 0 and 1 (k_apply_tn's CTAs) and of the middle and the final rows
+  const int64_t rbs = (int64_t)nb * ((b + 63) / 64), nflags = 1 + pl.ctas[0] + pl.ctas[1] + 2 * rbs;
   // doubles: Xp, YD, Z (np x 8), T, S (R x 8); fragments (16 bytes); ints: exponents by step, of U, V
-  // and tile columns, of the blocks' right-hand sides, the flag
+  // and tile columns, of the blocks' right-hand sides, the least estimates, the flags
   const size_t nd = (size_t)(3 * np + 2 * R) * 8, nf = 2 * (size_t)steps * TC_FRAG,
-               ni = (size_t)(steps * TC_KS + 2 * R + np + 8 * (int64_t)nb + 1);
+               ni = (size_t)(steps * TC_KS + 2 * R + np + 9 * (int64_t)nb + nflags);
   double* Xp = work.need<double>(nd + nf + (ni + 1) / 2);
   double *YD = Xp + np * 8, *Z = YD + np * 8, *TR = Z + np * 8, *SC = TR + R * 8;
   uint4* frag = reinterpret_cast<uint4*>(Xp + nd);
   int* ek = reinterpret_cast<int*>(Xp + nd + nf);
-  int *eU = ek + steps * TC_KS, *eV = eU + R, *eD = eV + R, *ef = eD + np, *bad = ef + 8 * (int64_t)nb;
+  int *eU = ek + steps * TC_KS, *eV = eU + R, *eD = eV + R, *ef = eD + np, *bad = ef + 9 * (int64_t)nb;
+  float* least = reinterpret_cast<float*>(ef + 8 * (int64_t)nb);
+  int *redo_tn[2] = {bad + 1, bad + 1 + pl.ctas[0]}, *redo_nn[2] = {redo_tn[1] + pl.ctas[1], redo_tn[1] + pl.ctas[1] + rbs};
   TLR_SITE_PRE(ctx);
-  k_apply_gather<<<blocks(np * 8, 256), 256, 0, ctx->stream>>>(M->N, np, nr, 8, M->dperm, X, ldx, Xp, bad);
+  k_apply_gather<<<blocks(np * 8, 256), 256, 0, ctx->stream>>>(M->N, np, nr, 8, M->dperm, X, ldx, Xp, bad, nflags);
   TLR_LAUNCH_CHECK(ctx);
   for (const void* f : {(const void*)k_apply_tn_tc, (const void*)k_apply_nn_tc})
     TLR_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM));
   ApTab T = pl.T;
+  T.gate = bad;
   auto tn = [&](int l, const double* x) {
     TLR_SITE_PRE(ctx);
     k_apply_split<1><<<(unsigned)nb * TC_SPC, 256, 0, ctx->stream>>>(pl.segs[0], T.row, b, x, TR, SC, eD, eU, eV, frag, ek, ef,
-                                                                             bad);
+                                                                     least, bad);
     TLR_LAUNCH_CHECK(ctx);
     if (pl.ctas[l] <= 0) return;
     T.pan = pl.lists[l];
     T.npan = pl.npan[l];
+    T.redo = redo_tn[l];
     TLR_SITE_PRE(ctx);
-    k_apply_tn_tc<<<2 * (unsigned)pl.ctas[l], TC_T, TC_SMEM, ctx->stream>>>(T, pl.segs[0], frag, ef, TR, SC, YD, eU, eV, eD, bad);
+    k_apply_tn_tc<<<2 * (unsigned)pl.ctas[l], TC_T, TC_SMEM, ctx->stream>>>(T, pl.segs[0], frag, ef, TR, SC, YD, eU, eV, eD,
+                                                                            tc_least((float)b), bad, redo_tn[l]);
     TLR_LAUNCH_CHECK(ctx);
+    run_tn<8, 2>(ctx, T, pl.ctas[l], x, TR, SC, YD);
   };
-  auto nn = [&](int q, int dmode, const double* x, const ApOut& o) {
+  // rows [D | U | V] (dmode, use_u, use_v) of the q-th segment list; f: the final rows
+  auto nn = [&](int q, int dmode, int use_u, int use_v, int64_t ktot, const double* x, const ApOut& o, int f) {
     TLR_SITE_PRE(ctx);
     k_apply_split<3><<<(unsigned)nb * TC_SPC, 256, 0, ctx->stream>>>(pl.segs[q], T.row, b, x, TR, SC, eD, eU, eV, frag, ek, ef,
-                                                                             bad);
+                                                                     least, bad);
     TLR_LAUNCH_CHECK(ctx);
+    T.redo = redo_nn[f];
     TLR_SITE_PRE(ctx);
     k_apply_nn_tc<<<(unsigned)((int64_t)nb * ((b + 15) / 16)), TC_T, TC_SMEM, ctx->stream>>>(T, dmode, pl.segs[q], frag, ek,
-                                                                                          ef, o, bad);
+                                                                                          ef, least, o, bad, redo_nn[f]);
     TLR_LAUNCH_CHECK(ctx);
+    run_nn<8, 2>(ctx, T, dmode, use_u, use_v, ktot, x, TR, SC, o);
   };
   if (op == TLR_OP_A) {  // kernel entries are at most 1, the diagonal's 1 + nugget
     TLR_SITE_PRE(ctx);
@@ -901,20 +972,18 @@ void apply_group_tc(tlr_ctx* ctx, const tlr_mat* M, int op, const ApPlan& pl, in
   ApOut fin{nullptr, nullptr, nullptr, Y, M->dperm, ldy, M->N, nr};
   tn(0, Xp);
   if (op == TLR_OP_A) {
-    nn(2, 1, Xp, fin);
+    nn(2, 1, 1, 1, kd + 2 * pl.R, Xp, fin, 1);
   } else if (op == TLR_OP_L) {
-    nn(2, 2, Xp, fin);
+    nn(2, 2, 1, 0, kd / 2 + pl.R, Xp, fin, 1);
   } else if (op == TLR_OP_LT) {
     fin.add = YD;
-    nn(1, 0, Xp, fin);
+    nn(1, 0, 0, 1, pl.R, Xp, fin, 1);
   } else {  // L (D) (L^T X); the first contraction has left the exponents of U's and the tiles' columns
     ApOut mid{YD, M->state == 2 ? M->dvec : nullptr, Z, nullptr, nullptr, 0, 0, nr};
-    nn(1, 0, Xp, mid);
+    nn(1, 0, 0, 1, pl.R, Xp, mid, 0);
     tn(1, Z);
-    nn(2, 2, Z, fin);
+    nn(2, 2, 1, 0, kd / 2 + pl.R, Z, fin, 1);
   }
-  T.gate = bad;
-  apply_run<8, 2>(ctx, M, op, pl, T, nr, Xp, YD, Z, TR, SC, Y, ldy);
 }
 
 template <int VEC>
@@ -958,13 +1027,21 @@ void tlr_apply(tlr_ctx* ctx, const tlr_mat* M, int op, int nrhs, const double* X
     al(M->Urow[i]);
     al(M->Vcol[i]);
   }
-  // Tensor cores where the DFMAs (1.67 ps per entry and column) take longer than the tensor cores' passes (3.2 ps
-  // per entry for up to eight columns) and their five further launches (45 us): measured, DFMA / tensor cores, us:
-  // 6.7e8 entries 2412 / 2200 (2 columns), 9134 / 2202 (8); 3.6e7 213 / 241 (2), 284 / 241 (3), 608 / 240 (8);
-  // 4.8e6 108 / 121 (4), 132 / 123 (6), 155 / 124 (8); 1.4e6 101 / 106 (8).
+  // Tensor cores where the DFMAs (1.67 ps per entry and accumulator column) take longer than the tensor cores' passes
+  // (3.2 ps per entry for up to eight columns), the DFMAs of eight columns for the share of the entries whose results
+  // are computed again, and their further launches.  That share is none for A and, for the factors' triangles of the
+  // covariance problems (normal right-hand sides), about 0.6 of L, 0.55 of L^T, 0.5 of both.  Measured, DFMA / tensor
+  // cores, us: A, 6.7e8 entries 2412 / 2260 (2 columns), 9103 / 2266 (8); 3.6e7 213 / 241 (2), 284 / 241 (3), 608 / 240
+  // (8); 4.8e6 108 / 121 (4), 155 / 124 (8).  8 columns, L, 3.7e8 entries 4548 / 3973; 5.4e7 932 / 907; 1.3e7 287 / 319;
+  // L^T 4439 / 3486, 880 / 840, 280 / 300; L (D) L^T, 7.3e8 entries 8899 / 5587; 1.1e8 1753 / 1693; 2.5e7 517 / 507;
+  // 4 columns 4570 / 5328, 949 / 1572, 312 / 495.
   const int ng = (nrhs + 7) / 8;  // right-hand sides in equal groups of at most eight
-  const double entries = 4.0 * b * (double)tr + (double)nb * b * b;
-  pl.tc = aligned && entries * (1.67 * ((nrhs + ng - 1) / ng) - 3.2) > 45e6;
+  const int nr = (nrhs + ng - 1) / ng, cols = nr <= 4 ? nr : nr <= 6 ? 6 : 8;
+  const double lower = 2.0 * b * (double)tr + 0.5 * nb * b * b;
+  const double entries = op == TLR_OP_L || op == TLR_OP_LT ? lower : 2.0 * lower;
+  const double again = op == TLR_OP_A ? 0.0 : op == TLR_OP_L ? 0.6 : op == TLR_OP_LT ? 0.55 : 0.5;
+  const double launches = op == TLR_OP_A ? 45e6 : op == TLR_OP_LLT ? 100e6 : 60e6;
+  pl.tc = aligned && entries * (1.67 * cols - 3.2 - 1.67 * 8 * again) > launches;
   std::vector<ApPanel> pans;
   int n0[4] = {0, 0, 0, 0};
   auto list = [&](int l, bool v, bool u, bool dg) {
@@ -1036,6 +1113,7 @@ void tlr_apply(tlr_ctx* ctx, const tlr_mat* M, int op, int nrhs, const double* X
   pl.T.nb = nb;
   pl.T.b = b;
   pl.T.unit = M->state == 2;
+  pl.T.N = M->N;
   pl.R = tr;
   pl.np = (int64_t)nb * b;
   for (int g = 0; g < ng; ++g) {
