@@ -529,11 +529,17 @@ static SolvePlan* plan_build(tlr_ctx* ctx, const tlr_mat* F) {
 }
 
 template <int NR>
+static constexpr size_t solve_smem(int xs) {
+  return sizeof(double) * ((size_t)SV_RLD * NR * SV_RB + SV_NC * SV_C * SV_T + (size_t)NR * xs);
+}
+
+template <int NR>
 static void solve_launch(tlr_ctx* ctx, const SolvePlan* P, SvVec v) {
   const int b = P->T.b;
   // whole chunks of a rows step, or all of the vector with zeros to a multiple of 64
-  v.xs = (int)std::min<int64_t>(SV_XS / NR / 1024 * 1024, (std::max<int64_t>(b, P->len) + 63) / 64 * 64);
-  const size_t smem = sizeof(double) * ((size_t)SV_RLD * NR * SV_RB + SV_NC * SV_C * SV_T + (size_t)NR * v.xs);
+  constexpr int most = SV_XS / NR / 1024 * 1024;
+  v.xs = (int)std::min<int64_t>(most, (std::max<int64_t>(b, P->len) + 63) / 64 * 64);
+  const size_t smem = solve_smem<NR>(v.xs);
   cudaLaunchConfig_t cf{};
   cudaLaunchAttribute at{};
   cf.blockDim = dim3(SV_T);
@@ -542,7 +548,8 @@ static void solve_launch(tlr_ctx* ctx, const SolvePlan* P, SvVec v) {
   cf.attrs = &at;
   cf.numAttrs = 1;
   auto kern = k_solve<NR>;
-  TLR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // the limit is the kernel's, for all contexts and threads: always the largest launch's, never this one's
+  TLR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)solve_smem<NR>(most)));
   at.id = cudaLaunchAttributeCooperative;  // the CTAs wait for one another: all resident, or none
   at.val.cooperative = 1;
   cf.gridDim = dim3((unsigned)ctx->sm_count);

@@ -327,7 +327,8 @@ constexpr size_t TRIM_SMEM_MAX = 220 * 1024;
 template <int CS, bool SM>
 void trim_launch(tlr_ctx* ctx, const TrimDev* dj, int cnt, size_t smem, int b, double eps) {
   auto kern = k_trim<CS, SM>;
-  TLR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // the limit is the kernel's, for all contexts and threads: always the largest launch's, never this one's
+  TLR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TRIM_SMEM_MAX));
   cudaLaunchConfig_t cf{};
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
