@@ -21,8 +21,8 @@
 //     matrix's trimming waits for;
 //   * the tiles of low rank run beside them on the side stream.
 // Measured, one thread per pair and rank classes one after another -> now: trimming a matrix of N = 16384, b = 512
-// (ranks up to 142, mean 27) 109 -> 12.4 ms; 12 tiles of rank 140 61 -> 9.8 ms; 57 of rank 64 12.9 -> 3.9; 400 of
-// rank 16 1.36 -> 1.04; 4 of rank 300 (b = 1024) 723 -> 61.
+// (ranks up to 142, mean 27) 109 -> 12.9 ms; 12 tiles of rank 140 61 -> 9.5 ms; 57 of rank 64 12.9 -> 3.7; 400 of
+// rank 16 1.36 -> 1.01; 4 of rank 300 (b = 1024) 723 -> 60.
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -128,9 +128,11 @@ __device__ __forceinline__ double pair_dot(const double* x, const double* y, int
 }
 
 // CS: CTAs of the tile's cluster.  SM: X and the norms live in shared memory, column c in CTA c % CS at place
-// c / CS; otherwise in global memory.
+// c / CS; otherwise in global memory.  Registers for the CTAs that share an SM: five single ones when ranks are low (2000
+// tiles of rank 16, b = 1024: 5.2 ms; 6.0 with three), two of clusters of four (57 tiles of rank 80: 6.5 ms; 9.8 with one,
+// 6.6 with four), one of clusters of eight, which are few.
 template <int CS, bool SM>
-__global__ void __launch_bounds__(TR_T) k_trim(const TrimDev* __restrict__ jobs, int b, double eps) {
+__global__ void __launch_bounds__(TR_T, CS == 1 ? 5 : CS == 4 ? 2 : 1) k_trim(const TrimDev* __restrict__ jobs, int b, double eps) {
   const TrimDev J = jobs[blockIdx.x / CS];
   const int rank = (int)(blockIdx.x % CS);
   const int r = J.r, tid = threadIdx.x, w = tid >> 5, l = tid & 31;
